@@ -38,6 +38,7 @@
 
 #include <cuda_bf16.h>
 
+#include "spg_ff.cuh"
 #include "spg_internal.h"
 
 namespace spg {
@@ -133,7 +134,7 @@ struct KSum {
         c = (t - s) - y;
         s = t;
     }
-    __device__ __forceinline__ double value() const { return (double)s - (double)c; }
+    __device__ __forceinline__ ff::FF value() const { return {s, -c}; }
 };
 
 // Packed float32 pairs (sm_100 and later issue one instruction for two
@@ -157,8 +158,8 @@ struct KSum2 {
         c = sub2(sub2(t, s), y);
         s = t;
     }
-    __device__ __forceinline__ double value_x() const { return (double)s.x - (double)c.x; }
-    __device__ __forceinline__ double value_y() const { return (double)s.y - (double)c.y; }
+    __device__ __forceinline__ ff::FF value_x() const { return {s.x, -c.x}; }
+    __device__ __forceinline__ ff::FF value_y() const { return {s.y, -c.y}; }
 };
 
 // Phase A of one z-step at a thread's VX voxels of plane z: the weighted
@@ -640,21 +641,30 @@ __device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pi
     }
 
     if (!aborted && (REC || DOT)) {
-        // block reduction of the item's sums, fixed order
-        double v[4] = {0.5 * kdl.value_x(), kdl.value_y(), kt.value(), kr.value()};
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int q = 0; q < 4; q++) v[q] += __shfl_down_sync(FULL, v[q], o);
-        if (lane == 0)
-#pragma unroll
-            for (int q = 0; q < 4; q++) sh.red[warp * 4 + q] = v[q];
-        __syncthreads();
-        if (tid == 0) {
-            double a[4] = {0, 0, 0, 0};
-            for (int w = 0; w < TY + 1; w++)
-                for (int q = 0; q < 4; q++) a[q] += sh.red[w * 4 + q];
-            for (int q = 0; q < 4; q++) P.partials[(long long)it * 4 + q] = a[q];
+        // block reduction of the item's sums, fixed order (float-float, or
+        // double where a float-float could overflow: spg_ff.cuh)
+        const ff::FF d = kdl.value_x();
+        const ff::FF v[4] = {{0.5f * d.hi, 0.5f * d.lo}, kdl.value_y(), kt.value(), kr.value()};
+        const bool big = ff::too_big(v[0]) || ff::too_big(v[1]) || ff::too_big(v[2]) || ff::too_big(v[3]);
+        double *const out = P.partials + (long long)it * 4;
+        if (!__syncthreads_or(big ? 1 : 0)) {
+            ff::FF *const red = reinterpret_cast<ff::FF *>(sh.red);
+            const ff::FF s = ff::warp_sum4(v, lane);
+            if ((lane & 7) == 0) red[warp * 4 + (lane >> 3)] = s;
+            __syncthreads();
+            if (warp == 0) {
+                const ff::FF t = ff::cross_warp_sum4(red, TY + 1, lane, ff::FF{0.f, 0.f});
+                if (lane < 4) out[lane] = ff::to_double(t);
+            }
+        } else {
+            const double w[4] = {ff::to_double(v[0]), ff::to_double(v[1]), ff::to_double(v[2]), ff::to_double(v[3])};
+            const double s = ff::warp_sum4(w, lane);
+            if ((lane & 7) == 0) sh.red[warp * 4 + (lane >> 3)] = s;
+            __syncthreads();
+            if (warp == 0) {
+                const double t = ff::cross_warp_sum4(sh.red, TY + 1, lane, 0.0);
+                if (lane < 4) out[lane] = t;
+            }
         }
     }
     __syncthreads();  // every stage consumed before the next item's prologue
@@ -775,10 +785,9 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
             if (sums) {
                 for (int q = V.item_begin + lane; q < V.item_end; q += 32)
                     for (int c = 0; c < 4; c++) a[c] += __ldcg(P.partials + (long long)q * 4 + c);
+                const double s = ff::warp_sum4(a, lane);
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                    for (int c = 0; c < 4; c++) a[c] += __shfl_down_sync(FULL, a[c], o);
+                for (int c = 0; c < 4; c++) a[c] = __shfl_sync(FULL, s, 8 * c);
             }
             if (lane == 0) {
                 if (rec) {
