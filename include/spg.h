@@ -152,8 +152,8 @@ enum { SPG_TILE_AUTO = 0, SPG_TILE_128x8 = 1, SPG_TILE_128x4 = 2, SPG_TILE_64x8 
        SPG_TILE_128x7_S4 = 9 };
 
 /* Create a solver for one volume (spg_create) or for nvol independent
- * volumes of possibly different sizes advanced together, one fused launch per
- * iteration for all of them (spg_create_batch; the paper refines classes and
+ * volumes of possibly different sizes advanced together, each iteration one
+ * fused pass over all of them (spg_create_batch; the paper refines classes and
  * the two gold-standard half-maps independently, Sec. 2 and Sec. 2.3).
  * params: one (or nvol) descriptions, copied. opt: NULL for defaults.
  * stream: a cudaStream_t or NULL. On success *out owns all device memory it
@@ -288,8 +288,11 @@ spg_status spg_get_x(spg_ctx *ctx, int vol, float *x);
  * Asynchronous; per-volume statistics are read with spg_round_stats. */
 spg_status spg_reweight(spg_ctx *ctx);
 
-/* Run k iterations (one fused launch each, replayed from a captured CUDA
- * graph when k is large). Asynchronous. Errors: SPG_ENOTREADY before the
+/* Run k iterations. The fused step runs many of them per launch (a cooperative
+ * launch with a barrier over the grid between iterations; up to about 10 ms
+ * of work each); the Fourier-domain data term and the plain kernel of the
+ * alternative readings launch per iteration, replayed from a captured CUDA
+ * graph when k is large. Asynchronous. Errors: SPG_ENOTREADY before the
  * first spg_reweight, SPG_EINVAL if the round would exceed
  * max_iters_per_round. */
 spg_status spg_iterate(spg_ctx *ctx, int k);

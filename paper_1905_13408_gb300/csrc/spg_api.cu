@@ -28,7 +28,13 @@ namespace {
 thread_local std::string g_last_error = "no error";
 
 constexpr long long kTimeoutNs = 2000000000LL;  // 2 s bound on any device-side wait
-constexpr int kGraphLen = 10;                   // iterations per captured graph
+constexpr int kGraphLen = 10;                   // iterations per captured graph (Fourier-domain term, plain steps)
+// Bounds on the iterations of one fused launch: the partial sums it keeps
+// (32 bytes per work item and iteration) and roughly how long it may hold the
+// GPU (work queued on other streams starts between launches). At 10 ms the
+// launch boundary, about 5 us, no longer shows.
+constexpr size_t kPartialBytes = 8u << 20;
+constexpr double kLaunchSeconds = 10e-3;
 constexpr uint64_t kStateMagic = 0x5350475354415445ull;  // "SPGSTATE"
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
@@ -90,6 +96,7 @@ struct spg_ctx {
 
     StepVariant var{4, 8, 3, false, true};
     int zchunk = 0, grid = 0, ctas_per_sm = 0, nitems = 0;
+    int iters_per_launch = 1;  // most iterations one launch of the plan runs
     std::vector<WorkItem> items_h;
 
     long long k_total = 0;  // host mirror of the device counters
@@ -449,7 +456,15 @@ spg_status build_plan(spg_ctx *ctx, const StepVariant &v, int zchunk_opt)
     CK(cudaMemcpyAsync(ctx->sched_d, sched.data(), sched.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream),
        "upload schedule");
     CK(dalloc(&ctx->items_d, items.size() * sizeof(WorkItem)), "alloc items");
-    CK(dalloc(&ctx->partials_d, items.size() * 4 * sizeof(double)), "alloc partials");
+    // iterations per launch: room for their partial sums, the time bound (from
+    // the bytes of an iteration), and with restart the items a CTA can track
+    int max_cta_items = 0;
+    for (int g = 0; g < G; g++) max_cta_items = std::max(max_cta_items, first[g + 1] - first[g]);
+    const double iter_s = 4e-6 + (double)ctx->total * 32.0 / 6.5e12;
+    const double fit = std::min((double)kPartialBytes / (items.size() * 4 * sizeof(double)), kLaunchSeconds / iter_s);
+    int per_launch = (int)std::max(1.0, std::min(fit, 1024.0));
+    if (ctx->opt.restart && max_cta_items > kMaxCtaItems) per_launch = 1;
+    CK(dalloc(&ctx->partials_d, (size_t)per_launch * items.size() * 4 * sizeof(double)), "alloc partials");
     CK(cudaMemcpyAsync(ctx->items_d, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice,
                        ctx->stream),
        "upload items");
@@ -476,6 +491,7 @@ spg_status build_plan(spg_ctx *ctx, const StepVariant &v, int zchunk_opt)
     ctx->nitems = (int)items.size();
     ctx->ctas_per_sm = occ;
     ctx->grid = G;
+    ctx->iters_per_launch = per_launch;
     if (ctx->gexec) {
         cudaGraphExecDestroy(ctx->gexec);
         ctx->gexec = nullptr;
@@ -506,6 +522,9 @@ StepParams step_params(const spg_ctx *c)
     // own row pass forms it from x_{k+1} and d_{k+1} as it reads them
     p.ybuf = (c->fourier && !c->xown) ? c->Ybuf : nullptr;
     p.timeout_ns = kTimeoutNs;
+    p.niter = 1;
+    p.tm_step = 0;
+    p.xouts = nullptr;
     return p;
 }
 
@@ -661,7 +680,24 @@ cudaError_t issue_iteration(spg_ctx *ctx, const StepParams &p)
 
 spg_status launch_steps(spg_ctx *ctx, int k)
 {
-    const StepParams p = step_params(ctx);
+    StepParams p = step_params(ctx);
+    if (!ctx->fourier && !ctx->kread) {
+        while (k > 0) {
+            p.niter = std::min(k, ctx->iters_per_launch);
+            cudaError_t e = step_launch(ctx->var, ctx->grid, p, ctx->stream);
+            if (e == cudaErrorCooperativeLaunchTooLarge && p.niter > 1) {
+                // fewer CTAs resident than planned for (a partitioned GPU):
+                // an iteration per launch needs none of them to wait
+                cudaGetLastError();
+                ctx->iters_per_launch = 1;
+                continue;
+            }
+            CK(e, "fused step launch");
+            ctx->launches += 1;
+            k -= p.niter;
+        }
+        return SPG_OK;
+    }
     // kernels of this library per iteration
     const long long per_iter = ctx->fourier ? (ctx->xown ? 4 : 2) : 1;
     if (ctx->fourier && !ctx->xown && k > 0 && !ctx->y_fresh) {
@@ -797,25 +833,27 @@ struct Sweep {
     DevState *st = nullptr;
     VolDesc *vol = nullptr;
     TmapSet *tm = nullptr;
+    float **outs = nullptr;
     std::vector<Entry> plan;
     std::vector<int> kvals;  // extrapolation indices copied to the device (kept alive)
     int launched = 0, kmom_dev = 0;
 
     explicit Sweep(spg_ctx *c) : ctx(c), v(c->var) { v.xd = false; }
     void add(float *xk, float *xkm1, float *xout, int k) { plan.push_back({xk, xkm1, xout, k}); }
-    // device state, descriptor and tensor maps of n planned steps, from a workspace
-    static void carve(Carve &cv, size_t n, DevState **st, VolDesc **vol, TmapSet **tm)
+    // device state, descriptor, tensor maps and outputs of n planned steps, from a workspace
+    static void carve(Carve &cv, size_t n, DevState **st, VolDesc **vol, TmapSet **tm, float ***outs)
     {
         *st = cv.take<DevState>(sizeof(DevState));
         *vol = cv.take<VolDesc>(sizeof(VolDesc));
         *tm = cv.take<TmapSet>(std::max<size_t>(1, n) * sizeof(TmapSet));
+        *outs = cv.take<float *>(std::max<size_t>(1, n) * sizeof(float *));
     }
     // cv: where the step state lives (carved after what cv already holds)
     cudaError_t upload(Carve &cv)
     {
         int occ = 0;
         cudaError_t e = step_configure(v, &occ);
-        carve(cv, plan.size(), &st, &vol, &tm);
+        carve(cv, plan.size(), &st, &vol, &tm, &outs);
         if (e == cudaSuccess) e = cudaMemsetAsync(st, 0, sizeof(DevState), ctx->stream);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(vol, ctx->vols_d, sizeof(VolDesc), cudaMemcpyDeviceToDevice, ctx->stream);
@@ -829,50 +867,55 @@ struct Sweep {
             if ((e = encode_set(ctx, ctx->vols_h[0], v, xq, &h[j])) != cudaSuccess) return e;
         }
         kvals.resize(plan.size());
+        std::vector<float *> ho(plan.size());
+        for (size_t j = 0; j < plan.size(); j++) ho[j] = plan[j].xout;
         if (!h.empty())
             e = cudaMemcpyAsync(tm, h.data(), h.size() * sizeof(TmapSet), cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);  // h goes out of scope
+        if (e == cudaSuccess && !ho.empty())
+            e = cudaMemcpyAsync(outs, ho.data(), ho.size() * sizeof(float *), cudaMemcpyHostToDevice, ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);  // h and ho go out of scope
         kmom_dev = -1;  // the copied descriptor's index is the context's: set before the first step
         return e;
     }
-    cudaError_t launch()
+    // The next n planned steps (consecutive k) in as few launches as the plan allows.
+    cudaError_t launch(int n)
     {
-        const Entry &E = plan[launched];
-        cudaError_t e = cudaSuccess;
-        if (kmom_dev != E.k) {
-            kvals[launched] = E.k;
-            e = cudaMemcpyAsync(reinterpret_cast<char *>(vol) + offsetof(VolDesc, kmom), &kvals[launched],
-                                sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
+        while (n > 0) {
+            const Entry &E = plan[launched];
+            cudaError_t e = cudaSuccess;
+            if (kmom_dev != E.k) {
+                kvals[launched] = E.k;
+                e = cudaMemcpyAsync(reinterpret_cast<char *>(vol) + offsetof(VolDesc, kmom), &kvals[launched],
+                                    sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
+                if (e != cudaSuccess) return e;
+                kmom_dev = E.k;
+            }
+            StepParams p = step_params(ctx);
+            p.vols = vol;
+            p.tmaps = tm + launched;
+            for (int q = 0; q < 4; q++) p.xbuf[q] = nullptr;  // every output comes from xouts
+            p.st = st;
+            p.nvol = 1;
+            p.hist_every = 0;  // no objective, no history
+            p.restart = 0;
+            p.fourier = 0;
+            p.ybuf = nullptr;
+            p.niter = std::min(n, ctx->iters_per_launch);
+            p.tm_step = 1;
+            p.xouts = outs + launched;
+            e = step_launch(v, ctx->grid, p, ctx->stream);
+            if (e == cudaErrorCooperativeLaunchTooLarge && p.niter > 1) {
+                cudaGetLastError();
+                ctx->iters_per_launch = 1;
+                continue;
+            }
             if (e != cudaSuccess) return e;
+            ctx->launches += 1;
+            launched += p.niter;
+            kmom_dev += p.niter;
+            n -= p.niter;
         }
-        const int cur = launched % 3;  // the private state's buffer index advances by one per step
-        StepParams p;
-        p.vols = vol;
-        p.items = ctx->items_d;
-        p.sched = ctx->sched_d;
-        p.tmaps = tm + launched;
-        p.xbuf[cur] = E.xk;
-        p.xbuf[(cur + 2) % 3] = E.xkm1;
-        p.xbuf[(cur + 1) % 3] = E.xout;
-        p.xbuf[3] = nullptr;
-        p.beta = ctx->beta_d;
-        p.beta_len = ctx->max_iters;
-        p.st = st;
-        p.partials = ctx->partials_d;
-        p.hist = ctx->hist_d;
-        p.nitems = ctx->nitems;
-        p.nvol = 1;
-        p.hist_cap = ctx->hist_cap;
-        p.hist_every = 0;  // no objective, no history
-        p.restart = 0;
-        p.fourier = 0;
-        p.ybuf = nullptr;
-        p.timeout_ns = kTimeoutNs;
-        e = step_launch(v, ctx->grid, p, ctx->stream);
-        ctx->launches += 1;
-        launched++;
-        kmom_dev = E.k + 1;
-        return e;
+        return cudaSuccess;
     }
     // SPG_ETIMEOUT if a step gave up waiting for its copies (synchronises).
     spg_status status()
@@ -1777,7 +1820,8 @@ spg_status spg_unrolled(spg_ctx *ctx, int K, float *xK)
         DevState *s0;
         VolDesc *v0;
         TmapSet *t0;
-        Sweep::carve(size, (size_t)K, &s0, &v0, &t0);
+        float **o0;
+        Sweep::carve(size, (size_t)K, &s0, &v0, &t0, &o0);
         CK(workspace(ctx, size.off, &cv.base), "alloc workspace");
     }
     float *buf[3];
@@ -1791,7 +1835,7 @@ spg_status spg_unrolled(spg_ctx *ctx, int K, float *xK)
         c = (c + 1) % 3;
     }
     CK(sw.upload(cv), "plan the unrolled steps");
-    for (int k = 0; k < K; k++) CK(sw.launch(), "fused step");
+    CK(sw.launch(K), "fused step");
     spg_status s = sw.status();
     if (s != SPG_OK) return fail(ctx, s, "spg_unrolled: a fused step failed");
     s = copy_volume_out(ctx, xK, buf[c], 4, d);
@@ -1834,7 +1878,8 @@ spg_status spg_backward(spg_ctx *ctx, int K, const float *gx, float *gb, float *
             DevState *s0;
             VolDesc *v0;
             TmapSet *t0;
-            Sweep::carve(t, nsteps, &s0, &v0, &t0);
+            float **o0;
+            Sweep::carve(t, nsteps, &s0, &v0, &t0, &o0);
             CK(workspace(ctx, t.off, &cv.base), "alloc workspace");
         } else {
             cv = t;  // the steps' state follows
@@ -1878,7 +1923,7 @@ spg_status spg_backward(spg_ctx *ctx, int K, const float *gx, float *gb, float *
                                    ctx->stream),
                    "ckpt");
             }
-            CK(sw.launch(), "fused step");
+            if (k % C == 0) CK(sw.launch(std::min(C, K - k)), "fused step");
             c = (c + 1) % 3;
         }
     }
@@ -1896,7 +1941,7 @@ spg_status spg_backward(spg_ctx *ctx, int K, const float *gx, float *gb, float *
         // seg[0] = x_{k0-1}, seg[1] = x_{k0}, seg[i+1] = x_{k0+i}
         CK(cudaMemcpyAsync(vol_at(seg, 0), vol_at(ck, 2 * sgm + 1), vb, cudaMemcpyDeviceToDevice, ctx->stream), "rst");
         CK(cudaMemcpyAsync(vol_at(seg, 1), vol_at(ck, 2 * sgm), vb, cudaMemcpyDeviceToDevice, ctx->stream), "rst");
-        for (int k = k0; k < k1 - 1; k++) CK(sw.launch(), "recompute");
+        CK(sw.launch(k1 - 1 - k0), "recompute");
         for (int k = k1 - 1; k >= k0; k--) {
             const int i = k - k0 + 1;
             AdjParams a;
@@ -2077,7 +2122,7 @@ spg_status spg_autotune(spg_ctx *ctx, int trial_iters, int info[6])
     for (int t : tiles)
         for (int z : zchunks) {
             if ((s = build_plan(ctx, variant_from_tile(t, ctx->bf16(), ctx->xd()), z)) != SPG_OK) continue;
-            if ((s = launch_steps(ctx, 2)) != SPG_OK) break;  // warm-up (graph capture happens here too)
+            if ((s = launch_steps(ctx, 2)) != SPG_OK) break;  // warm-up
             cudaEventRecord(e0, ctx->stream);
             if ((s = launch_steps(ctx, trial)) != SPG_OK) break;
             cudaEventRecord(e1, ctx->stream);

@@ -62,7 +62,7 @@ struct DevState {
     int err;                 // first device-detected error (spg_status), 0 if none
     int hist_count;          // history entries written so far
     unsigned int err_info;   // where the error was raised
-    int pad;
+    unsigned int bar;        // arrivals at the fused step's barriers between iterations
 };
 
 struct StepParams {
@@ -74,14 +74,21 @@ struct StepParams {
     const float *beta;       // extrapolation table beta_k (float32)
     int beta_len;            // its length
     DevState *st;
-    double *partials;        // [nitems][4] objective sums (data, l1, tv) and restart dot of the last step
+    double *partials;        // [niter][nitems][4] objective sums (data, l1, tv) and restart dot of the launch
     double *hist;            // ring [hist_cap][nvol][5]
     int nitems, nvol, hist_cap, hist_every;
     int restart;             // gradient restart of the extrapolation, per volume
     int fourier;             // data gradient = b (A^H (N A y - D y) of the Fourier-domain term), no w tile
     float *ybuf;             // Fourier-domain term: the step also writes y_{k+1} = x_{k+1} + beta_{k+1} d_{k+1} here
     long long timeout_ns;    // bound on any single barrier wait
+    int niter;               // iterations of this launch; above 1 a cooperative launch
+    int tm_step;             // tensor-map sets from one iteration's to the next's (0: the same maps)
+    float *const *xouts;     // output volume of each iteration, or null (the buffers rotate)
 };
+
+// Work items a CTA may hold for several iterations with gradient restart in
+// one launch (their extrapolation indices live in its shared memory).
+constexpr int kMaxCtaItems = 64;
 
 // Variant of the fused step: tile = (32*vx) x ty voxels, `stages` pipeline stages.
 struct StepVariant {

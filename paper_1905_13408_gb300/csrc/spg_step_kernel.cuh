@@ -1,5 +1,5 @@
-// Fused smoothing-proximal-gradient iteration for sm_103a (one launch per
-// iteration for every volume of a context).
+// Fused smoothing-proximal-gradient iteration for sm_103a: one launch runs
+// `niter` iterations for every volume of a context.
 //
 // Per voxel v the launch computes, from x_k, d_k = x_k - x_{k-1}, b, w, om1,
 // omtv (Sec. 2.1 Eq. 12, 16, 17, 20, 21; Sec. 2.2 Eq. 28 data term):
@@ -34,6 +34,25 @@
 // the same time. Warp r of TY computes row r; one extra warp computes the +y
 // halo row and the +x halo column. p_y crosses warps through a 3-deep shared
 // ring, p_x through a lane shuffle; p_z and the z-1 values stay in registers.
+//
+// Several iterations per launch (niter > 1, a cooperative launch): the
+// iterations are separated by a barrier over the grid's CTAs instead of a
+// kernel boundary. A launch per iteration paid, on the critical path of a
+// small volume, launch latency, a chain of five dependent loads (device state,
+// schedule, item, descriptor, extrapolation weight) before the first copy
+// could start, and the last CTA's objective sums and state update before the
+// next launch could read the state. Here schedule and descriptors are read
+// once, the extrapolation index is counted, and the objective partials of
+// every iteration are kept ([niter][nitems]) and reduced after the last one
+// by all CTAs together (a warp per iteration and volume). The copies of an
+// item's first planes are issued while the previous item's last ones are
+// computed. An iteration with the objective, one per launch (replayed from a
+// graph) -> this form: 28 x 32 x 40 9.7 -> 5.4 us, 64^3 11.3 -> 7.2,
+// 128^3 18.6 -> 14.0, 101 x 147 x 183 30.7 -> 24.4, 180^3 57.6 -> 47.9,
+// 256^3 86.8 -> 81.2, 512^3 618.4 -> 617.7; a batch of 24 volumes of 96^3 ..
+// 256^3 995 -> 992. (With the producer's position in shared memory instead of
+// the item's registers the long marches lost: 623.6 at 512^3, 1128 for the
+// batch: its warp is the last to arrive at every plane's barrier.)
 #pragma once
 
 #include <cuda_bf16.h>
@@ -147,6 +166,13 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 // a - b rounded once: the product b * (-1) is exact
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+
+// Barrier of the TY row warps (named barrier 1; the halo warp takes no part).
+template <int TY>
+__device__ __forceinline__ void row_warps_sync()
+{
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * TY) : "memory");
+}
 
 // Two compensated (Kahan) float32 accumulators advanced together.
 struct KSum2 {
@@ -361,6 +387,12 @@ __device__ __forceinline__ void ld_data(const unsigned char *tile, int idx, floa
     }
 }
 
+struct StateSnap {
+    int cur, k_round, hist_count, last;
+    long long k_total;
+    int rec0, pad;  // k_total modulo the recording interval at the launch's first iteration
+};
+
 template <int VX, int TY, int S, bool BF16>
 struct Cfg {
     static constexpr int TX = 32 * VX;
@@ -384,7 +416,9 @@ struct Cfg {
     static constexpr int OFF_RED = OFF_HX + 3 * 32 * 4;       // 32 x 4 doubles
     static constexpr int OFF_BAR = OFF_RED + 32 * 4 * 8;      // S mbarriers
     static constexpr int OFF_ST = OFF_BAR + al(S * 8);        // state snapshot
-    static constexpr int TOTAL = OFF_ST + 128 + 128;          // + alignment slack
+    static constexpr int OFF_KM = OFF_ST + 128;               // extrapolation index per item (restart)
+    static constexpr int TOTAL = OFF_KM + kMaxCtaItems * 4 + 128;  // + alignment slack
+    static_assert(sizeof(StateSnap) <= 64 && sizeof(WorkItem) <= 64, "state snapshot and next item share 128 bytes");
     static constexpr int THREADS = 32 * (TY + 1);
     static_assert(TY + 1 <= 32, "reduction scratch sized for at most 32 warps");
     static_assert(TY <= 32, "halo column handled by one lane per row");
@@ -415,12 +449,6 @@ __device__ __forceinline__ void issue_stage(unsigned char *sm, uint64_t *bars, c
     }
 }
 
-struct StateSnap {
-    int cur, k_round, rec, last;
-    long long k_total;
-    float pad0, pad1;
-};
-
 // Shared-memory carve-up of one CTA.
 struct Smem {
     unsigned char *sm;
@@ -429,21 +457,30 @@ struct Smem {
     float *hx_ring;
     double *red;
     StateSnap *snap;
+    WorkItem *next;  // the item after the current one (producer lane only)
+    int *kmom;  // restart: extrapolation index of each of the CTA's items
 };
 
-// Pipeline bookkeeping of one CTA (owned by thread 0 where noted).
+// Pipeline bookkeeping of one CTA (issued: producer lane only).
 struct Pipe {
-    unsigned gstep;         // steps consumed so far
-    unsigned issued_upto;   // steps issued so far (thread 0)
-    unsigned drain_from;    // first step that may be pending after an abort
+    unsigned gstep;       // steps consumed so far
+    unsigned iter_first;  // first step of the current iteration
+    unsigned issued;      // steps issued so far
+    unsigned drain_from;  // first step that may be pending after an abort
 };
 
 // One work item: plane-by-plane march over [z0, z1) of one x-y tile.
-// REC adds the three sums of F(x_k) (data, l1, TV) for the item.
-// Returns true when a barrier wait gave up (the CTA then stops).
+// REC adds the three sums of F(x_k) (data, l1, TV) for the item, written to
+// `part`. kmom: the volume's extrapolation index in this iteration; tm: the
+// iteration's tensor maps (of every volume); next_it: the CTA's next item in
+// this iteration (-1: none), whose first planes the producer fetches while
+// this item's last ones are computed. Ends with a barrier over the CTA
+// after the item's last stores. Returns true when a barrier wait gave up (the
+// CTA then stops).
 template <int VX, int TY, int S, bool BF16, bool XD, bool REC, bool DOT, bool FOURIER>
-__device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pipe &pp_, const WorkItem &W, int it,
-                                         int ia, int ib, float *xout_base, float *dout_base)
+__device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pipe &pp_, const WorkItem &W,
+                                         int next_it, double *part, int kmom, const TmapSet *tm, int ia, int ib,
+                                         float *xout_base, float *dout_base)
 {
     using C = Cfg<VX, TY, S, BF16>;
     constexpr int TX = C::TX, XW = C::XW, OW = C::OW;
@@ -451,10 +488,9 @@ __device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pi
     const bool main_warp = warp < TY;
     const int r = warp;  // tile row of this warp (r == TY: the +y halo row)
     const VolDesc V = P.vols[W.vol];
-    const TmapSet *tm = P.tmaps + W.vol;
     const int nsteps = (W.z1 - W.z0) + 2;
-    const float beta = SPG_GUARD(P.st, V.kmom >= 0 && V.kmom < P.beta_len, 2u) ? P.beta[V.kmom] : 0.f;
-    const float beta_next = (FOURIER && V.kmom + 1 < P.beta_len) ? P.beta[V.kmom + 1] : 0.f;
+    const float beta = SPG_GUARD(P.st, kmom >= 0 && kmom < P.beta_len, 2u) ? P.beta[kmom] : 0.f;
+    const float beta_next = (FOURIER && kmom + 1 < P.beta_len) ? P.beta[kmom + 1] : 0.f;
     // (per volume: restarts reset a volume's extrapolation index)
     const float tau = V.tau, lam_tv = V.lambda_tv, tl1 = V.tau * V.lambda_l1;
     const float inv_mu = 1.0f / V.mu, half_inv_mu = 0.5f / V.mu, half_mu = 0.5f * V.mu;
@@ -463,10 +499,25 @@ __device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pi
 
     // the TMA producer is lane 0 of the halo warp, which has no write phase
     const bool producer = (warp == TY) && (lane == 0);
+    // Producer: copies of the CTA's plane step d steps into this item, or
+    // past its end into the next one's (an item has at least 3 steps, so d
+    // never reaches a third item).
+    static_assert(S <= 4, "the producer runs at most 3 steps ahead");
+    auto issue = [&](int d) {
+        if (d < nsteps) {
+            issue_stage<C, S, !FOURIER>(sh.sm, sh.bars, tm + W.vol, W, ia, ib, g0, d);
+        } else if (next_it >= 0) {
+            const WorkItem N = *sh.next;
+            issue_stage<C, S, !FOURIER>(sh.sm, sh.bars, tm + N.vol, N, ia, ib, g0 + (unsigned)nsteps, d - nsteps);
+        } else {
+            return;
+        }
+        pp_.issued++;
+    };
     if (producer) {
-        const int pro = nsteps < S ? nsteps : S;
-        for (int j = 0; j < pro; j++) issue_stage<C, S, !FOURIER>(sh.sm, sh.bars, tm, W, ia, ib, g0, j);
-        pp_.issued_upto = g0 + pro;
+        if (next_it >= 0) *sh.next = P.items[next_it];
+        if (g0 == pp_.iter_first)
+            for (int d = 0; d < S; d++) issue(d);
     }
 
     // registers carried across z-steps
@@ -586,11 +637,9 @@ __device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pi
             pp_.drain_from = g0 + j;
             break;
         }
-        // refill the stage consumed in step j-1
-        if (producer && j >= 1 && j - 1 + S < nsteps) {
-            issue_stage<C, S, !FOURIER>(sh.sm, sh.bars, tm, W, ia, ib, g0, j - 1 + S);
-            pp_.issued_upto = g0 + j + S;
-        }
+        // refill the stage of the step before this one (of this item or of the
+        // one before), which every warp has finished with
+        if (producer && g0 + j != pp_.iter_first) issue(j - 1 + S);
 
         // ---- B: write plane z-1 ----
         if (main_warp && j >= 2) {
@@ -641,35 +690,125 @@ __device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pi
     }
 
     if (!aborted && (REC || DOT)) {
-        // block reduction of the item's sums, fixed order (float-float, or
-        // double where a float-float could overflow: spg_ff.cuh)
+        // reduction of the item's sums over the row warps (the halo warp has
+        // none and goes on), fixed order, in float-float or, where that could
+        // overflow, in double (spg_ff.cuh)
         const ff::FF d = kdl.value_x();
         const ff::FF v[4] = {{0.5f * d.hi, 0.5f * d.lo}, kdl.value_y(), kt.value(), kr.value()};
         const bool big = ff::too_big(v[0]) || ff::too_big(v[1]) || ff::too_big(v[2]) || ff::too_big(v[3]);
-        double *const out = P.partials + (long long)it * 4;
-        if (!__syncthreads_or(big ? 1 : 0)) {
-            ff::FF *const red = reinterpret_cast<ff::FF *>(sh.red);
-            const ff::FF s = ff::warp_sum4(v, lane);
-            if ((lane & 7) == 0) red[warp * 4 + (lane >> 3)] = s;
-            __syncthreads();
-            if (warp == 0) {
-                const ff::FF t = ff::cross_warp_sum4(red, TY + 1, lane, ff::FF{0.f, 0.f});
-                if (lane < 4) out[lane] = ff::to_double(t);
-            }
-        } else {
-            const double w[4] = {ff::to_double(v[0]), ff::to_double(v[1]), ff::to_double(v[2]), ff::to_double(v[3])};
-            const double s = ff::warp_sum4(w, lane);
-            if ((lane & 7) == 0) sh.red[warp * 4 + (lane >> 3)] = s;
-            __syncthreads();
-            if (warp == 0) {
-                const double t = ff::cross_warp_sum4(sh.red, TY + 1, lane, 0.0);
-                if (lane < 4) out[lane] = t;
+        const bool wide = __syncthreads_or(big ? 1 : 0) != 0;
+        if (main_warp) {
+            if (!wide) {
+                ff::FF *const red = reinterpret_cast<ff::FF *>(sh.red);
+                const ff::FF s = ff::warp_sum4(v, lane);
+                if ((lane & 7) == 0) red[warp * 4 + (lane >> 3)] = s;
+                row_warps_sync<TY>();
+                if (warp == 0) {
+                    const ff::FF t = ff::cross_warp_sum4(red, TY, lane, ff::FF{0.f, 0.f});
+                    if (lane < 4) part[lane] = ff::to_double(t);
+                }
+            } else {
+                const double w[4] = {ff::to_double(v[0]), ff::to_double(v[1]), ff::to_double(v[2]),
+                                     ff::to_double(v[3])};
+                const double s = ff::warp_sum4(w, lane);
+                if ((lane & 7) == 0) sh.red[warp * 4 + (lane >> 3)] = s;
+                row_warps_sync<TY>();
+                if (warp == 0) {
+                    const double t = ff::cross_warp_sum4(sh.red, TY, lane, 0.0);
+                    if (lane < 4) part[lane] = t;
+                }
             }
         }
+        if constexpr (DOT) __syncthreads();  // the next iteration's extrapolation depends on the sums
+    } else {
+        __syncthreads();
     }
-    __syncthreads();  // every stage consumed before the next item's prologue
     if (!aborted) pp_.gstep = g0 + nsteps;
     return aborted;
+}
+
+// Barrier over the CTAs of the grid (all resident: cooperative launch), the
+// producer lane's half: the CTA's stores of the iteration precede it (a CTA
+// barrier), are made visible, and the other CTAs' are visible to this CTA's
+// copies when it returns true. False when it gave up (bounded, or another
+// CTA did).
+__device__ __forceinline__ bool grid_barrier(DevState *st, unsigned target, long long limit_ns)
+{
+    // the next copies (async proxy) read what the grid's threads wrote with
+    // ordinary stores
+    asm volatile("fence.proxy.async;" ::: "memory");
+    __threadfence();
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&st->bar) : "memory");
+    const long long t0 = global_ns();
+    for (;;) {
+        for (int i = 0; i < 64; i++) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&st->bar) : "memory");
+            if (v >= target) {
+                __threadfence();
+                asm volatile("fence.proxy.async;" ::: "memory");
+                return true;
+            }
+        }
+        if (*(volatile int *)&st->err == (int)SPG_ETIMEOUT || global_ns() - t0 > limit_ns) return false;
+    }
+}
+
+// Iterations of this launch before iteration i that record the objective.
+__device__ __forceinline__ int recorded_before(int rec0, int every, int i)
+{
+    return every <= 0 ? 0 : (i + rec0 + every - 1) / every - (rec0 + every - 1) / every;
+}
+
+// Sums of volume V's item partials (one warp, fixed order): every lane gets
+// all four.
+__device__ __forceinline__ void volume_sums(const VolDesc &V, const double *part, int lane, double (&a)[4])
+{
+    a[0] = a[1] = a[2] = a[3] = 0.0;
+    for (int q = V.item_begin + lane; q < V.item_end; q += 32)
+        for (int c = 0; c < 4; c++) a[c] += __ldcg(part + (long long)q * 4 + c);
+    const double s = ff::warp_sum4(a, lane);
+#pragma unroll
+    for (int c = 0; c < 4; c++) a[c] = __shfl_sync(FULL, s, 8 * c);
+}
+
+// The restart product of volume V alone.
+__device__ __forceinline__ double volume_dot(const VolDesc &V, const double *part, int lane)
+{
+    double a = 0.0;
+    for (int q = V.item_begin + lane; q < V.item_end; q += 32) a += __ldcg(part + (long long)q * 4 + 3);
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) a += __shfl_xor_sync(FULL, a, m);
+    return a;
+}
+
+// Objective history of the launch: warp w of `nw` takes the (iteration,
+// volume) pairs w, w + nw, ... of those that record. Of more than hist_cap
+// entries only the newest are written (the ring keeps no others).
+__device__ __forceinline__ void write_history(const StepParams &P, const StateSnap &S, int w, int nw, int lane)
+{
+    const int total = recorded_before(S.rec0, P.hist_every, P.niter);
+    for (long long e = w; e < (long long)P.niter * P.nvol; e += nw) {
+        const int i = (int)(e / P.nvol), v = (int)(e % P.nvol);
+        if (P.hist_every <= 0 || (S.rec0 + i) % P.hist_every != 0) continue;
+        const int rank = recorded_before(S.rec0, P.hist_every, i);
+        if (total - rank > P.hist_cap) continue;
+        const VolDesc V = P.vols[v];
+        double a[4];
+        volume_sums(V, P.partials + (long long)i * P.nitems * 4, lane, a);
+        if (lane == 0) {
+            const int slot = (int)(((long long)S.hist_count + rank) % P.hist_cap);
+            double *h = P.hist + ((long long)slot * P.nvol + v) * 5;
+            const double l1 = (double)V.lambda_l1 * a[1], tv = (double)V.lambda_tv * a[2];
+            const double tot = a[0] + l1 + tv;
+            h[0] = (double)(S.k_total + i);
+            h[1] = a[0];
+            h[2] = l1;
+            h[3] = tv;
+            h[4] = tot;
+            if (!isfinite(tot)) atomicCAS(&P.st->err, 0, (int)SPG_ENONFINITE);
+        }
+    }
 }
 
 template <int VX, int TY, int S, bool BF16, bool XD, int MINB>
@@ -689,81 +828,134 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
     sh.snap = reinterpret_cast<StateSnap *>(sh.sm + C::OFF_ST);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+    sh.next = reinterpret_cast<WorkItem *>(sh.sm + C::OFF_ST + 64);
+    sh.kmom = reinterpret_cast<int *>(sh.sm + C::OFF_KM);
+    const bool producer = (warp == TY) && (lane == 0);
+
     if (tid == 0) {
         volatile DevState *st = P.st;
         StateSnap s;
         s.cur = st->cur;
         s.k_round = st->k_round;
         s.k_total = st->k_total;
-        s.rec = (P.hist_every > 0 && (s.k_total % P.hist_every) == 0) ? 1 : 0;
+        s.hist_count = st->hist_count;
+        s.rec0 = P.hist_every > 0 ? (int)(s.k_total % P.hist_every) : 0;
         s.last = 0;
+        s.pad = 0;
         *sh.snap = s;
         for (int i = 0; i < S; i++) mbar_init(&sh.bars[i], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    const int p0 = P.sched[blockIdx.x], p1 = P.sched[blockIdx.x + 1];
     __syncthreads();
-    // buffers: XD keeps x in 0/1 and d in 2/3; otherwise x_{k-1}, x_k, x_{k+1} rotate over 0..2
-    const int cur = sh.snap->cur;
-    const int nxt = XD ? (cur ^ 1) : (cur + 1) % 3;
-    const int ia = cur, ib = XD ? 2 + cur : (cur + 2) % 3;
-    const bool rec = sh.snap->rec != 0;
     // select without indexing the parameter array (keeps the parameters out of local memory)
     auto pick = [&](int i) { return i == 0 ? P.xbuf[0] : (i == 1 ? P.xbuf[1] : (i == 2 ? P.xbuf[2] : P.xbuf[3])); };
-    float *const xout_base = pick(nxt);
-    float *const dout_base = XD ? pick(2 + nxt) : nullptr;
-    if (tid == 0) {
-        const int p0 = P.sched[blockIdx.x];
-        const TmapSet *tm = P.tmaps + P.items[P.sched[gridDim.x + 1 + (p0 < P.nitems ? p0 : 0)]].vol;
-        prefetch_tmap(&tm->x[ia]);
-        prefetch_tmap(&tm->x[ib]);
-        prefetch_tmap(&tm->omtv);
-        prefetch_tmap(&tm->b);
-        prefetch_tmap(&tm->w);
-        prefetch_tmap(&tm->om1);
-    }
+    const bool many = P.niter > 1;
 
-    Pipe pipe{0, 0, 0};
+    Pipe pipe{0, 0, 0, 0};
     bool aborted = false;
-    const int p1 = P.sched[blockIdx.x + 1];
-    for (int p = P.sched[blockIdx.x]; p < p1 && !aborted; p++) {
-        const int it = P.sched[gridDim.x + 1 + p];
-        if (!SPG_GUARD(P.st, p1 <= P.nitems && it >= 0 && it < P.nitems, 1u)) break;
-        const WorkItem W = P.items[it];
-        bool done = false;
-        if constexpr (!BF16 && XD) {
-            // Fourier-domain data term (float32 storage, increment storage only)
-            if (P.fourier) {
-                aborted = rec ? run_item<VX, TY, S, BF16, XD, true, false, true>(P, sh, pipe, W, it, ia, ib,
-                                                                                 xout_base, dout_base)
-                              : run_item<VX, TY, S, BF16, XD, false, false, true>(P, sh, pipe, W, it, ia, ib,
-                                                                                  xout_base, dout_base);
-                done = true;
+    int cur = sh.snap->cur;
+    int rec_in = sh.snap->rec0;  // iterations since the last recorded one (0: this one records)
+    for (int itn = 0; itn < P.niter && !aborted; itn++) {
+        // buffers: XD keeps x in 0/1 and d in 2/3; otherwise x_{k-1}, x_k, x_{k+1} rotate over 0..2
+        const int nxt = XD ? (cur ^ 1) : (cur + 1) % 3;
+        const int ia = cur, ib = XD ? 2 + cur : (cur + 2) % 3;
+        const bool rec = P.hist_every > 0 && rec_in == 0;
+        float *const xout_base = P.xouts ? P.xouts[itn] : pick(nxt);
+        float *const dout_base = XD ? pick(2 + nxt) : nullptr;
+        const TmapSet *const tm = P.tmaps + (long long)itn * P.tm_step;
+        pipe.iter_first = pipe.gstep;
+        if (producer && p0 < p1 && (itn == 0 || P.tm_step)) {
+            const TmapSet *t = tm + P.items[P.sched[gridDim.x + 1 + p0]].vol;
+            prefetch_tmap(&t->x[ia]);
+            prefetch_tmap(&t->x[ib]);
+            prefetch_tmap(&t->omtv);
+            prefetch_tmap(&t->b);
+            prefetch_tmap(&t->w);
+            prefetch_tmap(&t->om1);
+        }
+        for (int p = p0; p < p1 && !aborted; p++) {
+            const int it = P.sched[gridDim.x + 1 + p];
+            if (!SPG_GUARD(P.st, p1 <= P.nitems && it >= 0 && it < P.nitems, 1u)) {
+                aborted = true;
+                pipe.drain_from = pipe.gstep;
+                break;
+            }
+            const WorkItem W = P.items[it];
+            const int next_it = p + 1 < p1 ? P.sched[gridDim.x + 2 + p] : -1;
+            const int kmom = (P.restart && many && itn > 0) ? sh.kmom[p - p0] : P.vols[W.vol].kmom + itn;
+            double *const part = P.partials + ((long long)itn * P.nitems + it) * 4;
+            bool done = false;
+            if constexpr (!BF16 && XD) {
+                // Fourier-domain data term (float32 storage, increment storage only)
+                if (P.fourier) {
+                    aborted = rec ? run_item<VX, TY, S, BF16, XD, true, false, true>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base)
+                                  : run_item<VX, TY, S, BF16, XD, false, false, true>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base);
+                    done = true;
+                }
+            }
+            if (!done) {
+                if (P.restart)
+                    aborted = rec ? run_item<VX, TY, S, BF16, XD, true, true, false>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base)
+                                  : run_item<VX, TY, S, BF16, XD, false, true, false>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base);
+                else
+                    aborted = rec ? run_item<VX, TY, S, BF16, XD, true, false, false>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base)
+                                  : run_item<VX, TY, S, BF16, XD, false, false, false>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base);
             }
         }
-        if (!done) {
-            if (P.restart)
-                aborted = rec ? run_item<VX, TY, S, BF16, XD, true, true, false>(P, sh, pipe, W, it, ia, ib,
-                                                                                 xout_base, dout_base)
-                              : run_item<VX, TY, S, BF16, XD, false, true, false>(P, sh, pipe, W, it, ia, ib,
-                                                                                  xout_base, dout_base);
-            else
-                aborted = rec ? run_item<VX, TY, S, BF16, XD, true, false, false>(P, sh, pipe, W, it, ia, ib,
-                                                                                  xout_base, dout_base)
-                              : run_item<VX, TY, S, BF16, XD, false, false, false>(P, sh, pipe, W, it, ia, ib,
-                                                                                   xout_base, dout_base);
+        if (aborted) break;
+        if (many) {
+            bool ok = true;
+            if (producer) ok = grid_barrier(P.st, (unsigned)(itn + 1) * gridDim.x, P.timeout_ns);
+            if (__syncthreads_or(ok ? 0 : 1)) {
+                aborted = true;
+                pipe.drain_from = pipe.gstep;
+            } else if (P.restart && itn + 1 < P.niter) {
+                // the extrapolation index of the next iteration, per item
+                const double *const parts = P.partials + (long long)itn * P.nitems * 4;
+                for (int p = p0 + warp; p < p1; p += TY + 1) {
+                    const VolDesc V = P.vols[P.items[P.sched[gridDim.x + 1 + p]].vol];
+                    const int km = itn > 0 ? sh.kmom[p - p0] : V.kmom;
+                    const bool again = volume_dot(V, parts, lane) > 0.0;
+                    if (lane == 0) sh.kmom[p - p0] = again ? 0 : km + 1;
+                }
+                __syncthreads();
+            }
         }
+        cur = nxt;
+        rec_in = rec_in + 1 == P.hist_every ? 0 : rec_in + 1;
     }
 
-    if (aborted && warp == TY && lane == 0) {
+    if (aborted && producer) {
         // record the timeout, then wait (bounded) for copies still in flight
         atomicCAS(&P.st->err, 0, (int)SPG_ETIMEOUT);
-        for (unsigned q = pipe.drain_from; q < pipe.issued_upto; q++) {
+        for (unsigned q = pipe.drain_from; q < pipe.issued; q++) {
             const int s = (int)(q % S);
             (void)mbar_wait(&sh.bars[s], (uint32_t)((q / S) & 1), P.timeout_ns);
         }
     }
 
-    // ---- last CTA: per-volume objective, then advance the device state ----
+    // ---- objective history, extrapolation indices, device state ----
+    VolDesc *const vols_rw = const_cast<VolDesc *>(P.vols);
+    const StateSnap snap = *sh.snap;
+    if (many && !aborted) {
+        // after the last grid barrier every CTA sees every partial
+        write_history(P, snap, blockIdx.x * (TY + 1) + warp, gridDim.x * (TY + 1), lane);
+        const double *const parts = P.partials + (long long)(P.niter - 1) * P.nitems * 4;
+        for (int p = p0 + warp; p < p1; p += TY + 1) {
+            // a volume's descriptor is advanced by the CTA that runs its first item
+            const int it = P.sched[gridDim.x + 1 + p];
+            const int v = P.items[it].vol;
+            const VolDesc V = P.vols[v];
+            if (it != V.item_begin) continue;
+            const int km = P.restart ? sh.kmom[p - p0] : V.kmom + P.niter - 1;  // index of the last iteration
+            const bool again = P.restart && volume_dot(V, parts, lane) > 0.0;
+            if (lane == 0) {
+                vols_rw[v].beta_last = P.beta[km];
+                vols_rw[v].kmom = again ? 0 : km + 1;
+            }
+        }
+    }
     __syncthreads();
     if (tid == 0) {
         __threadfence();
@@ -773,47 +965,28 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
     __syncthreads();
     if (!sh.snap->last) return;
     __threadfence();
-    {
-        // per volume: objective history (recorded steps), restart test, and
-        // the extrapolation index of the next step
-        const int hslot = P.st->hist_count % P.hist_cap;
-        const bool sums = rec || P.restart != 0;
-        VolDesc *vols_rw = const_cast<VolDesc *>(P.vols);
+    if (!many) {
+        // one iteration: the last CTA sums the objective and advances every volume
+        write_history(P, snap, warp, TY + 1, lane);
         for (int v = warp; v < P.nvol; v += TY + 1) {
             const VolDesc V = P.vols[v];
-            double a[4] = {0, 0, 0, 0};
-            if (sums) {
-                for (int q = V.item_begin + lane; q < V.item_end; q += 32)
-                    for (int c = 0; c < 4; c++) a[c] += __ldcg(P.partials + (long long)q * 4 + c);
-                const double s = ff::warp_sum4(a, lane);
-#pragma unroll
-                for (int c = 0; c < 4; c++) a[c] = __shfl_sync(FULL, s, 8 * c);
-            }
+            const bool again = P.restart && volume_dot(V, P.partials, lane) > 0.0;
+            __syncwarp();
             if (lane == 0) {
-                if (rec) {
-                    double *h = P.hist + ((long long)hslot * P.nvol + v) * 5;
-                    const double l1 = (double)V.lambda_l1 * a[1], tv = (double)V.lambda_tv * a[2];
-                    const double tot = a[0] + l1 + tv;
-                    h[0] = (double)sh.snap->k_total;
-                    h[1] = a[0];
-                    h[2] = l1;
-                    h[3] = tv;
-                    h[4] = tot;
-                    if (!isfinite(tot)) atomicCAS(&P.st->err, 0, (int)SPG_ENONFINITE);
-                }
                 vols_rw[v].beta_last = P.beta[V.kmom];
-                vols_rw[v].kmom = (P.restart != 0 && a[3] > 0.0) ? 0 : V.kmom + 1;
+                vols_rw[v].kmom = again ? 0 : V.kmom + 1;
             }
         }
     }
     __syncthreads();
     if (tid == 0) {
         DevState *st = P.st;
-        if (rec) st->hist_count = st->hist_count + 1;
-        st->cur = nxt;
-        st->k_round = sh.snap->k_round + 1;
-        st->k_total = sh.snap->k_total + 1;
+        st->hist_count = snap.hist_count + recorded_before(snap.rec0, P.hist_every, P.niter);
+        st->cur = XD ? (snap.cur + P.niter) & 1 : (snap.cur + P.niter) % 3;
+        st->k_round = snap.k_round + P.niter;
+        st->k_total = snap.k_total + P.niter;
         st->ticket = 0;
+        st->bar = 0;
         __threadfence();
     }
 }
@@ -830,8 +1003,23 @@ struct Launcher {
     }
     static cudaError_t launch(int grid, const StepParams &p, cudaStream_t s)
     {
-        spg_step_kernel<VX, TY, S, BF16, XD, MINB><<<grid, C::THREADS, C::TOTAL, s>>>(p);
-        return cudaGetLastError();
+        auto k = spg_step_kernel<VX, TY, S, BF16, XD, MINB>;
+        if (p.niter == 1) {
+            k<<<grid, C::THREADS, C::TOTAL, s>>>(p);
+            return cudaGetLastError();
+        }
+        // the iterations of one launch wait on one another: all CTAs resident
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(C::THREADS);
+        cfg.dynamicSmemBytes = C::TOTAL;
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, k, p);
     }
 };
 

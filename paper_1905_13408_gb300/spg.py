@@ -532,7 +532,7 @@ def volume_params(shape, lambda_l1=0.05, lambda_tv=0.1, mu=1e-3, eps=1e-3, eps_t
 
 
 class SPG:
-    """A solver context over one or more volumes (one fused launch per iteration)."""
+    """A solver context over one or more volumes (each iteration one fused pass over all of them)."""
 
     def __init__(self, volumes, data_dtype="f32", momentum="fista", hist_every=1, hist_capacity=4096,
                  max_iters=100000, tile="auto", zchunk=0, ctas_per_sm=0, storage="delta", restart=False,
