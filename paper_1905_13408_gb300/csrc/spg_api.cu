@@ -241,24 +241,6 @@ int tile_code(const StepVariant &v)
     return 0;
 }
 
-// Built-in tile choice: the widest tile that the volumes fill well.
-StepVariant default_variant(const spg_ctx *c)
-{
-    long long vox = 0, waste128 = 0, waste64 = 0;
-    for (const auto &v : c->vols_h) {
-        const long long n = (long long)v.nx * v.ny * v.nz;
-        vox += n;
-        waste128 += (round_up(v.nx, 128) - v.nx) * (long long)v.ny * v.nz;
-        waste64 += (round_up(v.nx, 64) - v.nx) * (long long)v.ny * v.nz;
-    }
-    const bool wide = waste128 <= vox / 8;
-    // 4 copy stages in flight: two CTAs per SM still fit (2 x 111 KB of shared
-    // memory), and at 512^3 the deeper pipeline moves 8 % more bytes per second
-    if (wide) return {4, 7, 4, c->bf16(), c->xd()};
-    if (waste64 <= vox / 8) return {2, 7, 4, c->bf16(), c->xd()};
-    return {2, 4, 4, c->bf16(), c->xd()};
-}
-
 cudaError_t encode_map(CUtensorMap *m, CUtensorMapDataType dt, void *base, const VolDesc &v, size_t es, int bx,
                        int by)
 {
@@ -353,64 +335,130 @@ long long lpt_schedule(const std::vector<long long> &cost, int G, std::vector<in
     return makespan;
 }
 
+// Item costs of the context's volumes cut into z-chunks of `chunk` planes.
+std::vector<long long> chunk_costs(const spg_ctx *ctx, int TX, int TY, int chunk)
+{
+    std::vector<long long> c;
+    for (const auto &d : ctx->vols_h) {
+        const long long cols = (long long)((d.nx + TX - 1) / TX) * ((d.ny + TY - 1) / TY);
+        const int nzi = d.nz - d.halo_lo - d.halo_hi;  // planes written (halo planes are only read)
+        const int nch = (nzi + chunk - 1) / chunk;
+        for (int q = 0; q < nch; q++) {
+            const int z0 = (int)((long long)nzi * q / nch), z1 = (int)((long long)nzi * (q + 1) / nch);
+            if (z1 > z0) c.insert(c.end(), cols, item_cost(z0, z1));
+        }
+    }
+    return c;
+}
+
+// Planes per work item for variant v with `slots` resident CTAs: the z-chunk
+// whose items, scheduled longest first, give the shortest makespan (one wave
+// of equal items when every column fits; finer chunks balance uneven
+// batches). *makespan in plane steps.
+int best_chunk(const spg_ctx *ctx, const StepVariant &v, long long slots, long long *makespan)
+{
+    const int TX = 32 * v.vx, TY = v.ty;
+    long long columns = 0, plane_tiles = 0;
+    int maxnz = 0;
+    for (const auto &d : ctx->vols_h) {
+        const long long cols = (long long)((d.nx + TX - 1) / TX) * ((d.ny + TY - 1) / TY);
+        columns += cols;
+        plane_tiles += cols * (d.nz - d.halo_lo - d.halo_hi);
+        maxnz = std::max(maxnz, d.nz);
+    }
+    std::vector<int> cand = {8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024};
+    for (int k = 1; k <= 16; k++) cand.push_back((maxnz + k - 1) / k);
+    if (columns <= slots) {
+        const long long per = std::max<long long>(1, slots / columns);
+        cand.push_back((int)((maxnz + per - 1) / per));
+    }
+    std::sort(cand.begin(), cand.end(), std::greater<int>());
+    long long best = -1;
+    int chunk = maxnz;
+    for (int c : cand) {
+        if (c < 1 || c > maxnz) continue;
+        if (plane_tiles / c > 400000) continue;  // keep the plan small
+        // no schedule is shorter than the work over the CTAs: skip a chunk that
+        // cannot win (of equal makespans the larger chunk, seen first, stays)
+        long long total = 0;
+        for (const auto &d : ctx->vols_h) {
+            const long long nzi = d.nz - d.halo_lo - d.halo_hi;
+            total += (long long)((d.nx + TX - 1) / TX) * ((d.ny + TY - 1) / TY) * (nzi + 2 * ((nzi + c - 1) / c));
+        }
+        if (best >= 0 && (total + slots - 1) / slots >= best) continue;
+        const auto cost = chunk_costs(ctx, TX, TY, c);
+        const int G = (int)std::min<long long>((long long)cost.size(), slots);
+        const long long ms = lpt_schedule(cost, G, nullptr, nullptr);
+        if (best < 0 || ms < best) {
+            best = ms;
+            chunk = c;
+        }
+    }
+    *makespan = best < 0 ? LLONG_MAX / 4 : best;
+    return std::max(1, chunk);
+}
+
+cudaError_t resident_ctas(const spg_ctx *ctx, const StepVariant &v, int *occ)
+{
+    const cudaError_t e = step_configure(v, occ);
+    if (e == cudaSuccess && ctx->opt.ctas_per_sm > 0) *occ = std::min(*occ, ctx->opt.ctas_per_sm);
+    return e;
+}
+
+// Built-in tile choice: the variant with the shortest makespan times its time
+// per plane step. Measured on volumes that stay in L2 (every resident CTA
+// marching; iteration time less the 3.2-3.5 us an iteration takes whatever its
+// steps): 128x7 with 4 copy stages 1.05 us a step, 64x7 0.80, 64x4 0.77. A
+// 128-wide step costs far less than two 64-wide ones, so the wide tile is the
+// better one as soon as a row is longer than 64, however much of its last
+// tile lies outside: 128x7 against 64-wide tiles, iterations with the objective:
+// 96^3 11.0 against 12.8 us, 101 x 147 x 183 21.3 / 24.8, 180^3 42.7 / 47.8,
+// 200^3 48.1 / 69.9, 40 x 300 x 300 27.0 / 32.8; the other way round
+// 64^3 8.8 / 7.3, 119 x 229 x 29 19.8 / 15.4.
+StepVariant default_variant(const spg_ctx *ctx)
+{
+    struct Choice {
+        StepVariant v;
+        double step_us;
+    };
+    const bool bf16 = ctx->bf16(), xd = ctx->xd();
+    const Choice choices[] = {{{4, 7, 4, bf16, xd}, 1.05}, {{2, 7, 4, bf16, xd}, 0.80}, {{2, 4, 4, bf16, xd}, 0.77}};
+    StepVariant best = choices[0].v;
+    double best_us = -1.0;
+    for (const Choice &c : choices) {
+        int occ = 0;
+        if (resident_ctas(ctx, c.v, &occ) != cudaSuccess || occ < 1) {
+            cudaGetLastError();
+            continue;
+        }
+        long long steps = 0;
+        const long long slots = (long long)ctx->num_sms * occ;
+        if (ctx->opt.zchunk > 0) {
+            const auto cost = chunk_costs(ctx, 32 * c.v.vx, c.v.ty, ctx->opt.zchunk);
+            steps = lpt_schedule(cost, (int)std::min<long long>((long long)cost.size(), slots), nullptr, nullptr);
+        } else {
+            best_chunk(ctx, c.v, slots, &steps);
+        }
+        const double us = (double)steps * c.step_us;
+        if (best_us < 0.0 || us < best_us) {
+            best_us = us;
+            best = c.v;
+        }
+    }
+    return best;
+}
+
 // Work plan: tensor maps for the variant's boxes, work items, grid size.
 spg_status build_plan(spg_ctx *ctx, const StepVariant &v, int zchunk_opt)
 {
     if (!step_variant_supported(v)) return fail(ctx, SPG_EINVAL, "unsupported tile variant");
     int occ = 0;
-    CK(step_configure(v, &occ), "configure fused step");
+    CK(resident_ctas(ctx, v, &occ), "configure fused step");
     if (occ < 1) return fail(ctx, SPG_ECUDA, "fused step does not fit on an SM");
-    if (ctx->opt.ctas_per_sm > 0) occ = std::min(occ, ctx->opt.ctas_per_sm);
     const int TX = 32 * v.vx, TY = v.ty;
     const long long slots = (long long)ctx->num_sms * occ;
-
-    long long columns = 0, plane_tiles = 0;
-    for (const auto &d : ctx->vols_h) {
-        const long long cols = (long long)((d.nx + TX - 1) / TX) * ((d.ny + TY - 1) / TY);
-        columns += cols;
-        plane_tiles += cols * (d.nz - d.halo_lo - d.halo_hi);
-    }
-    // Planes per work item: the z-chunk whose items, scheduled longest first
-    // over the resident CTAs, give the shortest makespan (one wave of equal
-    // items when every column fits; finer chunks balance uneven batches).
-    auto costs_for = [&](int chunk) {
-        std::vector<long long> c;
-        for (const auto &d : ctx->vols_h) {
-            const long long cols = (long long)((d.nx + TX - 1) / TX) * ((d.ny + TY - 1) / TY);
-            const int nzi = d.nz - d.halo_lo - d.halo_hi;  // planes written (halo planes are only read)
-            const int nch = (nzi + chunk - 1) / chunk;
-            for (int q = 0; q < nch; q++) {
-                const int z0 = (int)((long long)nzi * q / nch), z1 = (int)((long long)nzi * (q + 1) / nch);
-                if (z1 > z0) c.insert(c.end(), cols, item_cost(z0, z1));
-            }
-        }
-        return c;
-    };
-    int maxnz = 0;
-    for (const auto &d : ctx->vols_h) maxnz = std::max(maxnz, d.nz);
-    int chunk;
-    if (zchunk_opt > 0) {
-        chunk = zchunk_opt;
-    } else {
-        std::vector<int> cand = {8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024};
-        for (int k = 1; k <= 16; k++) cand.push_back((maxnz + k - 1) / k);
-        if (columns <= slots) cand.push_back((int)((maxnz + std::max<long long>(1, slots / columns) - 1) /
-                                                   std::max<long long>(1, slots / columns)));
-        long long best = -1;
-        chunk = maxnz;
-        for (int c : cand) {
-            if (c < 1 || c > maxnz) continue;
-            if (plane_tiles / c > 400000) continue;  // keep the plan small
-            const auto cost = costs_for(c);
-            const int G = (int)std::min<long long>((long long)cost.size(), slots);
-            const long long ms = lpt_schedule(cost, G, nullptr, nullptr);
-            if (best < 0 || ms < best || (ms == best && c > chunk)) {
-                best = ms;
-                chunk = c;
-            }
-        }
-    }
-    chunk = std::max(1, chunk);
+    long long makespan = 0;
+    const int chunk = zchunk_opt > 0 ? zchunk_opt : best_chunk(ctx, v, slots, &makespan);
 
     std::vector<WorkItem> items;
     for (int j = 0; j < ctx->nvol; j++) {
