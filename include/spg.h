@@ -465,11 +465,20 @@ const char *spg_noalloc_last_error(void);
  * shells k = 0 .. n/2, the shell of frequency index (h, k, l) being the
  * nearest integer to sqrt(h^2 + k^2 + l^2). counts (optional) receives the
  * number of coefficients per shell. fsc and counts are host arrays of at least
- * n/2 + 1 entries (max_shells). Uses cuFFT and allocates its own temporaries;
+ * n/2 + 1 entries (max_shells). Uses cuFFT (up to four plans, without work
+ * areas, are kept between calls) and allocates its own temporaries;
  * synchronises `stream`. Errors: SPG_EINVAL, SPG_ENOMEM, SPG_ECUDA with a
- * message in spg_fsc_last_error(). */
+ * message in spg_fsc_last_error().
+ *
+ * spg_fsc_ws takes the temporaries from the caller: a 256-byte aligned device
+ * buffer of at least the bytes spg_fsc_workspace gives for these maps (those
+ * already on the current device need no room for a copy), free for other use
+ * once the call returns; a null or too small workspace is allocated instead. */
 spg_status spg_fsc(int n, const float *a, const float *b, int max_shells, double *fsc, double *counts,
                    void *stream);
+spg_status spg_fsc_ws(int n, const float *a, const float *b, int max_shells, double *fsc, double *counts,
+                      void *workspace, size_t workspace_bytes, void *stream);
+spg_status spg_fsc_workspace(int n, const float *a, const float *b, size_t *bytes);
 const char *spg_fsc_last_error(void);
 
 /* Message for the last failing call on ctx (or a global message if ctx is

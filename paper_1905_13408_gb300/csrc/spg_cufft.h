@@ -9,7 +9,10 @@
 namespace spg {
 
 struct CufftApi {
-    cufftResult (*plan3d)(cufftHandle *, int, int, int, cufftType) = nullptr;
+    cufftResult (*create)(cufftHandle *) = nullptr;
+    cufftResult (*set_auto_allocation)(cufftHandle, int) = nullptr;
+    cufftResult (*make_plan3d)(cufftHandle, int, int, int, cufftType, size_t *) = nullptr;
+    cufftResult (*set_work_area)(cufftHandle, void *) = nullptr;
     cufftResult (*plan_many)(cufftHandle *, int, int *, int *, int, int, int *, int, int, cufftType,
                              int) = nullptr;
     cufftResult (*set_stream)(cufftHandle, cudaStream_t) = nullptr;

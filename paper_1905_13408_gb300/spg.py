@@ -39,7 +39,7 @@ EXPORTS = ["spg_create", "spg_create_batch", "spg_set_data", "spg_set_x", "spg_g
            "spg_get_state", "spg_set_state", "spg_backward", "spg_unrolled", "spg_probe_timeout",
            "spg_autotune", "spg_launch_count", "spg_plan_info", "spg_last_error", "spg_destroy",
            "spg_objective_noalloc", "spg_noalloc_last_error", "spg_set_anchor", "spg_param_scales",
-           "spg_fsc", "spg_fsc_last_error", "spg_set_data_fourier", "spg_backproject",
+           "spg_fsc", "spg_fsc_ws", "spg_fsc_workspace", "spg_fsc_last_error", "spg_set_data_fourier", "spg_backproject",
            "spg_backproject_last_error", "spg_grid_create", "spg_grid_add", "spg_grid_finish", "spg_grid_reset",
            "spg_grid_count", "spg_grid_last_error", "spg_grid_destroy", "spg_set_halo", "spg_step_bound",
            "spg_set_step_bound", "spg_get_planes", "spg_set_planes", "spg_set_lambdas"]
@@ -125,6 +125,8 @@ def load():
             "spg_noalloc_last_error": (ctypes.c_char_p, []),
             "spg_set_anchor": (I, [P, I, ctypes.c_float, V]),
             "spg_fsc": (I, [I, V, V, I, ctypes.POINTER(D), ctypes.POINTER(D), P]),
+            "spg_fsc_ws": (I, [I, V, V, I, ctypes.POINTER(D), ctypes.POINTER(D), V, ctypes.c_size_t, P]),
+            "spg_fsc_workspace": (I, [I, V, V, ctypes.POINTER(ctypes.c_size_t)]),
             "spg_fsc_last_error": (ctypes.c_char_p, []),
             "spg_set_data_fourier": (I, [P, I, V, V]),
             "spg_backproject": (I, [I, I, V, V, V, V, I, ctypes.c_float, V, V, P]),
@@ -214,6 +216,25 @@ def spg_param_scales(h, vol=0):
     return dict(zip(["rms_wb", "mean_w", "max_w", "min_w"], out[:]))
 
 
+def _workspace(nbytes, stream):
+    """A device buffer of nbytes from torch's caching allocator, taken on the
+    stream that will use it (so it cannot be one that work pending on another
+    stream still uses); None without torch or without room (the library then
+    allocates, and reports it, itself)."""
+    try:
+        import torch
+    except ImportError:  # pragma: no cover
+        return None
+    try:
+        if int(stream or 0) == torch.cuda.current_stream().cuda_stream:
+            return torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        on = torch.cuda.ExternalStream(int(stream)) if stream else torch.cuda.default_stream()
+        with torch.cuda.stream(on):
+            return torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    except torch.cuda.OutOfMemoryError:
+        return None
+
+
 def spg_fsc(a, b, stream=None):
     """(fsc, counts) for shells 0 .. n/2 of two n^3 float32 maps (Eq. 30)."""
     n = int(a.shape[0])
@@ -222,10 +243,17 @@ def spg_fsc(a, b, stream=None):
     m = n // 2 + 1
     fsc = np.zeros(m)
     cnt = np.zeros(m)
-    st = load().spg_fsc(n, pa, pb, m, fsc.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
-                        cnt.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), ctypes.c_void_p(stream or 0))
+    lib = load()
+    need = ctypes.c_size_t()
+    st = lib.spg_fsc_workspace(n, pa, pb, ctypes.byref(need))
+    if st == SPG_OK:
+        ws = _workspace(need.value, stream)
+        st = lib.spg_fsc_ws(n, pa, pb, m, fsc.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+                            cnt.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+                            ctypes.c_void_p(ws.data_ptr() if ws is not None else 0),
+                            need.value if ws is not None else 0, ctypes.c_void_p(stream or 0))
     if st != SPG_OK:
-        raise SPGError(st, load().spg_fsc_last_error().decode())
+        raise SPGError(st, lib.spg_fsc_last_error().decode())
     return fsc, cnt
 
 
