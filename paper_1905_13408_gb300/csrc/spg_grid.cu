@@ -15,9 +15,9 @@
 // or, mirrored, at -n, whichever lies in the stored half spectrum
 // [n][n][n/2+1] (both on the planes kx = 0 and kx = n/2). This halves both
 // the atomics and the accumulator against a full-spectrum scatter and gives
-// the same sums. A CTA takes an 8 x 8 tile of one image's coefficients,
-// sums their FP32 deposits in a shared-memory box and adds each touched
-// point once, with FP64 atomics, into an interleaved accumulator
+// the same sums. A warp takes an 8 x 8 tile of one image's coefficients,
+// sums their FP32 deposits in a shared-memory box of its own and adds each
+// touched point once, with FP64 atomics, into an interleaved accumulator
 // (Re num, Im num, N, unused: one 32-byte sector per grid point). A finishing
 // pass writes the Eq. 31 data term: N' = V N and
 // y = (-1)^(kx+ky+kz) num / sqrt(N), the sign moving the
@@ -30,6 +30,7 @@
 #include <string>
 
 #include "spg.h"
+#include "spg_ff.cuh"
 #include "spg_trace.h"
 
 namespace {
@@ -66,176 +67,327 @@ __device__ __forceinline__ void deposit(double *acc, int n, int x, int y, int z,
 }
 
 // One image coefficient's contribution: the first grid point of its support
-// on each axis and the per-axis kernel factors (the kernel factorises over
-// the axes: a product of 1-D Gaussians, or of 1-D hat functions); the
-// factors and the deposits are FP32 (the FP64 pipe is narrow), positions and
-// the nearest-point / floor decisions FP64 so they match a double-precision
-// reference.
+// on each axis, its position relative to that support, and the values it
+// spreads.
 struct Sample {
     int bx, by, bz;
-    float wx[3], wy[3], wz[3];
+    float fx, fy, fz;  // position minus the support's centre (kernel 0) or first point (kernel 1)
     float vre, vim, vcc;
 };
 
-__device__ __forceinline__ void make_sample(int n, const float *__restrict__ rot, const float2 *__restrict__ X,
-                                            const float *__restrict__ ctf, const float *__restrict__ pw, int kernel,
-                                            float h, int img, int kx, int ky, Sample &S)
+// p = r0 kx + r1 ky on one axis: the nearest point (half to even, kernel 0) or
+// floor (kernel 1) b and the remainder f, as exact arithmetic on the float32
+// entries gives them. The products are exact pairs (fused multiply-add), their
+// leading parts are added exactly and the sum is normalised (the tails can
+// exceed an ulp of the sum where the products cancel), so p = s + lo with |lo|
+// at most half an ulp of s and an error far below any half-way case of
+// float32 rotations; doubles gave the same decisions at 9 FP64 operations a coefficient and
+// half a dozen conversions, more than a millisecond of GB300's FP64 pipe for
+// 2048 images of 256^2.
+__device__ __forceinline__ void split_axis(float r0, float r1, int kx, int ky, int kernel, int &b, float &f)
 {
-    const float *R = rot + (long long)img * 9;  // row-major 3x3; columns 0 and 1 span the image plane
-    const double px = __dadd_rn(__dmul_rn(R[0], kx), __dmul_rn(R[1], ky));
-    const double py = __dadd_rn(__dmul_rn(R[3], kx), __dmul_rn(R[4], ky));
-    const double pz = __dadd_rn(__dmul_rn(R[6], kx), __dmul_rn(R[7], ky));
-    const long long src = (long long)img * n * n + (long long)ky * n + wrap(kx, n);
-    const float2 x = X[src];
-    const float c = ctf[src];
-    const float pc = pw ? pw[img] * c : c;
-    S.vre = pc * x.x;
-    S.vim = pc * x.y;
-    S.vcc = pc * c;
+    const float x = (float)kx, y = (float)ky;
+    const float p = __fmul_rn(r0, x), q = __fmul_rn(r1, y);
+    const spg::ff::FF u = spg::ff::two_sum(p, q);
+    const spg::ff::FF v =
+        spg::ff::two_sum(u.hi, __fadd_rn(u.lo, __fadd_rn(__fmaf_rn(r0, x, -p), __fmaf_rn(r1, y, -q))));
+    const float s = v.hi, lo = v.lo;
     if (kernel == 0) {
-        S.bx = __double2int_rn(px);
-        S.by = __double2int_rn(py);
-        S.bz = __double2int_rn(pz);
-        const float fx = (float)(px - S.bx), fy = (float)(py - S.by), fz = (float)(pz - S.bz);
-        const float ih = 1.0f / h;
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-            const float ex = fx - (d - 1), ey = fy - (d - 1), ez = fz - (d - 1);
-            S.wx[d] = expf(-ex * ex * ih);
-            S.wy[d] = expf(-ey * ey * ih);
-            S.wz[d] = expf(-ez * ez * ih);
-        }
-        S.bx -= 1;
-        S.by -= 1;
-        S.bz -= 1;
+        float c = rintf(s);
+        const float r = __fsub_rn(s, c);
+        // the rounding of s decides unless lo carries p across the half-way point
+        if (__fadd_rn(__fsub_rn(r, 0.5f), lo) > 0.f) c += 1.f;
+        else if (__fadd_rn(__fadd_rn(r, 0.5f), lo) < 0.f) c -= 1.f;
+        b = (int)c;
+        f = __fadd_rn(__fsub_rn(s, c), lo);
     } else {
-        const double flx = floor(px), fly = floor(py), flz = floor(pz);
-        S.bx = (int)flx;
-        S.by = (int)fly;
-        S.bz = (int)flz;
-        const float fx = (float)(px - flx), fy = (float)(py - fly), fz = (float)(pz - flz);
-        S.wx[0] = 1.f - fx;
-        S.wx[1] = fx;
-        S.wy[0] = 1.f - fy;
-        S.wy[1] = fy;
-        S.wz[0] = 1.f - fz;
-        S.wz[1] = fz;
-        S.wx[2] = S.wy[2] = S.wz[2] = 0.f;
+        float c = floorf(s);
+        if (__fsub_rn(s, c) == 0.f && lo < 0.f) c -= 1.f;
+        b = (int)c;
+        f = __fadd_rn(__fsub_rn(s, c), lo);
     }
 }
 
-// All deposits of one sample straight into the FP64 accumulator.
-__device__ __forceinline__ void deposit_sample(double *acc, int n, int span, const Sample &S, bool self_mate)
+__device__ __forceinline__ void make_sample(int n, const float *__restrict__ R, const float2 *__restrict__ X,
+                                            const float *__restrict__ ctf, float pw, int kernel, int kx, int ky,
+                                            Sample &S)
 {
+    const int src = ky * n + (kx < 0 ? kx + n : kx);
+    const float2 x = __ldcs(X + src);
+    const float c = __ldcs(ctf + src);
+    const float pc = pw * c;
+    S.vre = pc * x.x;
+    S.vim = pc * x.y;
+    S.vcc = pc * c;
+    // row-major 3x3; columns 0 and 1 span the image plane
+    split_axis(R[0], R[1], kx, ky, kernel, S.bx, S.fx);
+    split_axis(R[3], R[4], kx, ky, kernel, S.by, S.fy);
+    split_axis(R[6], R[7], kx, ky, kernel, S.bz, S.fz);
+    if (kernel == 0) {
+        S.bx -= 1;
+        S.by -= 1;
+        S.bz -= 1;
+    }
+}
+
+// Kernel weights of one axis: the kernel factorises over the axes, a product
+// of 1-D Gaussians exp(-e^2/h) (3 points) or of 1-D hat functions (2 points).
+__device__ __forceinline__ void axis_weights(int kernel, float ih, float f, float (&w)[3])
+{
+    if (kernel == 0) {
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            const float e = f - (d - 1);
+            w[d] = expf(-e * e * ih);
+        }
+    } else {
+        w[0] = 1.f - f;
+        w[1] = f;
+        w[2] = 0.f;
+    }
+}
+
+// All deposits of one sample straight into the FP64 accumulator (rare: kept
+// out of line).
+__device__ __noinline__ void deposit_sample(double *acc, int n, int kernel, float ih, Sample S, bool self_mate)
+{
+    const int span = kernel == 0 ? 3 : 2;
+    float wx[3], wy[3], wz[3];
+    axis_weights(kernel, ih, S.fx, wx);
+    axis_weights(kernel, ih, S.fy, wy);
+    axis_weights(kernel, ih, S.fz, wz);
     for (int dz = 0; dz < span; dz++)
         for (int dy = 0; dy < span; dy++) {
-            const float kyz = S.wy[dy] * S.wz[dz];
+            const float kyz = wy[dy] * wz[dz];
             for (int dx = 0; dx < span; dx++) {
-                const float K = S.wx[dx] * kyz;
+                const float K = wx[dx] * kyz;
                 deposit(acc, n, S.bx + dx, S.by + dy, S.bz + dz, (double)(K * S.vre), (double)(K * S.vim),
                         (double)(K * S.vcc), self_mate);
             }
         }
 }
 
-// One CTA grids an 8 x 8 tile of one image's half spectrum (kx in tile
-// columns, ky >= 0): the tile's deposits are first summed in FP32 in a
-// shared-memory box covering the support of all its samples, then each
-// touched box point goes to the FP64 accumulator once (with its mirror
-// point, as deposit() does). Neighbouring coefficients share most of their
-// support points, so this issues several times fewer global atomics than
-// depositing every sample directly. A tile whose box does not fit, and the
-// coefficient k = 0 (its own mate), deposit directly.
-constexpr int kTile = 8;
-constexpr int kBoxCap = 1536;  // box points (3 floats each: 18 KB)
-
-__global__ void __launch_bounds__(kTile * kTile) scatter_tile_kernel(int n, int m, const float *__restrict__ rot,
-                                                                     const float2 *__restrict__ X,
-                                                                     const float *__restrict__ ctf,
-                                                                     const float *__restrict__ pw, int kernel,
-                                                                     float h, double *acc)
+// The double that equals v, by integer operations for ordinary values (the
+// conversion runs on the FP64 pipe, 16 cycles a warp).
+__device__ __forceinline__ double widen(float v)
 {
-    extern __shared__ float box[];  // [kBoxCap][3]
-    __shared__ int red[kTile * kTile / 32][6];
-    __shared__ int geo[7];  // lo x, y, z; dims x, y, z; use box
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const float a = fabsf(v);
+    if (!(a >= 1.17549435e-38f && a <= 3.4028235e38f)) return (double)v;  // zero, denormal, infinite, NaN
+    const int u = __float_as_int(v);
+    return __hiloint2double(((u >> 3) & (int)0x8fffffff) + 0x38000000, u << 29);
+}
+
+// Bound: a coefficient's 27 deposits are a read-modify-write of 27 points in
+// shared memory (float4: re, im, N, unused) and its share of the tile's points
+// goes to L2 as FP64 atomics; reading the images takes 0.1 of 12 ms at 2048
+// images of 256^2 into 256^3.
+//
+// One warp per tile of 8 x 4 coefficients, in its own box: the lanes are the
+// support points of one sample at a time (27 or 8), so no two lanes meet and
+// the box needs no atomics (float32 atomics in shared memory are
+// compare-and-swap loops; they were what a form with a thread per sample waited
+// for). The samples' weights and values pass through shared memory, one row of
+// 32 samples each, so a lane fetches those of 4 samples at a time. The box's row
+// and plane strides are padded where that still fits (rows to 3 .. 5 modulo 8
+// points, planes to 1): the rows of a support then fall on different bank
+// groups. A tile whose box
+// exceeds the capacity is done in halves; what still does not fit (matrices
+// that are no rotations), and the coefficient k = 0 (its own mate), deposits
+// directly. In the flush the lanes are 10 points of a row by 3 values, so an
+// atomic instruction covers a run of whole 32-byte sectors. Tiles go out tile
+// by tile over all images, not image by image: the tiles of one |k| touch a
+// spherical shell of the accumulator (32 MB at the rim of 256^3), which stays
+// in L2.
+//
+// Measured, add and finish, against the thread-per-sample form (8 x 8 tiles,
+// float32 atomics in the box): 2048 images of 256^2 12.4 -> 7.4 ms (trilinear
+// 7.8 -> 5.6), 128 images 1.08 -> 0.73, 2048 of 128^2 3.20 -> 1.96, 4096 of 64^2
+// 1.64 -> 1.12, 512 of 288^2 4.24 -> 2.65. What bounds it now, at 256^2: shared
+// memory (800 wavefronts a tile, 64 % of its rate) and issue (2900 instructions
+// a tile, 53 %) with the 16 warps an SM's shared memory holds.
+constexpr int kTileX = 8, kTileY = 4;
+constexpr int kBoxCap = 768;   // box points per warp (12 KB)
+constexpr int kWarps = 8;      // per CTA; two CTAs per SM
+constexpr int kStageRow = 36;  // floats; rows 4 banks apart
+constexpr int kWarpSmem = kBoxCap * 16 + 13 * kStageRow * 4;
+
+__global__ void __launch_bounds__(kWarps * 32, 2)
+    scatter_tile_kernel(int n, int m, const float *__restrict__ rot, const float2 *__restrict__ X,
+                        const float *__restrict__ ctf, const float *__restrict__ pw, int kernel, float h, double *acc)
+{
+    extern __shared__ __align__(16) unsigned char gsm[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float4 *const box = reinterpret_cast<float4 *>(gsm + (size_t)warp * kWarpSmem);
+    // rows of 32 samples: wx[3], wy[3], wz[3], re, im, N, box offset
+    float *const stage = reinterpret_cast<float *>(box + kBoxCap);
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q = lane; q < kBoxCap; q += 32) box[q] = zero4;
     const int span = kernel == 0 ? 3 : 2;
-    const int ntx = (n + kTile - 1) / kTile, nty = (n / 2 + kTile - 1) / kTile;
-    const long long ntiles = (long long)m * nty * ntx;
+    const float ih = 1.0f / h;
+    const int dx = lane % span, dy = (lane / span) % span, dz = lane / (span * span);
+    const bool point = lane < span * span * span;
+    const int nh = n / 2 + 1;
+    const int ntx = (n + kTileX - 1) / kTileX, nty = (n / 2 + kTileY - 1) / kTileY;
     const float rmax2 = (n * 0.5f - 2.0f) * (n * 0.5f - 2.0f);
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int img = (int)(t / ((long long)nty * ntx));
-        const int rem = (int)(t % ((long long)nty * ntx));
-        const int kx = -n / 2 + (rem % ntx) * kTile + tid % kTile;
-        const int ky = (rem / ntx) * kTile + tid / kTile;
-        const bool ok = kx < n / 2 && ky < n / 2 && (ky > 0 || kx >= 0) && (float)(kx * kx + ky * ky) <= rmax2;
-        const bool self_mate = kx == 0 && ky == 0;
-        Sample S;
-        if (ok) make_sample(n, rot, X, ctf, pw, kernel, h, img, kx, ky, S);
-        // bounding box of the tile's supports (the self-mate sample goes direct)
-        const bool inbox = ok && !self_mate;
-        int v[6] = {inbox ? S.bx : INT_MAX, inbox ? S.by : INT_MAX, inbox ? S.bz : INT_MAX,
-                    inbox ? S.bx : INT_MIN, inbox ? S.by : INT_MIN, inbox ? S.bz : INT_MIN};
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int c = 0; c < 6; c++) {
-                const int u = __shfl_down_sync(0xffffffffu, v[c], o);
-                v[c] = c < 3 ? min(v[c], u) : max(v[c], u);
-            }
-        if (lane == 0)
-#pragma unroll
-            for (int c = 0; c < 6; c++) red[warp][c] = v[c];
-        __syncthreads();
-        if (tid == 0) {
-            int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
-            for (int w = 0; w < kTile * kTile / 32; w++)
-                for (int c = 0; c < 3; c++) {
-                    lo[c] = min(lo[c], red[w][c]);
-                    hi[c] = max(hi[c], red[w][3 + c]);
-                }
-            long long vol = 0;
-            if (lo[0] != INT_MAX) {
-                vol = 1;
-                for (int c = 0; c < 3; c++) {
-                    geo[c] = lo[c];
-                    geo[3 + c] = hi[c] - lo[c] + span;
-                    vol *= geo[3 + c];
-                }
-            }
-            geo[6] = (vol > 0 && vol <= kBoxCap) ? (int)vol : 0;
+    const int fpx = lane / 3, fcomp = lane - 3 * fpx;  // flush: point of the row and value
+    const unsigned conj = fcomp == 1 ? 0x80000000u : 0u;
+    const long long ys = 4LL * nh, zs = ys * n;        // accumulator strides, doubles
+    // work item (tile, image), the image counting faster, advanced by the number
+    // of warps without a division per item
+    const long long t0 = (long long)blockIdx.x * kWarps + warp, nwarps = (long long)gridDim.x * kWarps;
+    const int dtile = (int)(nwarps / m), dimg = (int)(nwarps % m);
+    int tile = (int)(t0 / m), img = (int)(t0 % m);
+    const int ntiles = nty * ntx;
+    auto next = [&]() {
+        tile += dtile;
+        img += dimg;
+        if (img >= m) {
+            img -= m;
+            tile++;
         }
-        __syncthreads();
-        const int vol = geo[6];
-        if (vol > 0) {
-            for (int q = tid; q < 3 * vol; q += blockDim.x) box[q] = 0.f;
-            __syncthreads();
-            if (inbox) {
-                const int dx0 = S.bx - geo[0], dy0 = S.by - geo[1], dz0 = S.bz - geo[2];
-                for (int dz = 0; dz < span; dz++)
-                    for (int dy = 0; dy < span; dy++) {
-                        const float kyz = S.wy[dy] * S.wz[dz];
-                        float *row = box + 3 * (((dz0 + dz) * geo[4] + (dy0 + dy)) * geo[3] + dx0);
-                        for (int dx = 0; dx < span; dx++) {
-                            const float K = S.wx[dx] * kyz;
-                            atomicAdd(row + 3 * dx + 0, K * S.vre);
-                            atomicAdd(row + 3 * dx + 1, K * S.vim);
-                            atomicAdd(row + 3 * dx + 2, K * S.vcc);
+    };
+    for (; tile < ntiles; next()) {
+        const int kx0 = -n / 2 + (tile % ntx) * kTileX, ky0 = (tile / ntx) * kTileY;
+        {
+            // the tile's nearest coefficient to the origin lies outside the disc
+            const int nx = kx0 > 0 ? kx0 : (kx0 + kTileX - 1 < 0 ? kx0 + kTileX - 1 : 0);
+            if ((float)(nx * nx + ky0 * ky0) > rmax2) continue;
+        }
+        const long long img2 = (long long)img * n * n;
+        const int kx = kx0 + lane % kTileX, ky = ky0 + lane / kTileX;
+        const bool ok = kx < n / 2 && ky < n / 2 && (ky > 0 || kx >= 0) && (float)(kx * kx + ky * ky) <= rmax2;
+        Sample S;
+        if (ok)
+            make_sample(n, rot + (long long)img * 9, X + img2, ctf + img2, pw ? pw[img] : 1.f, kernel, kx, ky, S);
+        const bool self = kx == 0 && ky == 0;
+        if (ok && self) deposit_sample(acc, n, kernel, ih, S, true);
+        unsigned todo = __ballot_sync(0xffffffffu, ok && !self);
+        unsigned now = todo;  // samples of this pass: all that are left, or a half of the tile
+        while (todo) {
+            const bool mine = (now >> lane & 1u) != 0;
+            const int lx = __reduce_min_sync(0xffffffffu, mine ? S.bx : INT_MAX);
+            const int ly = __reduce_min_sync(0xffffffffu, mine ? S.by : INT_MAX);
+            const int lz = __reduce_min_sync(0xffffffffu, mine ? S.bz : INT_MAX);
+            const int ux = __reduce_max_sync(0xffffffffu, mine ? S.bx : INT_MIN);
+            const int uy = __reduce_max_sync(0xffffffffu, mine ? S.by : INT_MIN);
+            const int uz = __reduce_max_sync(0xffffffffu, mine ? S.bz : INT_MIN);
+            const long long ex = (long long)ux - lx + span, ey = (long long)uy - ly + span, ez = (long long)uz - lz + span;
+            // compared one factor at a time: the extents of non-rotations are unbounded
+            const bool fits = ex <= kBoxCap && ey <= kBoxCap && ez <= kBoxCap && ex * ey * ez <= kBoxCap;
+            if (!fits) {
+                const unsigned half = now & 0xffffu;
+                if (half && half != now) {
+                    now = half;
+                    continue;
+                }
+                if (mine) deposit_sample(acc, n, kernel, ih, S, false);
+                todo &= ~now;
+                now = todo;
+                continue;
+            }
+            const int EX = (int)ex, EY = (int)ey, EZ = (int)ez;
+            const int r8 = EX & 7;
+            int DX = EX + (r8 < 3 ? 3 - r8 : (r8 > 5 ? 11 - r8 : 0));
+            if (DX * EY * EZ > kBoxCap) DX = EX;
+            int DXY = DX * EY + ((1 - DX * EY) & 7);
+            if (DXY * EZ > kBoxCap) DXY = DX * EY;
+            const int vol = DXY * EZ;
+            {
+                // a lane without a sample in this pass stages a deposit of nothing
+                float wx[3], wy[3], wz[3];
+                axis_weights(kernel, ih, mine ? S.fx : 0.f, wx);
+                axis_weights(kernel, ih, mine ? S.fy : 0.f, wy);
+                axis_weights(kernel, ih, mine ? S.fz : 0.f, wz);
+                const int off = mine ? (S.bz - lz) * DXY + (S.by - ly) * DX + (S.bx - lx) : 0;
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    stage[d * kStageRow + lane] = wx[d];
+                    stage[(3 + d) * kStageRow + lane] = wy[d];
+                    stage[(6 + d) * kStageRow + lane] = wz[d];
+                }
+                stage[9 * kStageRow + lane] = mine ? S.vre : 0.f;
+                stage[10 * kStageRow + lane] = mine ? S.vim : 0.f;
+                stage[11 * kStageRow + lane] = mine ? S.vcc : 0.f;
+                stage[12 * kStageRow + lane] = __int_as_float(off);
+            }
+            __syncwarp();
+            // deposits: one sample at a time, a lane per support point
+            float4 *const mybox = box + (point ? dz * DXY + dy * DX + dx : 0);
+            const float *const swx = stage + (point ? dx : 0) * kStageRow;
+            const float *const swy = stage + (3 + dy) * kStageRow;
+            const float *const swz = stage + (6 + (point ? dz : 0)) * kStageRow;
+#pragma unroll 1
+            for (int j = 0; j < 32; j += 4) {
+                if (!(now >> j & 15u)) continue;
+                auto row4 = [&](const float *r) { return *reinterpret_cast<const float4 *>(r + j); };
+                const float4 ax = row4(swx), ay = row4(swy), az = row4(swz), of = row4(stage + 12 * kStageRow);
+                const float4 re = row4(stage + 9 * kStageRow), im = row4(stage + 10 * kStageRow);
+                const float4 cc = row4(stage + 11 * kStageRow);
+                auto add = [&](float x, float y, float z, float o, float r, float i, float c) {
+                    const float K = x * (y * z);
+                    if (point) {
+                        float4 *const p = mybox + __float_as_int(o);
+                        float4 v = *p;
+                        v.x += K * r;
+                        v.y += K * i;
+                        v.z += K * c;
+                        *p = v;
+                    }
+                    __syncwarp();
+                };
+                add(ax.x, ay.x, az.x, of.x, re.x, im.x, cc.x);
+                add(ax.y, ay.y, az.y, of.y, re.y, im.y, cc.y);
+                add(ax.z, ay.z, az.z, of.z, re.z, im.z, cc.z);
+                add(ax.w, ay.w, az.w, of.w, re.w, im.w, cc.w);
+            }
+            // flush: row by row, 10 points by 3 values. Point x goes to the
+            // stored half where x (modulo n) <= n/2, its mirror -x, conjugated,
+            // where that does; on the planes 0 and n/2 both do.
+            const int wx0 = wrap(lx, n), wy0 = wrap(ly, n), wz0 = wrap(lz, n);
+            // boxes that cross no plane where an index wraps or changes sides
+            // (four of five): one direction, rows and planes at fixed strides
+            const bool fwd = wx0 > 0 && wx0 + EX <= nh - 1, back = wx0 >= nh && wx0 + EX <= n;
+            if ((fwd || back) && wy0 > 0 && wy0 + EY <= n && wz0 > 0 && wz0 + EZ <= n) {
+                const long long sy = fwd ? ys : -ys, sz = (fwd ? zs : -zs) - (long long)EY * sy;
+                const unsigned flip = fwd ? 0u : conj;
+                for (int x0 = 0; x0 < EX; x0 += 10) {
+                    const int px = x0 + fpx;
+                    const bool on = lane < 30 && px < EX;
+                    double *to = acc + (fwd ? 4LL * (wx0 + px) + fcomp + zs * wz0 + ys * wy0
+                                            : 4LL * (n - wx0 - px) + fcomp + zs * (n - wz0) + ys * (n - wy0));
+                    const float *src = reinterpret_cast<const float *>(box + (on ? px : 0)) + fcomp;
+                    for (int z = 0; z < EZ; z++, to += sz, src += 4 * (DXY - EY * DX)) {
+                        int y = 0;
+                        for (; y + 4 <= EY; y += 4, src += 16 * DX) {
+                            float v[4];
+#pragma unroll
+                            for (int c = 0; c < 4; c++) v[c] = on ? src[4 * c * DX] : 0.f;
+#pragma unroll
+                            for (int c = 0; c < 4; c++, to += sy)
+                                if (v[c] != 0.f) atomicAdd(to, widen(__uint_as_float(__float_as_uint(v[c]) ^ flip)));
+                        }
+                        for (; y < EY; y++, src += 4 * DX, to += sy) {
+                            const float v = on ? *src : 0.f;
+                            if (v != 0.f) atomicAdd(to, widen(__uint_as_float(__float_as_uint(v) ^ flip)));
                         }
                     }
+                }
+            } else {
+                // a lane per box point, every index wrapped on its own
+                const int EXY = EX * EY;
+                for (int q = lane; q < EXY * EZ; q += 32) {
+                    const int z = q / EXY, r = q - z * EXY, y = r / EX, x = r - y * EX;
+                    const float4 v = box[z * DXY + y * DX + x];
+                    if (v.x == 0.f && v.y == 0.f && v.z == 0.f) continue;
+                    deposit(acc, n, lx + x, ly + y, lz + z, widen(v.x), widen(v.y), widen(v.z), false);
+                }
             }
-            __syncthreads();
-            for (int q = tid; q < vol; q += blockDim.x) {
-                const float re = box[3 * q], im = box[3 * q + 1], w = box[3 * q + 2];
-                if (re == 0.f && im == 0.f && w == 0.f) continue;
-                const int gx = geo[0] + q % geo[3], gy = geo[1] + (q / geo[3]) % geo[4], gz = geo[2] + q / (geo[3] * geo[4]);
-                deposit(acc, n, gx, gy, gz, (double)re, (double)im, (double)w, false);
-            }
-        } else if (inbox) {
-            deposit_sample(acc, n, span, S, false);
+            __syncwarp();
+            for (int q = lane; q < vol; q += 32) box[q] = zero4;
+            __syncwarp();  // the box and the stage are reused
+            todo &= ~now;
+            now = todo;
         }
-        if (ok && self_mate) deposit_sample(acc, n, span, S, true);
-        __syncthreads();  // the box and geo are reused by the next tile
     }
 }
 
@@ -254,7 +406,17 @@ __global__ void finish_kernel(int n, const double *__restrict__ acc, float2 *y_h
         const double sgn = ((kx + ky + kz) & 1) ? -1.0 : 1.0;
         float2 y = make_float2(0.f, 0.f);
         if (w > 0) {
-            const double s = sgn / sqrt(w);
+            // 1/sqrt(w) to 44 bits: a float32 estimate and one Newton step in
+            // double (the results are float32; double sqrt and division kept
+            // the narrow FP64 pipe busy for 30 operations a point)
+            const float wf = (float)w;
+            double s;
+            if (wf > 1e-37f && wf < 1e38f) {
+                const double r = (double)rsqrtf(wf);
+                s = sgn * fma(0.5 * r, fma(-w * r, r, 1.0), r);
+            } else {
+                s = sgn / sqrt(w);
+            }
             y = make_float2((float)(a[0] * s), (float)(a[1] * s));
         }
         y_half[q] = y;
@@ -387,16 +549,17 @@ extern "C" spg_status spg_grid_add(spg_grid *g, int m, const float *rot, const v
         a.dev = dst;
         off += align256(a.bytes);
     }
-    // the tile kernel's shared box exceeds the default 48 KB (set per call: per device)
-    e = cudaFuncSetAttribute(scatter_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kBoxCap * 3 * (int)sizeof(float));
+    // the warps' boxes exceed the default 48 KB (set per call: per device)
+    constexpr int smem = kWarps * kWarpSmem;
+    e = cudaFuncSetAttribute(scatter_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return cuda_fail(g, e, "spg_grid_add: configure");
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const long long tiles = (long long)m * ((n / 2 + kTile - 1) / kTile) * ((n + kTile - 1) / kTile);
-    const int grid = (int)std::min<long long>(tiles, (long long)std::max(nsm, 1) * 12 * 4);
-    scatter_tile_kernel<<<grid, kTile * kTile, kBoxCap * 3 * sizeof(float), g->stream>>>(
+    const long long tiles =
+        (long long)m * ((n / 2 + kTileY - 1) / kTileY) * ((n + kTileX - 1) / kTileX);
+    const int grid = (int)std::min<long long>((tiles + kWarps - 1) / kWarps, (long long)std::max(nsm, 1) * 2);
+    scatter_tile_kernel<<<grid, kWarps * 32, smem, g->stream>>>(
         n, m, static_cast<const float *>(in[0].dev), static_cast<const float2 *>(in[1].dev),
         static_cast<const float *>(in[2].dev), static_cast<const float *>(in[3].dev), g->kernel, g->h, g->acc);
     e = cudaGetLastError();
