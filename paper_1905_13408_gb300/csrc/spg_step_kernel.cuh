@@ -611,10 +611,12 @@ __device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pi
                 const float cxu = XK[(cr - 1) * XW + cc], cmu = XM[(cr - 1) * XW + cc];
                 const float cd = XD ? cm : cx - cm;
                 const int hx = W.x0 + TX, hy = W.y0 + lane;
-                const float ax = (cx - cxl) + beta * (cd - (XD ? cml : cxl - cml));
-                const float ay = hy >= 1 ? (cx - cxu) + beta * (cd - (XD ? cmu : cxu - cmu)) : 0.f;
-                const float az = z >= 1 ? (cx - cxz) + beta * (cd - cdz) : 0.f;
-                const float s2 = ax * ax + ay * ay + az * az;
+                // the operations of phase_a, so that a voxel's result does not depend
+                // on where the tiles' borders lie
+                const float ax = fmaf(beta, cd - (XD ? cml : cxl - cml), cx - cxl);
+                const float ay = hy >= 1 ? fmaf(beta, cd - (XD ? cmu : cxu - cmu), cx - cxu) : 0.f;
+                const float az = z >= 1 ? fmaf(beta, cd - cdz, cx - cxz) : 0.f;
+                const float s2 = fmaf(ax, ax, fmaf(ay, ay, az * az));
                 const bool in = hx < V.nx && hy < V.ny && z < V.nz;
                 const float sc = in ? OM[lane * OW + TX] * fminf(inv_mu, rsqrtf(s2)) : 0.f;
                 sh.hx_ring[slot * 32 + lane] = ax * sc;
