@@ -33,7 +33,7 @@ constexpr int kGraphLen = 10;                   // iterations per captured graph
 // (32 bytes per work item and iteration) and roughly how long it may hold the
 // GPU (work queued on other streams starts between launches). At 10 ms the
 // launch boundary, about 5 us, no longer shows.
-constexpr size_t kPartialBytes = 8u << 20;
+constexpr size_t kPartialBytes = 1u << 20;
 constexpr double kLaunchSeconds = 10e-3;
 constexpr uint64_t kStateMagic = 0x5350475354415445ull;  // "SPGSTATE"
 
@@ -90,6 +90,8 @@ struct spg_ctx {
     double *partials_d = nullptr;
     double *hist_d = nullptr;
     double *plane_part_d = nullptr;
+    WorkItem *aux_items_d = nullptr;  // march items of the auxiliary passes
+    int naux = 0;
     double *vol_out_d = nullptr;
     double *maxw_d = nullptr;
     double *rstats_d = nullptr;
@@ -206,7 +208,7 @@ void free_all(spg_ctx *c)
     for (void *p : fs)
         if (p) cudaFree(p);
     void *ps[] = {c->vols_d, c->items_d, c->sched_d, c->tmaps_d, c->plane_vol_d, c->X[0], c->X[1], c->X[2], c->X[3], c->B, c->W,
-                  c->OM1, c->OMTV, c->beta_d, c->st_d, c->partials_d, c->hist_d, c->plane_part_d,
+                  c->OM1, c->OMTV, c->beta_d, c->st_d, c->partials_d, c->hist_d, c->plane_part_d, c->aux_items_d,
                   c->vol_out_d, c->maxw_d, c->rstats_d};
     for (void *p : ps)
         if (p) cudaFree(p);
@@ -584,6 +586,8 @@ AuxParams aux_params(const spg_ctx *c)
     a.nplanes = c->nplanes;
     a.nvol = c->nvol;
     a.st = c->st_d;
+    a.items = c->aux_items_d;
+    a.nitems = c->naux;
     a.plane_part = c->plane_part_d;
     a.vol_out = c->vol_out_d;
     a.readings = c->kread;
@@ -1060,6 +1064,15 @@ spg_status spg_create_batch(int nvol, const spg_volume_params *params, const spg
     }
     ctx->total = off;
     ctx->nplanes = plane;
+    std::vector<std::pair<int, int>> aux_range;
+    const std::vector<WorkItem> aux = aux_items(ctx->vols_h, &aux_range);
+    ctx->naux = (int)aux.size();
+    const int nparts = std::max(plane * AUX_SEG, ctx->naux);
+    for (int j = 0; j < nvol; j++) {
+        VolDesc &d = ctx->vols_h[j];
+        d.aux_begin = aux_range[j].first;
+        d.aux_end = aux_range[j].second;
+    }
 
     auto bail = [&](cudaError_t err, const char *what) {
         std::string m = std::string("spg_create: ") + what + ": " + cudaGetErrorString(err);
@@ -1088,8 +1101,9 @@ spg_status spg_create_batch(int nvol, const spg_volume_params *params, const spg
     if ((e = dalloc(&ctx->st_d, sizeof(DevState))) != cudaSuccess) return bail(e, "alloc state");
     if ((e = dalloc(&ctx->hist_d, (size_t)ctx->hist_cap * nvol * 5 * sizeof(double))) != cudaSuccess)
         return bail(e, "alloc history");
-    if ((e = dalloc(&ctx->plane_part_d, (size_t)plane * AUX_SEG * 4 * sizeof(double))) != cudaSuccess)
+    if ((e = dalloc(&ctx->plane_part_d, (size_t)nparts * 4 * sizeof(double))) != cudaSuccess)
         return bail(e, "alloc partials");
+    if ((e = dalloc(&ctx->aux_items_d, aux.size() * sizeof(WorkItem))) != cudaSuccess) return bail(e, "alloc items");
     if ((e = dalloc(&ctx->vol_out_d, (size_t)nvol * 8 * sizeof(double))) != cudaSuccess) return bail(e, "alloc");
     if ((e = dalloc(&ctx->maxw_d, (size_t)nvol * sizeof(double))) != cudaSuccess) return bail(e, "alloc");
     if ((e = dalloc(&ctx->rstats_d, (size_t)nvol * 6 * sizeof(double))) != cudaSuccess) return bail(e, "alloc");
@@ -1112,6 +1126,9 @@ spg_status spg_create_batch(int nvol, const spg_volume_params *params, const spg
     if ((e = cudaMemcpyAsync(ctx->plane_vol_d, ctx->plane_vol_h.data(), plane * sizeof(int), cudaMemcpyHostToDevice,
                              ctx->stream)) != cudaSuccess)
         return bail(e, "upload plane map");
+    if ((e = cudaMemcpyAsync(ctx->aux_items_d, aux.data(), aux.size() * sizeof(WorkItem), cudaMemcpyHostToDevice,
+                             ctx->stream)) != cudaSuccess)
+        return bail(e, "upload items");
     if ((e = cudaMemcpyAsync(ctx->vols_d, ctx->vols_h.data(), nvol * sizeof(VolDesc), cudaMemcpyHostToDevice,
                              ctx->stream)) != cudaSuccess)
         return bail(e, "upload descriptors");
@@ -1177,7 +1194,7 @@ spg_status spg_set_data(spg_ctx *ctx, int vol, const void *b, const void *w, spg
         ctx->reweighted = false;
     }
     ctx->launches += 1;
-    CK(launch_validate(aux_params(ctx), vol, d.nz, ctx->B, ctx->W, store_bf16, ctx->maxw_d, ctx->stream),
+    CK(launch_validate(aux_params(ctx), vol, d.aux_end - d.aux_begin, ctx->B, ctx->W, store_bf16, ctx->maxw_d, ctx->stream),
        "validate");
     double o[8];
     CK(cudaMemcpyAsync(o, ctx->vol_out_d + (size_t)vol * 8, sizeof(o), cudaMemcpyDeviceToHost, ctx->stream),
@@ -1372,7 +1389,7 @@ spg_status spg_set_anchor(spg_ctx *ctx, int vol, float gamma, const float *x_anc
     // stage the anchor in the l1-weight buffer (re-set by the next spg_reweight)
     spg_status s = copy_volume_in(ctx, ctx->OM1, 4, d, x_anchor);
     if (s != SPG_OK) return s;
-    CK(launch_anchor(aux_params(ctx), vol, d.nz, ctx->B, ctx->W, ctx->bf16(), ctx->OM1, gamma, ctx->maxw_d,
+    CK(launch_anchor(aux_params(ctx), vol, d.aux_end - d.aux_begin, ctx->B, ctx->W, ctx->bf16(), ctx->OM1, gamma, ctx->maxw_d,
                      ctx->stream),
        "anchor");
     ctx->launches += 1;
@@ -1712,7 +1729,8 @@ spg_status spg_certificate(spg_ctx *ctx, int vol, double *out)
     const float *xb[4] = {ctx->X[c], ctx->X[k], ctx->xd() ? nullptr : ctx->X[ctx->aux_of(k)],
                           ctx->xd() ? ctx->X[ctx->aux_of(k)] : nullptr};
     if (!ctx->certQ) CK(dalloc(&ctx->certQ, (size_t)ctx->total * 3 * sizeof(float)), "alloc certificate field");
-    CK(launch_certificate4(aux_params(ctx), xb, ctx->W, ctx->bf16(), ctx->OMTV, ctx->certQ, ctx->total, ctx->stream),
+    CK(launch_certificate(aux_params(ctx), vol, ctx->vols_h[vol].nz, xb, ctx->W, ctx->bf16(), ctx->OMTV, ctx->certQ,
+                          ctx->total, ctx->stream),
        "certificate");
     ctx->launches += 2;
     double o[8];

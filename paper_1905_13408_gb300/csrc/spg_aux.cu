@@ -4,16 +4,33 @@
 // and the plain step used under alternative readings of the paper.
 //
 // None of them is on the fused hot path, so they use plain global loads.
-// All but the two adjoint passes run AUX_SEG CTAs per z-plane (one per row
-// segment), every reduction keeps one partial per segment, and the last CTA
-// to finish sums the partials of each volume in segment order, so the
-// results are deterministic; the adjoint passes march over z (a CTA per
-// tile of rows and run of planes) and keep one scalar partial per CTA,
-// which the host sums in a fixed order. No kernel here waits on another CTA.
+// The adopted reading's re-weighting and objective,
+// the validation and the anchor march over z: a CTA takes 8 rows (a warp each)
+// of a 128-voxel chunk over a run of planes (AuxParams::items), each lane 4
+// voxels by 16-byte loads, the plane below kept in registers and the loads of
+// several planes issued together. The kernels of the alternative readings, the
+// certificate and the parameter scales run AUX_SEG CTAs per z-plane (one per row segment).
+// Every reduction keeps one partial per CTA, and the last CTA to finish sums
+// the partials of each volume in a fixed order, so the results are
+// deterministic; the adjoint passes keep one scalar partial per CTA, which the
+// host sums in a fixed order. No kernel here waits on another CTA.
+//
+// Sums across a CTA run in float-float (spg_ff.cuh): with double shuffles
+// GB300's narrow FP64 pipe took most of these passes' time on small volumes.
+// Measured (whole calls, host work included), a CTA per row segment with double
+// sums -> march with float-float sums: re-weighting 64^3 23.0 -> 12.1 us,
+// 101 x 147 x 183 42.9 -> 25.2, 256^3 114 -> 62, 512^3 520 -> 349 (12 bytes a
+// voxel at the copy rate: 237); objective 50.1 -> 38.2, 61.3 -> 50.3, 124 -> 100,
+// 495 -> 436 (20 bytes: 396); spg_set_data with its validation 45.2 -> 33.3,
+// 84.4 -> 71.9, 146 -> 98, 717 -> 518 (copies and one read, 24 bytes: 475).
+// The certificate as one march without its stored field was slower than its two
+// row-segment passes (256^3 254 us against 224, 512^3 1649 against 1307: 16
+// warps per SM waiting for each plane's loads) and is not kept.
 #include <cuda_bf16.h>
 
 #include <algorithm>
 
+#include "spg_ff.cuh"
 #include "spg_internal.h"
 
 namespace spg {
@@ -40,6 +57,7 @@ struct KSum {
         s = t;
     }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
+    __device__ __forceinline__ ff::FF pair() const { return {s, -c}; }
 };
 
 __device__ __forceinline__ float ld_data(const void *p, bool bf16, long long i)
@@ -87,6 +105,86 @@ __device__ __forceinline__ double block_max(double v, double *scratch)
     return v;
 }
 
+// CTA sums of 4 float-float values (double where those could overflow), fixed
+// order; lane q < 4 of warp 0 returns quantity q. red: 4 doubles per warp.
+__device__ __forceinline__ double block_sum4(const ff::FF (&v)[4], double *red)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const bool big = ff::too_big(v[0]) || ff::too_big(v[1]) || ff::too_big(v[2]) || ff::too_big(v[3]);
+    double r = 0.0;
+    if (!__syncthreads_or(big ? 1 : 0)) {
+        ff::FF *const rf = reinterpret_cast<ff::FF *>(red);
+        const ff::FF s = ff::warp_sum4(v, lane);
+        if ((lane & 7) == 0) rf[warp * 4 + (lane >> 3)] = s;
+        __syncthreads();
+        if (warp == 0) r = ff::to_double(ff::cross_warp_sum4(rf, nw, lane, ff::FF{0.f, 0.f}));
+    } else {
+        const double w[4] = {ff::to_double(v[0]), ff::to_double(v[1]), ff::to_double(v[2]), ff::to_double(v[3])};
+        const double s = ff::warp_sum4(w, lane);
+        if ((lane & 7) == 0) red[warp * 4 + (lane >> 3)] = s;
+        __syncthreads();
+        if (warp == 0) r = ff::cross_warp_sum4(red, nw, lane, 0.0);
+    }
+    __syncthreads();
+    return r;
+}
+
+// CTA maximum of floats (exact); valid in thread 0. red: one float per warp.
+__device__ __forceinline__ float block_fmax(float v, float *red)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(FULL, v, o));
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        v = lane < (int)(blockDim.x >> 5) ? red[lane] : v;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(FULL, v, o));
+    }
+    __syncthreads();
+    return v;
+}
+
+// A CTA's partial of a march: three sums and, as a float in the first slot, a
+// maximum (or a fourth sum).
+__device__ __forceinline__ float *part_max(double *pp) { return reinterpret_cast<float *>(pp); }
+
+// Last CTA: sums (slots 1 .. 3, or 0 .. 3 without a maximum) and the maximum of
+// the partials [b, e) of one volume, by `nw` warps of which this is warp w, in
+// a fixed order: every lane gets all values. With nw > 1 the warps' results
+// meet in `red` (4 doubles a warp) behind CTA barriers.
+__device__ __forceinline__ void part_total(double *part, int b, int e, int w, int nw, bool has_max, double *red,
+                                           double (&a)[4], float &mx)
+{
+    const int lane = threadIdx.x & 31;
+    a[0] = a[1] = a[2] = a[3] = 0.0;
+    mx = 0.f;
+    for (int q = b + w * 32 + lane; q < e; q += 32 * nw) {
+        double *pp = part + (long long)q * 4;
+        if (has_max) mx = fmaxf(mx, __ldcg(part_max(pp)));
+        else a[0] += __ldcg(pp);
+        a[1] += __ldcg(pp + 1);
+        a[2] += __ldcg(pp + 2);
+        a[3] += __ldcg(pp + 3);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
+    double s = ff::warp_sum4(a, lane);
+    if (nw > 1) {
+        float *const rm = reinterpret_cast<float *>(red + 32 * 4);
+        if ((lane & 7) == 0) red[w * 4 + (lane >> 3)] = s;
+        if (lane == 0) rm[w] = mx;
+        __syncthreads();
+        s = ff::cross_warp_sum4(red, nw, lane, 0.0);
+        s = __shfl_sync(FULL, s, lane >> 3);
+        for (int k = 0; k < nw; k++) mx = fmaxf(mx, rm[k]);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int c = 0; c < 4; c++) a[c] = __shfl_sync(FULL, s, 8 * c);
+}
+
 // Last-CTA election on a counter; returns true in every thread of the last CTA.
 __device__ bool last_block(unsigned int *ticket, int *flag_smem)
 {
@@ -100,114 +198,6 @@ __device__ bool last_block(unsigned int *ticket, int *flag_smem)
     const bool last = *flag_smem != 0;
     if (last) __threadfence();
     return last;
-}
-
-// ---------------- validation ----------------
-// One CTA per z-plane of volume `vol`: max w, min w, count(w <= 0 or w not
-// finite), count(b not finite).
-__global__ void validate_kernel(AuxParams a, int vol, const void *b, const void *w, bool bf16, double *maxw_out)
-{
-    __shared__ double scratch[32 * 4];
-    __shared__ int flag;
-    const VolDesc V = a.vols[vol];
-    const int z = blockIdx.x / AUX_SEG;
-    int r0, r1;
-    seg_rows(V.ny, blockIdx.x % AUX_SEG, r0, r1);
-    // per-thread work in float32 and integers (max and min are exact in any precision)
-    float fmx = 0.f, fmn = INFINITY;
-    int bad_w = 0, bad_b = 0;
-    for (int t = threadIdx.x; t < (r1 - r0) * V.nx; t += blockDim.x) {
-        const int x = t % V.nx, y = r0 + t / V.nx;
-        const long long i = V.off + ((long long)z * V.ny + y) * V.pitch + x;
-        const float wv = ld_data(w, bf16, i), bv = ld_data(b, bf16, i);
-        const bool wfin = isfinite(wv);
-        bad_w += (!(wv > 0.f) || !wfin) ? 1 : 0;
-        bad_b += isfinite(bv) ? 0 : 1;
-        if (wfin) {
-            fmx = fmaxf(fmx, wv);
-            fmn = fminf(fmn, wv);
-        }
-    }
-    double mx = block_max((double)fmx, scratch);
-    const double nmn = block_max(-(double)fmn, scratch);
-    double c[2] = {(double)bad_w, (double)bad_b};
-    block_sum<2>(c, scratch);
-    if (threadIdx.x == 0) {
-        double *pp = a.plane_part + (long long)blockIdx.x * 4;
-        pp[0] = mx;
-        pp[1] = -nmn;
-        pp[2] = c[0];
-        pp[3] = c[1];
-    }
-    if (!last_block(&a.st->ticket_aux, &flag)) return;
-    {
-        double m = 0, n = INFINITY, c2[2] = {0, 0};
-        for (int q = threadIdx.x; q < V.nz * AUX_SEG; q += blockDim.x) {
-            const double *pp = a.plane_part + (long long)q * 4;
-            m = fmax(m, __ldcg(pp + 0));
-            n = fmin(n, __ldcg(pp + 1));
-            c2[0] += __ldcg(pp + 2);
-            c2[1] += __ldcg(pp + 3);
-        }
-        m = block_max(m, scratch);
-        n = -block_max(-n, scratch);
-        block_sum<2>(c2, scratch);
-        const double bw = c2[0], bb = c2[1];
-        if (threadIdx.x != 0) return;
-        double *o = a.vol_out + (long long)vol * 8;
-        o[0] = m;
-        o[1] = n;
-        o[2] = bw;
-        o[3] = bb;
-        maxw_out[vol] = m;
-        a.st->ticket_aux = 0;
-        __threadfence();
-    }
-}
-
-// ---------------- implicit-gradient anchor (Eq. 22 / Eq. 31) ----------------
-__device__ __forceinline__ void st_data(void *p, bool bf16, long long i, float v)
-{
-    if (bf16) {
-        __nv_bfloat16 h = __float2bfloat16_rn(v);
-        reinterpret_cast<uint16_t *>(p)[i] = *reinterpret_cast<uint16_t *>(&h);
-    } else {
-        reinterpret_cast<float *>(p)[i] = v;
-    }
-}
-
-// w' = w + 2 gamma, b' = (w b + 2 gamma a) / w'; then max w' per volume.
-__global__ void anchor_kernel(AuxParams a, int vol, void *b, void *w, bool bf16, const float *anchor, float gamma,
-                              double *maxw_out)
-{
-    __shared__ double scratch[32 * 4];
-    __shared__ int flag;
-    const VolDesc V = a.vols[vol];
-    const int z = blockIdx.x / AUX_SEG;
-    int r0, r1;
-    seg_rows(V.ny, blockIdx.x % AUX_SEG, r0, r1);
-    double mx = 0.0;
-    for (int t = threadIdx.x; t < (r1 - r0) * V.nx; t += blockDim.x) {
-        const int x = t % V.nx, y = r0 + t / V.nx;
-        const long long i = V.off + ((long long)z * V.ny + y) * V.pitch + x;
-        const float wv = ld_data(w, bf16, i), bv = ld_data(b, bf16, i);
-        const float w2 = wv + 2.0f * gamma;
-        const float b2 = (wv * bv + 2.0f * gamma * anchor[i]) / w2;
-        st_data(w, bf16, i, w2);
-        st_data(b, bf16, i, b2);
-        mx = fmax(mx, (double)ld_data(w, bf16, i));
-    }
-    mx = block_max(mx, scratch);
-    if (threadIdx.x == 0) a.plane_part[(long long)blockIdx.x * 4] = mx;
-    if (!last_block(&a.st->ticket_aux, &flag)) return;
-    double m = 0;
-    for (int q = threadIdx.x; q < V.nz * AUX_SEG; q += blockDim.x) m = fmax(m, __ldcg(a.plane_part + (long long)q * 4));
-    m = block_max(m, scratch);
-    if (threadIdx.x == 0) {
-        maxw_out[vol] = m;
-        a.st->ticket_aux = 0;
-        __threadfence();
-    }
 }
 
 // Sec. 2.5 scales: sum (w b)^2, sum w, max w, min w of one volume.
@@ -415,38 +405,265 @@ __device__ __forceinline__ void unpack4(const float4 v, float (&o)[4])
     o[3] = v.w;
 }
 
-// x and D x (Eq. 12, zero on first planes) at voxels x0 .. x0+3 of row (y, z);
-// inactive lanes (x0 >= nx) get zeros but still take part in the shuffle.
-__device__ __forceinline__ void grad4_at(const VolDesc &V, const float *xs, int x0, int y, int z, int lane,
-                                         bool act, float (&xc)[4], float (&gx)[4], float (&gy)[4], float (&gz)[4])
+// Where a thread of a march works: its row, first voxel and planes.
+struct March {
+    int x0, y, z0, z1, lane;
+    bool act;      // row and first voxel inside the volume
+    long long i;   // element index of voxel x0 of the row on plane z0
+    long long PS;  // plane stride
+};
+
+__device__ __forceinline__ March march_place(const VolDesc &V, const WorkItem &W)
 {
-    const long long row = V.off + ((long long)z * V.ny + y) * V.pitch;
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 c = act ? ld4(xs + row + x0) : zero;
-    float xl = __shfl_up_sync(FULL, c.w, 1);
-    if (lane == 0) xl = (act && x0 >= 1) ? xs[row + x0 - 1] : c.x;
-    if (x0 == 0) xl = c.x;
-    const float4 u = (act && y >= 1) ? ld4(xs + row - V.pitch + x0) : c;
-    const float4 w = (act && z >= 1) ? ld4(xs + row - (long long)V.pitch * V.ny + x0) : c;
-    float uu[4], ww[4];
-    unpack4(c, xc);
-    unpack4(u, uu);
-    unpack4(w, ww);
+    March M;
+    M.lane = threadIdx.x & 31;
+    M.x0 = W.x0 + 4 * M.lane;
+    M.y = W.y0 + (threadIdx.x >> 5);
+    M.z0 = W.z0;
+    M.z1 = W.z1;
+    M.act = M.y < V.ny && M.x0 < V.nx;
+    M.PS = (long long)V.pitch * V.ny;
+    M.i = V.off + ((long long)W.z0 * V.ny + (M.y < V.ny ? M.y : 0)) * V.pitch + (M.x0 < V.nx ? M.x0 : 0);
+    return M;
+}
+
+// ---------------- validation ----------------
+// max w, min w, count(w <= 0 or w not finite), count(b not finite) of volume
+// `vol`, over its march items.
+__global__ void __launch_bounds__(AUX_THREADS)
+    validate_kernel(AuxParams a, int vol, const void *b, const void *w, bool bf16, double *maxw_out)
+{
+    __shared__ float red[32];
+    __shared__ int cnt[2], flag;
+    const VolDesc V = a.vols[vol];
+    const WorkItem W = a.items[V.aux_begin + blockIdx.x];
+    const March M = march_place(V, W);
+    float fmx = 0.f, nmn = -INFINITY;
+    int bad_w = 0, bad_b = 0;
+    constexpr int U = 4;
+    for (int z = M.z0; z < M.z1; z += U) {
+        float4 bv[U], wv[U];
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
-        gx[q] = xc[q] - (q ? xc[q - 1] : xl);
-        gy[q] = xc[q] - uu[q];
-        gz[q] = xc[q] - ww[q];
+        for (int u = 0; u < U; u++)
+            if (M.act && z + u < M.z1) {
+                const long long i = M.i + (long long)(z + u - M.z0) * M.PS;
+                bv[u] = ld4_data(b, bf16, i);
+                wv[u] = ld4_data(w, bf16, i);
+            }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (!(M.act && z + u < M.z1)) continue;
+            float bb[4], ww[4];
+            unpack4(bv[u], bb);
+            unpack4(wv[u], ww);
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                if (M.x0 + q >= V.nx) continue;
+                const bool wfin = isfinite(ww[q]);
+                bad_w += (!(ww[q] > 0.f) || !wfin) ? 1 : 0;
+                bad_b += isfinite(bb[q]) ? 0 : 1;
+                if (wfin) {
+                    fmx = fmaxf(fmx, ww[q]);
+                    nmn = fmaxf(nmn, -ww[q]);
+                }
+            }
+        }
+    }
+    if (threadIdx.x < 2) cnt[threadIdx.x] = 0;
+    const float mx = block_fmax(fmx, red), nm = block_fmax(nmn, red);
+    bad_w = __reduce_add_sync(FULL, bad_w);
+    bad_b = __reduce_add_sync(FULL, bad_b);
+    if (M.lane == 0 && (bad_w | bad_b)) {
+        atomicAdd(&cnt[0], bad_w);
+        atomicAdd(&cnt[1], bad_b);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float *pp = part_max(a.plane_part + (long long)blockIdx.x * 4);
+        pp[0] = mx;
+        pp[1] = nm;
+        pp[2] = __int_as_float(cnt[0]);
+        pp[3] = __int_as_float(cnt[1]);
+    }
+    if (!last_block(&a.st->ticket_aux, &flag)) return;
+    float m = 0.f, n = -INFINITY;
+    unsigned long long bw = 0, bb = 0;
+    for (int q = threadIdx.x; q < V.aux_end - V.aux_begin; q += blockDim.x) {
+        const float4 p = __ldcg(reinterpret_cast<const float4 *>(a.plane_part + (long long)q * 4));
+        m = fmaxf(m, p.x);
+        n = fmaxf(n, p.y);
+        bw += (unsigned)__float_as_int(p.z);
+        bb += (unsigned)__float_as_int(p.w);
+    }
+    m = block_fmax(m, red);
+    n = block_fmax(n, red);
+    const bool any_w = __syncthreads_or(bw != 0) != 0, any_b = __syncthreads_or(bb != 0) != 0;
+    if (threadIdx.x != 0) return;
+    double *o = a.vol_out + (long long)vol * 8;
+    o[0] = m;
+    o[1] = -n;
+    o[2] = any_w ? 1.0 : 0.0;  // whether there are any; the counts are not used
+    o[3] = any_b ? 1.0 : 0.0;
+    maxw_out[vol] = m;
+    a.st->ticket_aux = 0;
+    __threadfence();
+}
+
+// ---------------- implicit-gradient anchor (Eq. 22 / Eq. 31) ----------------
+__device__ __forceinline__ void st_data(void *p, bool bf16, long long i, float v)
+{
+    if (bf16) {
+        __nv_bfloat16 h = __float2bfloat16_rn(v);
+        reinterpret_cast<uint16_t *>(p)[i] = *reinterpret_cast<uint16_t *>(&h);
+    } else {
+        reinterpret_cast<float *>(p)[i] = v;
     }
 }
 
-__global__ void reweight4_kernel(AuxParams a, const float *xcur, float *om1, float *omtv, const double *maxw,
-                                 double *rstats, VolDesc *vols_rw);
-__global__ void objective4_kernel(AuxParams a, const float *xcur, const void *b, const void *w, bool bf16,
-                                  const float *om1, const float *omtv);
+// w' = w + 2 gamma, b' = (w b + 2 gamma a) / w'; then max w' of the volume.
+__global__ void __launch_bounds__(AUX_THREADS)
+    anchor_kernel(AuxParams a, int vol, void *b, void *w, bool bf16, const float *anchor, float gamma, double *maxw_out)
+{
+    __shared__ float red[32];
+    __shared__ int flag;
+    const VolDesc V = a.vols[vol];
+    const WorkItem W = a.items[V.aux_begin + blockIdx.x];
+    const March M = march_place(V, W);
+    float mx = 0.f;
+    constexpr int U = 2;
+    for (int z = M.z0; z < M.z1; z += U) {
+        float4 bv[U], wv[U], av[U];
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (M.act && z + u < M.z1) {
+                const long long i = M.i + (long long)(z + u - M.z0) * M.PS;
+                bv[u] = ld4_data(b, bf16, i);
+                wv[u] = ld4_data(w, bf16, i);
+                av[u] = ld4(anchor + i);
+            }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (!(M.act && z + u < M.z1)) continue;
+            const long long i = M.i + (long long)(z + u - M.z0) * M.PS;
+            float bb[4], ww[4], an[4];
+            unpack4(bv[u], bb);
+            unpack4(wv[u], ww);
+            unpack4(av[u], an);
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                if (M.x0 + q >= V.nx) continue;  // the padding stays as it is
+                const float w2 = ww[q] + 2.0f * gamma;
+                const float b2 = (ww[q] * bb[q] + 2.0f * gamma * an[q]) / w2;
+                st_data(w, bf16, i + q, w2);
+                st_data(b, bf16, i + q, b2);
+                mx = fmaxf(mx, bf16 ? __uint_as_float((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(w2)) << 16) : w2);
+            }
+        }
+    }
+    mx = block_fmax(mx, red);
+    if (threadIdx.x == 0) *part_max(a.plane_part + (long long)blockIdx.x * 4) = mx;
+    if (!last_block(&a.st->ticket_aux, &flag)) return;
+    float m = 0.f;
+    for (int q = threadIdx.x; q < V.aux_end - V.aux_begin; q += blockDim.x)
+        m = fmaxf(m, __ldcg(part_max(a.plane_part + (long long)q * 4)));
+    m = block_fmax(m, red);
+    if (threadIdx.x == 0) {
+        maxw_out[vol] = m;
+        a.st->ticket_aux = 0;
+        __threadfence();
+    }
+}
 
-// Last CTA of a re-weighting launch: per-volume max omtv, nnz, sums, and
-// tau = 1/L (FP64), then the round restarts.
+// D x (Eq. 12) at 4 voxels: c on their row, xl at x0-1, u on the row above
+// (y-1), w on the plane below; a missing neighbour is the voxel itself.
+__device__ __forceinline__ void grad4(const float (&c)[4], float xl, const float (&u)[4], const float (&w)[4],
+                                      float (&gx)[4], float (&gy)[4], float (&gz)[4])
+{
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        gx[q] = c[q] - (q ? c[q - 1] : xl);
+        gy[q] = c[q] - u[q];
+        gz[q] = c[q] - w[q];
+    }
+}
+
+// x on U planes from plane z on, and what their differences need: the row
+// above and, for a chunk's first lane, the voxel to the left. Planes from z1 on
+// are not read.
+template <int U>
+struct XRows {
+    float4 c[U], u[U];
+    float l[U];
+    __device__ __forceinline__ void load(const VolDesc &V, const March &M, const float *x, int z)
+    {
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < U; k++) {
+            const bool ok = M.act && z + k < M.z1;
+            const long long i = M.i + (long long)(z + k - M.z0) * M.PS;
+            c[k] = ok ? ld4(x + i) : zero;
+            u[k] = (ok && M.y >= 1) ? ld4(x + i - V.pitch) : c[k];
+            l[k] = (ok && M.lane == 0 && M.x0 >= 1) ? x[i - 1] : 0.f;
+        }
+    }
+    // neighbours of plane k: xl from the lane before (every lane calls it)
+    __device__ __forceinline__ void take(const March &M, int k, float (&cc)[4], float &xl, float (&uu)[4]) const
+    {
+        unpack4(c[k], cc);
+        unpack4(u[k], uu);
+        xl = __shfl_up_sync(FULL, cc[3], 1);
+        if (M.lane == 0) xl = l[k];
+        if (M.x0 == 0) xl = cc[0];
+    }
+};
+
+// One volume's re-weighting statistics and step tau = 1/L (FP64).
+__device__ __forceinline__ void set_round(const AuxParams &a, int v, const VolDesc &W, double m, double n, double s1,
+                                          double s2, const double *maxw, double *rstats, VolDesc *vols_rw)
+{
+    const double L = maxw[v] + 12.0 * (double)W.lambda_tv * m / (double)W.mu;
+    const double tau = 1.0 / L;
+    double *o = rstats + (long long)v * 6;
+    o[0] = m;
+    o[1] = n;
+    o[2] = s1;
+    o[3] = s2;
+    o[4] = L;
+    o[5] = tau;
+    vols_rw[v].tau = (float)tau;
+    vols_rw[v].kmom = 0;  // extrapolation restarts with the round
+    vols_rw[v].beta_last = 0.f;
+}
+
+__device__ __forceinline__ void set_objective(const AuxParams &a, int v, const VolDesc &W, double d, double l, double t)
+{
+    double *o = a.vol_out + (long long)v * 8;
+    o[0] = d;
+    o[1] = (double)W.lambda_l1 * l;
+    o[2] = (double)W.lambda_tv * t;
+    o[3] = o[0] + o[1] + o[2];
+}
+
+// Last CTA of a march over all volumes: f(volume, descriptor, sums, maximum)
+// once per volume, by one thread: a warp per volume, or all warps together
+// where there are fewer volumes than warps.
+template <class F>
+__device__ __forceinline__ void per_volume(const AuxParams &a, bool has_max, double *red, F f)
+{
+    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+    const bool together = a.nvol < nw;
+    for (int v = together ? 0 : warp; v < a.nvol; v += together ? 1 : nw) {
+        const VolDesc W = a.vols[v];
+        double s[4];
+        float mx;
+        part_total(a.plane_part, W.aux_begin, W.aux_end, together ? warp : 0, together ? nw : 1, has_max, red, s, mx);
+        if (lane == 0 && (!together || warp == 0)) f(v, W, s, mx);
+    }
+    __syncthreads();
+}
+
+// Last CTA of a re-weighting launch over row segments: per-volume max omtv,
+// nnz, sums, and tau = 1/L, then the round restarts.
 __device__ void reweight_finish(const AuxParams &a, const double *maxw, double *rstats, VolDesc *vols_rw,
                                 double *scratch)
 {
@@ -463,20 +680,7 @@ __device__ void reweight_finish(const AuxParams &a, const double *maxw, double *
         m = block_max(m, scratch);
         block_sum<3>(c3, scratch);
         const double n = c3[0], s1 = c3[1], s2 = c3[2];
-        if (threadIdx.x == 0) {
-            const double L = maxw[v] + 12.0 * (double)W.lambda_tv * m / (double)W.mu;
-            const double tau = 1.0 / L;
-            double *o = rstats + (long long)v * 6;
-            o[0] = m;
-            o[1] = n;
-            o[2] = s1;
-            o[3] = s2;
-            o[4] = L;
-            o[5] = tau;
-            vols_rw[v].tau = (float)tau;
-            vols_rw[v].kmom = 0;  // extrapolation restarts with the round
-            vols_rw[v].beta_last = 0.f;
-        }
+        if (threadIdx.x == 0) set_round(a, v, W, m, n, s1, s2, maxw, rstats, vols_rw);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -486,7 +690,7 @@ __device__ void reweight_finish(const AuxParams &a, const double *maxw, double *
     }
 }
 
-// Last CTA of an objective launch: per-volume (data, l1, tv, total).
+// Last CTA of an objective launch over row segments.
 __device__ void objective_finish(const AuxParams &a, double *scratch)
 {
     for (int v = 0; v < a.nvol; v++) {
@@ -500,12 +704,7 @@ __device__ void objective_finish(const AuxParams &a, double *scratch)
         }
         block_sum<3>(c3, scratch);
         if (threadIdx.x != 0) continue;
-        const double d = c3[0], l = c3[1], t = c3[2];
-        double *o = a.vol_out + (long long)v * 8;
-        o[0] = d;
-        o[1] = (double)W.lambda_l1 * l;
-        o[2] = (double)W.lambda_tv * t;
-        o[3] = o[0] + o[1] + o[2];
+        set_objective(a, v, W, c3[0], c3[1], c3[2]);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -603,116 +802,152 @@ __global__ void objective_kernel(AuxParams a, const float *xcur, const void *b, 
     objective_finish(a, scratch);
 }
 
-// Re-weighting of the adopted reading, row-vector walk (same results as
-// reweight_kernel; padding columns of the pitch get zero weights).
-__global__ void reweight4_kernel(AuxParams a, const float *xcur, float *om1, float *omtv, const double *maxw,
-                                 double *rstats, VolDesc *vols_rw)
+// Re-weighting of the adopted reading, march (same results as
+// reweight_kernel; padding columns of the pitch get zero weights). Bound: x
+// read once, two volumes written, 12 bytes a voxel.
+__global__ void __launch_bounds__(AUX_THREADS, 4)
+    reweight_march_kernel(AuxParams a, const float *xcur, float *om1, float *omtv, const double *maxw, double *rstats,
+                          VolDesc *vols_rw)
 {
-    __shared__ double scratch[32 * 4];
+    __shared__ double red[32 * 4 + 16];
     __shared__ int flag;
-    const int plane = blockIdx.x / AUX_SEG;
-    const int vol = a.plane_vol[plane];
-    const VolDesc V = a.vols[vol];
-    const int z = plane - V.plane_begin;
-    int r0, r1;
-    seg_rows(V.ny, blockIdx.x % AUX_SEG, r0, r1);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int nchunk = (V.nx + 127) / 128;
-    float fmx = 0.f, nnz = 0.f;
+    const WorkItem W = a.items[blockIdx.x];
+    const VolDesc V = a.vols[W.vol];
+    const March M = march_place(V, W);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float pw[4];  // the plane below
+    unpack4((M.act && M.z0 >= 1) ? ld4(xcur + M.i - M.PS) : zero, pw);
+    float fmx = 0.f;
+    int nnz = 0;
     KSum c1, c2;
-    for (int rc = warp; rc < (r1 - r0) * nchunk; rc += nwarps) {
-        const int y = r0 + rc / nchunk, x0 = (rc % nchunk) * 128 + 4 * lane;
-        const bool act = x0 < V.nx;
-        float xc[4], gx[4], gy[4], gz[4], o1[4], ot[4];
-        grad4_at(V, xcur, x0, y, z, lane, act, xc, gx, gy, gz);
-        float s1 = 0.f, s2 = 0.f;
+    constexpr int U = 4;  // planes whose loads are in flight together
+    for (int z = M.z0; z < M.z1; z += U) {
+        XRows<U> X;
+        X.load(V, M, xcur, z);
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const bool valid = act && x0 + q < V.nx;
-            const float gn = sqrtf(gx[q] * gx[q] + gy[q] * gy[q] + gz[q] * gz[q]);
-            o1[q] = valid ? V.eps / (fabsf(xc[q]) + V.eps) : 0.f;
-            ot[q] = valid ? V.eps_tv / (gn + V.eps_tv) : 0.f;
-            fmx = fmaxf(fmx, ot[q]);
-            nnz += (valid && xc[q] != 0.f) ? 1.f : 0.f;
-            s1 += o1[q];
-            s2 += ot[q];
+        for (int k = 0; k < U; k++) {
+            if (z + k >= M.z1) break;
+            float xc[4], uu[4], xl, gx[4], gy[4], gz[4], o1[4], ot[4];
+            X.take(M, k, xc, xl, uu);
+            if (z + k == 0)
+#pragma unroll
+                for (int q = 0; q < 4; q++) pw[q] = xc[q];
+            grad4(xc, xl, uu, pw, gx, gy, gz);
+            const bool own = z + k >= V.halo_lo && z + k < V.nz - V.halo_hi;  // not a neighbour's plane
+            float s1 = 0.f, s2 = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const bool valid = M.act && M.x0 + q < V.nx;
+                const float gn = sqrtf(gx[q] * gx[q] + gy[q] * gy[q] + gz[q] * gz[q]);
+                o1[q] = valid ? V.eps / (fabsf(xc[q]) + V.eps) : 0.f;
+                ot[q] = valid ? V.eps_tv / (gn + V.eps_tv) : 0.f;
+                if (own) {
+                    fmx = fmaxf(fmx, ot[q]);
+                    nnz += (valid && xc[q] != 0.f) ? 1 : 0;
+                    s1 += o1[q];
+                    s2 += ot[q];
+                }
+                pw[q] = xc[q];
+            }
+            if (M.act) {
+                const long long i = M.i + (long long)(z + k - M.z0) * M.PS;
+                *reinterpret_cast<float4 *>(om1 + i) = make_float4(o1[0], o1[1], o1[2], o1[3]);
+                *reinterpret_cast<float4 *>(omtv + i) = make_float4(ot[0], ot[1], ot[2], ot[3]);
+            }
+            c1.add(s1);
+            c2.add(s2);
         }
-        if (act) {
-            const long long i = V.off + ((long long)z * V.ny + y) * V.pitch + x0;
-            *reinterpret_cast<float4 *>(om1 + i) = make_float4(o1[0], o1[1], o1[2], o1[3]);
-            *reinterpret_cast<float4 *>(omtv + i) = make_float4(ot[0], ot[1], ot[2], ot[3]);
-        }
-        c1.add(s1);
-        c2.add(s2);
     }
-    const double mx = block_max((double)fmx, scratch);
-    double sm[3] = {(double)nnz, c1.value(), c2.value()};
-    block_sum<3>(sm, scratch);
-    if (threadIdx.x == 0) {
-        double *pp = a.plane_part + (long long)blockIdx.x * 4;
-        pp[0] = mx;
-        pp[1] = sm[0];
-        pp[2] = sm[1];
-        pp[3] = sm[2];
-    }
+    fmx = block_fmax(fmx, reinterpret_cast<float *>(red));
+    const ff::FF v[4] = {{0.f, 0.f}, {(float)nnz, 0.f}, c1.pair(), c2.pair()};
+    const double s = block_sum4(v, red);
+    double *pp = a.plane_part + (long long)blockIdx.x * 4;
+    if (threadIdx.x == 0) *part_max(pp) = fmx;
+    else if (threadIdx.x < 4) pp[threadIdx.x] = s;
     if (!last_block(&a.st->ticket_aux, &flag)) return;
-    reweight_finish(a, maxw, rstats, vols_rw, scratch);
+    per_volume(a, true, red, [&](int vol, const VolDesc &D, const double (&t)[4], float mx) {
+        set_round(a, vol, D, (double)mx, t[1], t[2], t[3], maxw, rstats, vols_rw);
+    });
+    if (threadIdx.x == 0) {
+        a.st->k_round = 0;
+        a.st->ticket_aux = 0;
+        __threadfence();
+    }
 }
 
-// Objective of the adopted reading, row-vector walk (same sums as
-// objective_kernel; padding columns contribute nothing).
-__global__ void objective4_kernel(AuxParams a, const float *xcur, const void *b, const void *w, bool bf16,
-                                  const float *om1, const float *omtv)
+// Objective of the adopted reading, march (same sums as objective_kernel;
+// padding columns contribute nothing). Bound: 20 bytes a voxel.
+__global__ void __launch_bounds__(AUX_THREADS, 4)
+    objective_march_kernel(AuxParams a, const float *xcur, const void *b, const void *w, bool bf16, const float *om1,
+                           const float *omtv)
 {
-    __shared__ double scratch[32 * 4];
+    __shared__ double red[32 * 4 + 16];
     __shared__ int flag;
-    const int plane = blockIdx.x / AUX_SEG;
-    const int vol = a.plane_vol[plane];
-    const VolDesc V = a.vols[vol];
-    const int z = plane - V.plane_begin;
-    int r0, r1;
-    seg_rows(V.ny, blockIdx.x % AUX_SEG, r0, r1);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int nchunk = (V.nx + 127) / 128;
+    const WorkItem W = a.items[blockIdx.x];
+    const VolDesc V = a.vols[W.vol];
+    const March M = march_place(V, W);
     const float mu = V.mu;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float pw[4];
+    unpack4((M.act && M.z0 >= 1) ? ld4(xcur + M.i - M.PS) : zero, pw);
     KSum kd, kl, kt;
-    for (int rc = warp; rc < (r1 - r0) * nchunk; rc += nwarps) {
-        const int y = r0 + rc / nchunk, x0 = (rc % nchunk) * 128 + 4 * lane;
-        const bool act = x0 < V.nx;
-        const long long i = V.off + ((long long)z * V.ny + y) * V.pitch + x0;
-        float xc[4], gx[4], gy[4], gz[4], o1[4], ot[4], bv[4], wv[4];
-        grad4_at(V, xcur, x0, y, z, lane, act, xc, gx, gy, gz);
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        unpack4(act ? ld4(om1 + i) : zero, o1);
-        unpack4(act ? ld4(omtv + i) : zero, ot);
-        unpack4((act && w) ? ld4_data(b, bf16, i) : zero, bv);
-        unpack4((act && w) ? ld4_data(w, bf16, i) : zero, wv);
-        float sd = 0.f, sl = 0.f, st = 0.f;
+    constexpr int U = 1;  // more warps per SM beat more planes per warp here (2 planes at 2 CTAs: 522 us)
+    for (int z = M.z0; z < M.z1; z += U) {
+        XRows<U> X;
+        X.load(V, M, xcur, z);
+        float4 f1[U], ft[U], fb[U], fw[U];
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            if (!(act && x0 + q < V.nx)) continue;
-            const float qq = gx[q] * gx[q] + gy[q] * gy[q] + gz[q] * gz[q];
-            const float h = qq <= mu * mu ? qq * (0.5f / mu) : qq * rsqrtf(qq) - 0.5f * mu;
-            const float r = xc[q] - bv[q];
-            sd += 0.5f * wv[q] * r * r;
-            sl += o1[q] * fabsf(xc[q]);
-            st += ot[q] * h;
+        for (int k = 0; k < U; k++) {
+            const bool ok = M.act && z + k < M.z1;
+            const long long i = M.i + (long long)(z + k - M.z0) * M.PS;
+            f1[k] = ok ? ld4(om1 + i) : zero;
+            ft[k] = ok ? ld4(omtv + i) : zero;
+            fb[k] = (ok && w) ? ld4_data(b, bf16, i) : zero;
+            fw[k] = (ok && w) ? ld4_data(w, bf16, i) : zero;
         }
-        kd.add(sd);
-        kl.add(sl);
-        kt.add(st);
+#pragma unroll
+        for (int k = 0; k < U; k++) {
+            if (z + k >= M.z1) break;
+            float xc[4], uu[4], xl, gx[4], gy[4], gz[4], o1[4], ot[4], bv[4], wv[4];
+            X.take(M, k, xc, xl, uu);
+            if (z + k == 0)
+#pragma unroll
+                for (int q = 0; q < 4; q++) pw[q] = xc[q];
+            grad4(xc, xl, uu, pw, gx, gy, gz);
+            unpack4(f1[k], o1);
+            unpack4(ft[k], ot);
+            unpack4(fb[k], bv);
+            unpack4(fw[k], wv);
+            const bool own = z + k >= V.halo_lo && z + k < V.nz - V.halo_hi;
+            float sd = 0.f, sl = 0.f, st = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const float x = xc[q];
+                pw[q] = x;
+                if (!(own && M.act && M.x0 + q < V.nx)) continue;
+                const float qq = gx[q] * gx[q] + gy[q] * gy[q] + gz[q] * gz[q];
+                const float h = qq <= mu * mu ? qq * (0.5f / mu) : qq * rsqrtf(qq) - 0.5f * mu;
+                const float r = x - bv[q];
+                sd += 0.5f * wv[q] * r * r;
+                sl += o1[q] * fabsf(x);
+                st += ot[q] * h;
+            }
+            kd.add(sd);
+            kl.add(sl);
+            kt.add(st);
+        }
     }
-    double sm[3] = {kd.value(), kl.value(), kt.value()};
-    block_sum<3>(sm, scratch);
-    if (threadIdx.x == 0) {
-        double *pp = a.plane_part + (long long)blockIdx.x * 4;
-        pp[0] = sm[0];
-        pp[1] = sm[1];
-        pp[2] = sm[2];
-        pp[3] = 0;
-    }
+    const ff::FF v[4] = {kd.pair(), kl.pair(), kt.pair(), {0.f, 0.f}};
+    const double s = block_sum4(v, red);
+    if (threadIdx.x < 4) a.plane_part[(long long)blockIdx.x * 4 + threadIdx.x] = s;
     if (!last_block(&a.st->ticket_aux, &flag)) return;
-    objective_finish(a, scratch);
+    per_volume(a, false, red, [&](int vol, const VolDesc &D, const double (&t)[4], float) {
+        set_objective(a, vol, D, t[0], t[1], t[2]);
+    });
+    if (threadIdx.x == 0) {
+        a.st->ticket_aux = 0;
+        __threadfence();
+    }
 }
 
 // ---------------- one iteration under alternative readings ----------------
@@ -1283,8 +1518,8 @@ __global__ void __launch_bounds__(adj::THREADS) adjoint_apply_kernel(AdjParams a
 // xbuf = {x_{k+1}, x_k, x_{k-1} or null, d_k or null}.
 #define CERT_WALK_BEGIN                                                                  \
     const int plane_ = blockIdx.x / AUX_SEG;                                             \
-    const VolDesc V = a.vols[a.plane_vol[plane_]];                                       \
-    const int zz_ = plane_ - V.plane_begin;                                              \
+    const VolDesc V = a.vols[vol];                                                       \
+    const int zz_ = plane_;                                                              \
     int r0, r1;                                                                          \
     seg_rows(V.ny, blockIdx.x % AUX_SEG, r0, r1);                                        \
     const int lane_ = threadIdx.x & 31, warp_ = threadIdx.x >> 5, nw_ = blockDim.x >> 5; \
@@ -1335,7 +1570,7 @@ __device__ __forceinline__ void grad4_y(const VolDesc &V, const float *x, const 
     }
 }
 
-__global__ void certificate_q_kernel(AuxParams a, const float *xplus, const float *xk, const float *aux, int xd,
+__global__ void certificate_q_kernel(AuxParams a, int vol, const float *xplus, const float *xk, const float *aux, int xd,
                                      const float *omtv, float *Q, long long S)
 {
     CERT_WALK_BEGIN
@@ -1358,10 +1593,10 @@ __global__ void certificate_q_kernel(AuxParams a, const float *xplus, const floa
     ADJ_WALK_END
 }
 
-__global__ void certificate_r_kernel(AuxParams a, const float *xplus, const float *xk, const float *aux, int xd,
+__global__ void certificate_r_kernel(AuxParams a, int vol, const float *xplus, const float *xk, const float *aux, int xd,
                                      const void *w, bool bf16, const float *Q, long long S)
 {
-    __shared__ double scratch[32 * 4];
+    __shared__ double scratch[32 * 4 + 16];
     __shared__ int flag;
     KSum ks;
     CERT_WALK_BEGIN
@@ -1390,20 +1625,15 @@ __global__ void certificate_r_kernel(AuxParams a, const float *xplus, const floa
     }
     ks.add(acc);
     ADJ_WALK_END
-    double sm[1] = {ks.value()};
-    block_sum<1>(sm, scratch);
-    if (threadIdx.x == 0) a.plane_part[(long long)blockIdx.x * 4] = sm[0];
+    const ff::FF fv[4] = {ks.pair(), {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    const double s4 = block_sum4(fv, scratch);
+    if (threadIdx.x < 4) a.plane_part[(long long)blockIdx.x * 4 + threadIdx.x] = s4;
     if (!last_block(&a.st->ticket_aux, &flag)) return;
-    for (int v = 0; v < a.nvol; v++) {
-        const VolDesc W = a.vols[v];
-        double accv[1] = {0};
-        for (int q = (W.plane_begin + W.halo_lo) * AUX_SEG + threadIdx.x; q < (W.plane_begin + W.nz - W.halo_hi) * AUX_SEG; q += blockDim.x)
-            accv[0] += __ldcg(a.plane_part + (long long)q * 4);
-        block_sum<1>(accv, scratch);
-        if (threadIdx.x == 0) a.vol_out[(long long)v * 8 + 4] = accv[0];
-    }
-    __syncthreads();
+    double t[4];
+    float mx;
+    part_total(a.plane_part, V.halo_lo * AUX_SEG, (V.nz - V.halo_hi) * AUX_SEG, warp_, nw_, false, scratch, t, mx);
     if (threadIdx.x == 0) {
+        a.vol_out[(long long)vol * 8 + 4] = t[0];
         a.st->ticket_aux = 0;
         __threadfence();
     }
@@ -1411,17 +1641,17 @@ __global__ void certificate_r_kernel(AuxParams a, const float *xplus, const floa
 
 }  // namespace
 
-cudaError_t launch_validate(const AuxParams &a, int vol, int nz, const void *b, const void *w, bool bf16,
+cudaError_t launch_validate(const AuxParams &a, int vol, int nitems, const void *b, const void *w, bool bf16,
                             double *maxw_out, cudaStream_t s)
 {
-    validate_kernel<<<nz * AUX_SEG, AUX_THREADS, 0, s>>>(a, vol, b, w, bf16, maxw_out);
+    validate_kernel<<<nitems, AUX_THREADS, 0, s>>>(a, vol, b, w, bf16, maxw_out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_anchor(const AuxParams &a, int vol, int nz, void *b, void *w, bool bf16, const float *anchor,
+cudaError_t launch_anchor(const AuxParams &a, int vol, int nitems, void *b, void *w, bool bf16, const float *anchor,
                           float gamma, double *maxw_out, cudaStream_t s)
 {
-    anchor_kernel<<<nz * AUX_SEG, AUX_THREADS, 0, s>>>(a, vol, b, w, bf16, anchor, gamma, maxw_out);
+    anchor_kernel<<<nitems, AUX_THREADS, 0, s>>>(a, vol, b, w, bf16, anchor, gamma, maxw_out);
     return cudaGetLastError();
 }
 
@@ -1488,7 +1718,7 @@ cudaError_t launch_reweight(const AuxParams &a, const float *const *xbuf, float 
                             const double *maxw, double *rstats, VolDesc *vols_rw, cudaStream_t s)
 {
     if (a.readings == 0)
-        reweight4_kernel<<<a.nplanes * AUX_SEG, AUX_THREADS, 0, s>>>(a, xbuf[0], om1, omtv, maxw, rstats, vols_rw);
+        reweight_march_kernel<<<a.nitems, AUX_THREADS, 0, s>>>(a, xbuf[0], om1, omtv, maxw, rstats, vols_rw);
     else
         reweight_kernel<<<a.nplanes * AUX_SEG, AUX_THREADS, 0, s>>>(a, xbuf[0], om1, omtv, maxw, rstats, vols_rw);
     return cudaGetLastError();
@@ -1498,22 +1728,42 @@ cudaError_t launch_objective(const AuxParams &a, const float *const *xbuf, const
                              bool bf16, const float *om1, const float *omtv, cudaStream_t s)
 {
     if (a.readings == 0)
-        objective4_kernel<<<a.nplanes * AUX_SEG, AUX_THREADS, 0, s>>>(a, xbuf[0], b, w, bf16, om1, omtv);
+        objective_march_kernel<<<a.nitems, AUX_THREADS, 0, s>>>(a, xbuf[0], b, w, bf16, om1, omtv);
     else
         objective_kernel<<<a.nplanes * AUX_SEG, AUX_THREADS, 0, s>>>(a, xbuf[0], b, w, bf16, om1, omtv);
     return cudaGetLastError();
 }
 
-cudaError_t launch_certificate4(const AuxParams &a, const float *const *xbuf, const void *w, bool bf16,
-                                const float *omtv, float *Q, long long stride, cudaStream_t s)
+cudaError_t launch_certificate(const AuxParams &a, int vol, int nz, const float *const *xbuf, const void *w, bool bf16,
+                               const float *omtv, float *Q, long long stride, cudaStream_t s)
 {
     const bool xd = xbuf[3] != nullptr;
     const float *aux = xd ? xbuf[3] : xbuf[2];
-    certificate_q_kernel<<<a.nplanes * AUX_SEG, AUX_THREADS, 0, s>>>(a, xbuf[0], xbuf[1], aux, xd ? 1 : 0, omtv, Q,
-                                                                     stride);
-    certificate_r_kernel<<<a.nplanes * AUX_SEG, AUX_THREADS, 0, s>>>(a, xbuf[0], xbuf[1], aux, xd ? 1 : 0, w, bf16, Q,
-                                                                     stride);
+    certificate_q_kernel<<<nz * AUX_SEG, AUX_THREADS, 0, s>>>(a, vol, xbuf[0], xbuf[1], aux, xd ? 1 : 0, omtv, Q, stride);
+    certificate_r_kernel<<<nz * AUX_SEG, AUX_THREADS, 0, s>>>(a, vol, xbuf[0], xbuf[1], aux, xd ? 1 : 0, w, bf16, Q,
+                                                              stride);
     return cudaGetLastError();
+}
+
+std::vector<WorkItem> aux_items(const std::vector<VolDesc> &vols, std::vector<std::pair<int, int>> *ranges)
+{
+    long long tiles = 0;
+    for (const auto &d : vols) tiles += (long long)((d.nx + 127) / 128) * ((d.ny + 7) / 8) * d.nz;
+    // planes per item: about two waves of 4 CTAs per SM, 2 .. 32 planes (an
+    // item reads the plane below its first one again)
+    const int zc = (int)std::max<long long>(2, std::min<long long>(32, tiles / 1216));
+    std::vector<WorkItem> items;
+    ranges->clear();
+    for (size_t j = 0; j < vols.size(); j++) {
+        const auto &d = vols[j];
+        const int begin = (int)items.size();
+        for (int z = 0; z < d.nz; z += zc)
+            for (int y = 0; y < d.ny; y += 8)
+                for (int x = 0; x < d.nx; x += 128)
+                    items.push_back(WorkItem{(int)j, x, y, z, std::min(d.nz, z + zc), 0, 0, 0});
+        ranges->push_back({begin, (int)items.size()});
+    }
+    return items;
 }
 
 cudaError_t launch_generic_step(const GenericParams &g, cudaStream_t s)

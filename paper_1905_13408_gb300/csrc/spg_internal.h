@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
 #include <vector>
 
 #include "spg.h"
@@ -34,6 +35,7 @@ struct VolDesc {
     int kmom;                    // index of the next step's extrapolation weight in the beta table
     float beta_last;             // extrapolation weight used by the last step
     int readings;                // SPG_READ_* flags (0: the adopted readings, the fused path)
+    int aux_begin, aux_end;      // march items of the auxiliary passes that belong to this volume
     int halo_lo, halo_hi;        // first / last z-plane is a neighbour's plane (read, never written or summed)
 };
 
@@ -103,20 +105,27 @@ cudaError_t step_configure(const StepVariant &v, int *ctas_per_sm);
 cudaError_t step_launch(const StepVariant &v, int grid, const StepParams &p, cudaStream_t s);
 bool step_variant_supported(const StepVariant &v);
 
-// Auxiliary kernels (spg_aux.cu). Every one runs AUX_SEG CTAs per z-plane of
-// every volume (row segments) and reduces per-segment partials in a fixed order.
+// Auxiliary kernels (spg_aux.cu). The adopted reading's run one CTA per march
+// item (8 rows of a 128-voxel chunk over a run of planes), the others AUX_SEG
+// CTAs per z-plane of every volume (row segments); the last CTA reduces the
+// CTAs' partials in a fixed order.
 constexpr int AUX_SEG = 8;
 struct AuxParams {
     const VolDesc *vols;
     const int *plane_vol;    // volume of each global plane
     int nplanes, nvol;
     DevState *st;
-    double *plane_part;      // [nplanes * AUX_SEG][4]
+    const WorkItem *items;   // march items of every volume
+    int nitems;
+    double *plane_part;      // [max(nplanes * AUX_SEG, nitems)][4]
     double *vol_out;         // [nvol][8]
     int readings;            // SPG_READ_* flags of the context (0: the row-vector kernels)
 };
 
-cudaError_t launch_validate(const AuxParams &a, int vol, int nz, const void *b, const void *w, bool bf16,
+// March items of the given volumes, and each volume's range of them.
+std::vector<WorkItem> aux_items(const std::vector<VolDesc> &vols, std::vector<std::pair<int, int>> *ranges);
+// nitems: march items of volume `vol`.
+cudaError_t launch_validate(const AuxParams &a, int vol, int nitems, const void *b, const void *w, bool bf16,
                             double *maxw_out, cudaStream_t s);
 cudaError_t launch_convert_to_bf16(const float *src, uint16_t *dst, long long n, cudaStream_t s);
 cudaError_t launch_convert_to_f32(const uint16_t *src, float *dst, long long n, cudaStream_t s);
@@ -125,11 +134,11 @@ cudaError_t launch_reweight(const AuxParams &a, const float *const *xbuf, float 
                             const double *maxw, double *rstats, VolDesc *vols_rw, cudaStream_t s);
 cudaError_t launch_objective(const AuxParams &a, const float *const *xbuf, const void *b, const void *w,
                              bool bf16, const float *om1, const float *omtv, cudaStream_t s);
-// Strong-convexity certificate of the last step, xbuf = {x_{k+1}, x_k,
-// x_{k-1} or null, d_k or null}: two row-vector passes (Q = P(x+) - P(y) stored in
-// 3 fields of `stride` elements each, then the residual sum).
-cudaError_t launch_certificate4(const AuxParams &a, const float *const *xbuf, const void *w, bool bf16,
-                                const float *omtv, float *Q, long long stride, cudaStream_t s);
+// Strong-convexity certificate of volume `vol`'s last step, xbuf = {x_{k+1},
+// x_k, x_{k-1} or null, d_k or null}: two row-vector passes (Q = P(x+) - P(y)
+// stored in 3 fields of `stride` elements each, then the residual sum).
+cudaError_t launch_certificate(const AuxParams &a, int vol, int nz, const float *const *xbuf, const void *w, bool bf16,
+                               const float *omtv, float *Q, long long stride, cudaStream_t s);
 
 // Adjoint of one step (spg_aux.cu): given gnext = dL/dx_{k+1} and the step's
 // inputs, accumulates into gcur (dL/dx_k), gprev (dL/dx_{k-1}), gb, gw and the
@@ -246,7 +255,7 @@ cudaError_t launch_zfft_residual(float2 *F, const float *N, const float2 *Cd, fl
                                  const float2 *tw, cudaStream_t s);
 
 // Fold gamma |x - a|^2 into (b, w) of volume `vol` (a: float32 volume in the pitched layout).
-cudaError_t launch_anchor(const AuxParams &a, int vol, int nz, void *b, void *w, bool bf16, const float *anchor,
+cudaError_t launch_anchor(const AuxParams &a, int vol, int nitems, void *b, void *w, bool bf16, const float *anchor,
                           float gamma, double *maxw_out, cudaStream_t s);
 // RMS(w b), mean w, max w, min w of volume `vol` into vol_out[vol][0..3].
 cudaError_t launch_scales(const AuxParams &a, int vol, int nz, const void *b, const void *w, bool bf16,
