@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <functional>
+#include <map>
 #include <numeric>
 #include <queue>
 #include <climits>
@@ -14,6 +15,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "spg.h"
@@ -304,10 +306,9 @@ cudaError_t encode_set(const spg_ctx *ctx, const VolDesc &d, const StepVariant &
 long long item_cost(int z0, int z1) { return (long long)(z1 - z0) + 2; }
 
 // Longest-processing-time-first assignment of items to G CTAs: each item,
-// longest first, goes to the least-loaded CTA (lowest index on ties). Returns
-// the makespan in plane steps; with order/first given, fills the items of
-// CTA g as order[first[g] .. first[g+1]), longest first.
-long long lpt_schedule(const std::vector<long long> &cost, int G, std::vector<int> *order, std::vector<int> *first)
+// longest first, goes to the least-loaded CTA (lowest index on ties). Fills the
+// items of CTA g as order[first[g] .. first[g+1]), longest first.
+void lpt_schedule(const std::vector<long long> &cost, int G, std::vector<int> *order, std::vector<int> *first)
 {
     const int n = (int)cost.size();
     std::vector<int> idx(n);
@@ -316,41 +317,53 @@ long long lpt_schedule(const std::vector<long long> &cost, int G, std::vector<in
     using Slot = std::pair<long long, int>;
     std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
     for (int g = 0; g < G; g++) heap.push({0, g});
-    std::vector<int> owner(order ? n : 0);
-    long long makespan = 0;
+    std::vector<int> owner(n);
     for (int i : idx) {
         Slot sl = heap.top();
         heap.pop();
         sl.first += cost[i];
-        makespan = std::max(makespan, sl.first);
-        if (order) owner[i] = sl.second;
+        owner[i] = sl.second;
         heap.push(sl);
     }
-    if (order) {
-        first->assign(G + 1, 0);
-        for (int i = 0; i < n; i++) (*first)[owner[i] + 1]++;
-        for (int g = 0; g < G; g++) (*first)[g + 1] += (*first)[g];
-        order->assign(n, 0);
-        std::vector<int> pos(first->begin(), first->end() - 1);
-        for (int i : idx) (*order)[pos[owner[i]]++] = i;
-    }
-    return makespan;
+    first->assign(G + 1, 0);
+    for (int i = 0; i < n; i++) (*first)[owner[i] + 1]++;
+    for (int g = 0; g < G; g++) (*first)[g + 1] += (*first)[g];
+    order->assign(n, 0);
+    std::vector<int> pos(first->begin(), first->end() - 1);
+    for (int i : idx) (*order)[pos[owner[i]]++] = i;
 }
 
-// Item costs of the context's volumes cut into z-chunks of `chunk` planes.
-std::vector<long long> chunk_costs(const spg_ctx *ctx, int TX, int TY, int chunk)
+// Makespan of the longest-first schedule (lpt_schedule) of the context's
+// volumes cut into z-chunks of `chunk` planes, over at most `slots` CTAs. Items
+// of one cost are handed out together to CTAs of one load, so the work is the
+// number of distinct loads, not of items (creating a context tries some dozen
+// chunks for each tile).
+long long chunk_makespan(const spg_ctx *ctx, int TX, int TY, int chunk, long long slots)
 {
-    std::vector<long long> c;
+    std::map<long long, long long, std::greater<long long>> items;  // cost -> count
+    long long n = 0;
     for (const auto &d : ctx->vols_h) {
         const long long cols = (long long)((d.nx + TX - 1) / TX) * ((d.ny + TY - 1) / TY);
         const int nzi = d.nz - d.halo_lo - d.halo_hi;  // planes written (halo planes are only read)
         const int nch = (nzi + chunk - 1) / chunk;
         for (int q = 0; q < nch; q++) {
             const int z0 = (int)((long long)nzi * q / nch), z1 = (int)((long long)nzi * (q + 1) / nch);
-            if (z1 > z0) c.insert(c.end(), cols, item_cost(z0, z1));
+            if (z1 <= z0) continue;
+            items[item_cost(z0, z1)] += cols;
+            n += cols;
         }
     }
-    return c;
+    std::map<long long, long long> loads;  // load -> CTAs
+    loads[0] = std::min(n, slots);
+    for (auto [cost, left] : items)
+        while (left > 0) {
+            const auto least = loads.begin();
+            const long long load = least->first, k = std::min(least->second, left);
+            if ((least->second -= k) == 0) loads.erase(least);
+            loads[load + cost] += k;
+            left -= k;
+        }
+    return loads.empty() ? 0 : loads.rbegin()->first;
 }
 
 // Planes per work item for variant v with `slots` resident CTAs: the z-chunk
@@ -388,9 +401,7 @@ int best_chunk(const spg_ctx *ctx, const StepVariant &v, long long slots, long l
             total += (long long)((d.nx + TX - 1) / TX) * ((d.ny + TY - 1) / TY) * (nzi + 2 * ((nzi + c - 1) / c));
         }
         if (best >= 0 && (total + slots - 1) / slots >= best) continue;
-        const auto cost = chunk_costs(ctx, TX, TY, c);
-        const int G = (int)std::min<long long>((long long)cost.size(), slots);
-        const long long ms = lpt_schedule(cost, G, nullptr, nullptr);
+        const long long ms = chunk_makespan(ctx, TX, TY, c, slots);
         if (best < 0 || ms < best) {
             best = ms;
             chunk = c;
@@ -435,12 +446,17 @@ StepVariant default_variant(const spg_ctx *ctx)
         }
         long long steps = 0;
         const long long slots = (long long)ctx->num_sms * occ;
-        if (ctx->opt.zchunk > 0) {
-            const auto cost = chunk_costs(ctx, 32 * c.v.vx, c.v.ty, ctx->opt.zchunk);
-            steps = lpt_schedule(cost, (int)std::min<long long>((long long)cost.size(), slots), nullptr, nullptr);
-        } else {
+        // whole columns are the least work; no schedule is shorter than that
+        // over the resident CTAs
+        long long work = 0;
+        for (const auto &d : ctx->vols_h)
+            work += (long long)((d.nx + 32 * c.v.vx - 1) / (32 * c.v.vx)) * ((d.ny + c.v.ty - 1) / c.v.ty) *
+                    (d.nz - d.halo_lo - d.halo_hi + 2);
+        if (best_us >= 0.0 && (double)(work / slots) * c.step_us >= best_us) continue;
+        if (ctx->opt.zchunk > 0)
+            steps = chunk_makespan(ctx, 32 * c.v.vx, c.v.ty, ctx->opt.zchunk, slots);
+        else
             best_chunk(ctx, c.v, slots, &steps);
-        }
         const double us = (double)steps * c.step_us;
         if (best_us < 0.0 || us < best_us) {
             best_us = us;
@@ -910,13 +926,31 @@ struct Sweep {
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(vol, ctx->vols_d, sizeof(VolDesc), cudaMemcpyDeviceToDevice, ctx->stream);
         if (e != cudaSuccess) return e;
+        // every step shares the maps of omtv, b, w and om1, and the steps' iterates
+        // lie in a few buffers: one map each (at 50 + 95 steps, 1160 encodings
+        // took the host 0.3 ms while the GPU waited; now about 20)
         std::vector<TmapSet> h(plan.size());
+        TmapSet base;
+        float *const none[4] = {nullptr, nullptr, nullptr, nullptr};
+        if ((e = encode_set(ctx, ctx->vols_h[0], v, none, &base)) != cudaSuccess) return e;
+        std::unordered_map<float *, CUtensorMap> xmaps;
+        auto xmap = [&](float *x, CUtensorMap *to) -> cudaError_t {
+            auto it = xmaps.find(x);
+            if (it == xmaps.end()) {
+                CUtensorMap m;
+                cudaError_t err = encode_map(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, x, ctx->vols_h[0], 4,
+                                             32 * v.vx + 8, v.ty + 2);
+                if (err != cudaSuccess) return err;
+                it = xmaps.emplace(x, m).first;
+            }
+            *to = it->second;
+            return cudaSuccess;
+        };
         for (size_t j = 0; j < plan.size(); j++) {
             const int cur = (int)(j % 3);
-            float *xq[4] = {nullptr, nullptr, nullptr, nullptr};
-            xq[cur] = plan[j].xk;
-            xq[(cur + 2) % 3] = plan[j].xkm1;
-            if ((e = encode_set(ctx, ctx->vols_h[0], v, xq, &h[j])) != cudaSuccess) return e;
+            h[j] = base;
+            if ((e = xmap(plan[j].xk, &h[j].x[cur])) != cudaSuccess) return e;
+            if ((e = xmap(plan[j].xkm1, &h[j].x[(cur + 2) % 3])) != cudaSuccess) return e;
         }
         kvals.resize(plan.size());
         std::vector<float *> ho(plan.size());
@@ -1923,11 +1957,13 @@ spg_status spg_backward(spg_ctx *ctx, int K, const float *gx, float *gb, float *
     const VolDesc &d = ctx->vols_h[0];
     const size_t vb = (size_t)ctx->total * 4;
     const int nck = (K + C - 1) / C;  // checkpoints at k = 0, C, 2C, ... (< K)
-    // one forward sweep plus, per segment, the recomputation of all but its last step
-    const size_t nsteps = (size_t)K + (size_t)(K - nck);
+    // one forward sweep up to the last checkpoint plus, per segment, the
+    // recomputation of all but its last step
+    const int Ks = (nck - 1) * C;
+    const size_t nsteps = (size_t)Ks + (size_t)(K - nck);
     // workspace: checkpoints, segment, adjoint volumes, scalar partials, the steps' state
     float *ck = nullptr, *seg = nullptr, *ga[3], *m = nullptr, *accb = nullptr, *accw = nullptr;
-    double *pp = nullptr;
+    double *pp = nullptr, *ps = nullptr;
     const int nblk = adjoint_blocks(d.nx, d.ny, d.nz);  // CTAs of each adjoint pass, one scalar partial each
     Carve cv;
     for (int pass = 0; pass < 2; pass++) {
@@ -1940,6 +1976,7 @@ spg_status spg_backward(spg_ctx *ctx, int K, const float *gx, float *gb, float *
         accb = t.take<float>(vb);
         accw = t.take<float>(vb);
         pp = t.take<double>((size_t)K * nblk * 4 * sizeof(double));
+        ps = t.take<double>((size_t)K * 2 * sizeof(double));  // their sums per step
         if (pass == 0) {
             DevState *s0;
             VolDesc *v0;
@@ -1963,7 +2000,7 @@ spg_status spg_backward(spg_ctx *ctx, int K, const float *gx, float *gb, float *
     for (int q = 0; q < 3; q++) b3[q] = vol_at(seg, q);
     {
         int c = 0;
-        for (int k = 0; k < K; k++) {
+        for (int k = 0; k < Ks; k++) {
             sw.add(b3[c], b3[(c + 2) % 3], b3[(c + 1) % 3], k);
             c = (c + 1) % 3;
         }
@@ -1982,14 +2019,14 @@ spg_status spg_backward(spg_ctx *ctx, int K, const float *gx, float *gb, float *
         CK(cudaMemcpyAsync(b3[0], ctx->X[ctx->cur()], vb, cudaMemcpyDeviceToDevice, ctx->stream), "copy x0");
         CK(cudaMemcpyAsync(b3[2], b3[0], vb, cudaMemcpyDeviceToDevice, ctx->stream), "copy x0");
         int c = 0;
-        for (int k = 0; k < K; k++) {
+        for (int k = 0; k <= Ks; k++) {
             if (k % C == 0) {
                 CK(cudaMemcpyAsync(vol_at(ck, 2 * (k / C)), b3[c], vb, cudaMemcpyDeviceToDevice, ctx->stream), "ckpt");
                 CK(cudaMemcpyAsync(vol_at(ck, 2 * (k / C) + 1), b3[(c + 2) % 3], vb, cudaMemcpyDeviceToDevice,
                                    ctx->stream),
                    "ckpt");
             }
-            if (k % C == 0) CK(sw.launch(std::min(C, K - k)), "fused step");
+            if (k % C == 0 && k < Ks) CK(sw.launch(C), "fused step");
             c = (c + 1) % 3;
         }
     }
@@ -2044,16 +2081,16 @@ spg_status spg_backward(spg_ctx *ctx, int K, const float *gx, float *gb, float *
     }
     if ((s = copy_volume_out(ctx, gb, accb, 4, d)) != SPG_OK) return s;
     if ((s = copy_volume_out(ctx, gw, accw, 4, d)) != SPG_OK) return s;
-    const size_t segs = (size_t)nblk;
-    std::vector<double> hp((size_t)K * segs * 4);
-    CK(cudaMemcpyAsync(hp.data(), pp, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream), "read");
+    CK(launch_adjoint_scalars(pp, nblk, K, ps, ctx->stream), "scalar gradients");
+    ctx->launches += 1;
+    std::vector<double> hp((size_t)K * 2);
+    CK(cudaMemcpyAsync(hp.data(), ps, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream), "read");
     CK(cudaStreamSynchronize(ctx->stream), "synchronise");
     double s1 = 0, s2 = 0;
-    for (int k = K - 1; k >= 0; k--)
-        for (size_t q = 0; q < segs; q++) {
-            s1 += hp[((size_t)k * segs + q) * 4 + 0];
-            s2 += hp[((size_t)k * segs + q) * 4 + 1];
-        }
+    for (int k = K - 1; k >= 0; k--) {
+        s1 += hp[(size_t)k * 2 + 0];
+        s2 += hp[(size_t)k * 2 + 1];
+    }
     g_scalars[0] = s1;
     g_scalars[1] = s2;
     return device_status(ctx);

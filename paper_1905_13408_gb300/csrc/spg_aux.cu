@@ -1134,31 +1134,6 @@ constexpr int THREADS = 32 * (TY + 1); // warp TY: the row below the tile
 constexpr int ZC = 8;                  // planes per CTA
 }  // namespace adj
 
-// f at the lane's voxels of the row whose voxel x0 is element i (zeros where
-// `ok` is false) and at x0-1: from the lane before, loaded by a chunk's first
-// lane, and the voxel's own value at the volume's first column (zero backward
-// difference along x). Every lane of the warp calls it.
-__device__ __forceinline__ void row4(const float *f, const Lane4 &L, long long i, bool ok, float (&c)[4], float &l)
-{
-    unpack4(ldz4(f + i, ok), c);
-    l = __shfl_up_sync(FULL, c[3], 1);
-    if (L.lane == 0) l = (ok && L.x0 >= 1) ? f[i - 1] : c[0];
-    if (L.x0 == 0) l = c[0];
-}
-
-// f on the row whose voxel x0 is element i when `have`, else a copy of c
-// (a missing backward neighbour: the voxel stands in for it).
-__device__ __forceinline__ void row4_or(const float *f, long long i, bool have, bool ok, const float (&c)[4],
-                                        float (&r)[4])
-{
-    if (have) {
-        unpack4(ldz4(f + i, ok), r);
-    } else {
-#pragma unroll
-        for (int q = 0; q < 4; q++) r[q] = c[q];
-    }
-}
-
 // (D y)_a at the lane's 4 voxels (Eq. 12 on y = x_k + beta (x_k - x_{k-1})),
 // differences of x_k and of d = x_k - x_{k-1} taken separately: xc, mc on
 // the voxels' row (xl, ml at x0-1), xu, mu_ on the row below in y, xw, mw on
@@ -1251,63 +1226,103 @@ __device__ __forceinline__ long long adj_row(const VolDesc &V, int x0, int y, in
     return V.off + ((long long)z * V.ny + y) * V.pitch + x0;
 }
 
-__global__ void __launch_bounds__(adj::THREADS) adjoint_mask_kernel(AdjParams a)
+// One field's loads for a plane of the march, issued an iteration before their
+// use: the warp's row, the row above and, for a chunk's first lane, the voxel
+// to the left.
+struct RowLoads {
+    float4 c, u;
+    float l;
+    __device__ __forceinline__ void load(const VolDesc &V, const Lane4 &L, const float *f, long long i, bool ok)
+    {
+        c = ldz4(f + i, ok);
+        u = ldz4(f + i - V.pitch, ok && L.y >= 1);
+        l = (L.lane == 0 && ok && L.x0 >= 1) ? f[i - 1] : 0.f;
+    }
+    // the values, with the voxel itself for a missing neighbour (every lane calls it)
+    __device__ __forceinline__ void take(const Lane4 &L, float (&cc)[4], float &cl, float (&uu)[4]) const
+    {
+        unpack4(c, cc);
+        cl = __shfl_up_sync(FULL, cc[3], 1);
+        if (L.lane == 0) cl = l;
+        if (L.x0 == 0) cl = cc[0];
+        if (L.y >= 1) {
+            unpack4(u, uu);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; q++) uu[q] = cc[q];
+        }
+    }
+};
+
+// Bound (both passes, 128^3): the latency of their loads with the 16 warps an
+// SM holds; 36 + 12 and 24 + 8 bytes a voxel, mostly from L2. The loads of a
+// plane are therefore issued one iteration ahead: the next plane's rows before
+// this plane's barrier, the rest once this plane's are consumed (24.2 -> 19.0 us
+// and 23.5 -> 19.7 us a pass, 125 registers).
+__global__ void __launch_bounds__(adj::THREADS, 2) adjoint_mask_kernel(AdjParams a)
 {
     __shared__ __align__(16) float ring[3][adj::TY + 1][128];  // p_y of the tile's rows and the row below it
-    __shared__ double scratch[32 * 4];
+    __shared__ double scratch[32 * 4 + 16];
     const VolDesc V = a.vols[0];
     AdjPlace P = adj_place(V);
     Lane4 &L = P.L;
     const float beta = a.beta, mu = V.mu;
+    const bool writes = P.r < adj::TY && P.row_in;
     KSum k1, k2;
     // x_k, x_{k-1} on the warp's row of the current plane, and p there
-    float xc[4], mc[4], xl, ml, pc[3][4];
-    {
-        const int z = P.z0;
-        L.z = z;
-        L.i = P.row_in ? adj_row(V, L.x0, L.y, z) : 0;
-        float xu[4], mu_[4], xw[4], mw[4], ot[4], g[3][4];
-        row4(a.xk, L, L.i, L.act, xc, xl);
-        row4(a.xkm1, L, L.i, L.act, mc, ml);
-        row4_or(a.xk, L.i - V.pitch, L.y >= 1, L.act, xc, xu);
-        row4_or(a.xkm1, L.i - V.pitch, L.y >= 1, L.act, mc, mu_);
-        row4_or(a.xk, L.i - P.PS, z >= 1, L.act, xc, xw);
-        row4_or(a.xkm1, L.i - P.PS, z >= 1, L.act, mc, mw);
-        unpack4(ldz4(a.omtv + L.i, L.act), ot);
-        dy4(xc, mc, xl, ml, xu, mu_, xw, mw, beta, g);
+    float xc[4], mc[4], pc[3][4];
+    RowLoads rx, rm;
+    float4 rot, fb, fw, f1, fg, fgb, fgw;  // omtv of the next plane; b, w, om1, gnext, gb, gw of this one
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto load_rows = [&](long long i, bool ok) {
+        rx.load(V, L, a.xk, i, ok);
+        rm.load(V, L, a.xkm1, i, ok);
+        rot = ldz4(a.omtv + i, ok);
+    };
+    auto load_rest = [&](long long i, bool ok) {
+        fb = ok ? ld4_data(a.b, a.bf16, i) : zero;
+        fw = ok ? ld4_data(a.w, a.bf16, i) : zero;
+        f1 = ldz4(a.om1 + i, ok);
+        fg = ldz4(a.gnext + i, ok);
+        fgb = ldz4(a.gb + i, ok);
+        fgw = ldz4(a.gw + i, ok);
+    };
+    // p at the loaded rows' plane z, the plane below in (xw, mw); into the ring
+    auto p_rows = [&](const float (&xw)[4], const float (&mw)[4], bool have, bool ok, int z, float (&xn)[4],
+                      float (&mn)[4], float (&pn)[3][4]) {
+        float xu[4], mu_[4], ot[4], g[3][4], xl, ml;
+        rx.take(L, xn, xl, xu);
+        rm.take(L, mn, ml, mu_);
+        unpack4(rot, ot);
+        if (have)
+            dy4(xn, mn, xl, ml, xu, mu_, xw, mw, beta, g);
+        else
+            dy4(xn, mn, xl, ml, xu, mu_, xn, mn, beta, g);
 #pragma unroll
         for (int q = 0; q < 4; q++) {
-            const bool valid = L.act && L.x0 + q < V.nx;
+            const bool valid = ok && L.x0 + q < V.nx;
             const float sc = p_scale(g[0][q], g[1][q], g[2][q], ot[q], mu);
 #pragma unroll
-            for (int c = 0; c < 3; c++) pc[c][q] = valid ? g[c][q] * sc : 0.f;
+            for (int c = 0; c < 3; c++) pn[c][q] = valid ? g[c][q] * sc : 0.f;
         }
-        *reinterpret_cast<float4 *>(&ring[z % 3][P.r][4 * L.lane]) = make_float4(pc[1][0], pc[1][1], pc[1][2], pc[1][3]);
+        *reinterpret_cast<float4 *>(&ring[z % 3][P.r][4 * L.lane]) = make_float4(pn[1][0], pn[1][1], pn[1][2], pn[1][3]);
+    };
+    L.i = P.row_in ? adj_row(V, L.x0, L.y, P.z0) : 0;
+    {
+        float xw[4], mw[4];
+        load_rows(L.i, L.act);
+        unpack4(ldz4(a.xk + L.i - P.PS, L.act && P.z0 >= 1), xw);
+        unpack4(ldz4(a.xkm1 + L.i - P.PS, L.act && P.z0 >= 1), mw);
+        load_rest(L.i, L.act && writes);
+        p_rows(xw, mw, P.z0 >= 1, L.act, P.z0, xc, mc, pc);
+        load_rows(L.i + P.PS, L.act && P.z0 + 1 < V.nz);
     }
     for (int z = P.z0; z < P.z1; z++) {
         // p on the next plane (zero beyond the volume)
-        const bool zn = z + 1 < V.nz;
-        const bool okn = L.act && zn;
         const long long in_ = L.i + P.PS;
-        float xn[4], mn[4], xnl, mnl, pn[3][4];
-        {
-            float xu[4], mu_[4], ot[4], g[3][4];
-            row4(a.xk, L, in_, okn, xn, xnl);
-            row4(a.xkm1, L, in_, okn, mn, mnl);
-            row4_or(a.xk, in_ - V.pitch, L.y >= 1, okn, xn, xu);
-            row4_or(a.xkm1, in_ - V.pitch, L.y >= 1, okn, mn, mu_);
-            unpack4(ldz4(a.omtv + in_, okn), ot);
-            dy4(xn, mn, xnl, mnl, xu, mu_, xc, mc, beta, g);
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const bool valid = okn && L.x0 + q < V.nx;
-                const float sc = p_scale(g[0][q], g[1][q], g[2][q], ot[q], mu);
-#pragma unroll
-                for (int c = 0; c < 3; c++) pn[c][q] = valid ? g[c][q] * sc : 0.f;
-            }
-            *reinterpret_cast<float4 *>(&ring[(z + 1) % 3][P.r][4 * L.lane]) =
-                make_float4(pn[1][0], pn[1][1], pn[1][2], pn[1][3]);
-        }
+        float xn[4], mn[4], pn[3][4];
+        p_rows(xc, mc, true, L.act && z + 1 < V.nz, z + 1, xn, mn, pn);
+        load_rows(in_ + P.PS, L.act && z + 1 < P.z1 && z + 2 < V.nz);
         __syncthreads();  // p_y of plane z of every row of the tile is in the ring
         // p_x at x+1: the next lane's first voxel; a chunk's last lane evaluates it
         float pxn = __shfl_down_sync(FULL, pc[0][0], 1);
@@ -1323,7 +1338,7 @@ __global__ void __launch_bounds__(adj::THREADS) adjoint_mask_kernel(AdjParams a)
                 pxn = ga[0] * p_scale(ga[0], ga[1], ga[2], a.omtv[j], mu);
             }
         }
-        if (P.r < adj::TY && P.row_in) {
+        if (writes) {
             float px[4] = {pc[0][1], pc[0][2], pc[0][3], pxn};
 #pragma unroll
             for (int q = 0; q < 4; q++)
@@ -1331,13 +1346,13 @@ __global__ void __launch_bounds__(adj::THREADS) adjoint_mask_kernel(AdjParams a)
             const float4 pyv = *reinterpret_cast<const float4 *>(&ring[z % 3][P.r + 1][4 * L.lane]);
             const float py[4] = {pyv.x, pyv.y, pyv.z, pyv.w};  // zero when row y + 1 is outside
             float bv[4], wv[4], o1[4], gn[4], gb[4], gw[4], m[4];
-            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-            unpack4(L.act ? ld4_data(a.b, a.bf16, L.i) : zero, bv);
-            unpack4(L.act ? ld4_data(a.w, a.bf16, L.i) : zero, wv);
-            unpack4(ldz4(a.om1 + L.i, L.act), o1);
-            unpack4(ldz4(a.gnext + L.i, L.act), gn);
-            unpack4(ldz4(a.gb + L.i, L.act), gb);
-            unpack4(ldz4(a.gw + L.i, L.act), gw);
+            unpack4(fb, bv);
+            unpack4(fw, wv);
+            unpack4(f1, o1);
+            unpack4(fg, gn);
+            unpack4(fgb, gb);
+            unpack4(fgw, gw);
+            load_rest(in_, L.act && z + 1 < P.z1);
             float s1 = 0.f, s2 = 0.f;
 #pragma unroll
             for (int q = 0; q < 4; q++) {
@@ -1372,16 +1387,11 @@ __global__ void __launch_bounds__(adj::THREADS) adjoint_mask_kernel(AdjParams a)
 #pragma unroll
             for (int c = 0; c < 3; c++) pc[c][q] = pn[c][q];
         }
-        xl = xnl;
-        ml = mnl;
         L.i = in_;
     }
-    double sm[2] = {k1.value(), k2.value()};
-    block_sum<2>(sm, scratch);
-    if (threadIdx.x == 0) {
-        a.plane_part[(long long)blockIdx.x * 4 + 0] = sm[0];
-        a.plane_part[(long long)blockIdx.x * 4 + 1] = sm[1];
-    }
+    const ff::FF fv[4] = {k1.pair(), k2.pair(), {0.f, 0.f}, {0.f, 0.f}};
+    const double sm = block_sum4(fv, scratch);
+    if (threadIdx.x < 2) a.plane_part[(long long)blockIdx.x * 4 + threadIdx.x] = sm;
 }
 
 // hq at the lane's 4 voxels from D y and D m there (zero where !ok or beyond nx)
@@ -1399,53 +1409,64 @@ __device__ __forceinline__ void hq4(const float (&g)[3][4], const float (&qc)[4]
     }
 }
 
-__global__ void __launch_bounds__(adj::THREADS) adjoint_apply_kernel(AdjParams a)
+__global__ void __launch_bounds__(adj::THREADS, 2) adjoint_apply_kernel(AdjParams a)
 {
     __shared__ __align__(16) float ring[3][adj::TY + 1][128];  // hq_y of the tile's rows and the row below it
     const VolDesc V = a.vols[0];
     AdjPlace P = adj_place(V);
     Lane4 &L = P.L;
     const float beta = a.beta, mu = V.mu;
+    const bool writes = P.r < adj::TY && P.row_in;
+    const bool alias = a.gprev == a.gcur;  // k = 0: x_{-1} = x_0
     // x_k, x_{k-1} and m on the warp's row of the current plane, and hq there
-    float xc[4], mc[4], qc[4], xl, ml, ql, hc[3][4];
+    float xc[4], mc[4], qc[4], hc[3][4];
+    RowLoads rx, rm, rq;
+    float4 rot, fw, fgc, fgp;  // omtv of the next plane; w, gcur, gprev of this one
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto load_rows = [&](long long i, bool ok) {
+        rx.load(V, L, a.xk, i, ok);
+        rm.load(V, L, a.xkm1, i, ok);
+        rq.load(V, L, a.m, i, ok);
+        rot = ldz4(a.omtv + i, ok);
+    };
+    auto load_rest = [&](long long i, bool ok) {
+        fw = ok ? ld4_data(a.w, a.bf16, i) : zero;
+        fgc = ldz4(a.gcur + i, ok);
+        fgp = ldz4(a.gprev + i, ok && !alias && !a.prev_fresh);
+    };
+    auto h_rows = [&](const float (&xw)[4], const float (&mw)[4], const float (&qw)[4], bool have, bool ok, int z,
+                      float (&xn)[4], float (&mn)[4], float (&qn)[4], float (&hn)[3][4]) {
+        float xu[4], mu_[4], qu[4], ot[4], g[3][4], xl, ml, ql;
+        rx.take(L, xn, xl, xu);
+        rm.take(L, mn, ml, mu_);
+        rq.take(L, qn, ql, qu);
+        unpack4(rot, ot);
+        if (have) {
+            dy4(xn, mn, xl, ml, xu, mu_, xw, mw, beta, g);
+            hq4(g, qn, ql, qu, qw, ot, mu, ok, L.x0, V.nx, hn);
+        } else {
+            dy4(xn, mn, xl, ml, xu, mu_, xn, mn, beta, g);
+            hq4(g, qn, ql, qu, qn, ot, mu, ok, L.x0, V.nx, hn);
+        }
+        *reinterpret_cast<float4 *>(&ring[z % 3][P.r][4 * L.lane]) = make_float4(hn[1][0], hn[1][1], hn[1][2], hn[1][3]);
+    };
+    L.i = P.row_in ? adj_row(V, L.x0, L.y, P.z0) : 0;
     {
-        const int z = P.z0;
-        L.z = z;
-        L.i = P.row_in ? adj_row(V, L.x0, L.y, z) : 0;
-        float xu[4], mu_[4], qu[4], xw[4], mw[4], qw[4], ot[4], g[3][4];
-        row4(a.xk, L, L.i, L.act, xc, xl);
-        row4(a.xkm1, L, L.i, L.act, mc, ml);
-        row4(a.m, L, L.i, L.act, qc, ql);
-        row4_or(a.xk, L.i - V.pitch, L.y >= 1, L.act, xc, xu);
-        row4_or(a.xkm1, L.i - V.pitch, L.y >= 1, L.act, mc, mu_);
-        row4_or(a.m, L.i - V.pitch, L.y >= 1, L.act, qc, qu);
-        row4_or(a.xk, L.i - P.PS, z >= 1, L.act, xc, xw);
-        row4_or(a.xkm1, L.i - P.PS, z >= 1, L.act, mc, mw);
-        row4_or(a.m, L.i - P.PS, z >= 1, L.act, qc, qw);
-        unpack4(ldz4(a.omtv + L.i, L.act), ot);
-        dy4(xc, mc, xl, ml, xu, mu_, xw, mw, beta, g);
-        hq4(g, qc, ql, qu, qw, ot, mu, L.act, L.x0, V.nx, hc);
-        *reinterpret_cast<float4 *>(&ring[z % 3][P.r][4 * L.lane]) = make_float4(hc[1][0], hc[1][1], hc[1][2], hc[1][3]);
+        float xw[4], mw[4], qw[4];
+        const bool below = L.act && P.z0 >= 1;
+        load_rows(L.i, L.act);
+        unpack4(ldz4(a.xk + L.i - P.PS, below), xw);
+        unpack4(ldz4(a.xkm1 + L.i - P.PS, below), mw);
+        unpack4(ldz4(a.m + L.i - P.PS, below), qw);
+        load_rest(L.i, L.act && writes);
+        h_rows(xw, mw, qw, P.z0 >= 1, L.act, P.z0, xc, mc, qc, hc);
+        load_rows(L.i + P.PS, L.act && P.z0 + 1 < V.nz);
     }
     for (int z = P.z0; z < P.z1; z++) {
-        const bool zn = z + 1 < V.nz;
-        const bool okn = L.act && zn;
         const long long in_ = L.i + P.PS;
-        float xn[4], mn[4], qn[4], xnl, mnl, qnl, hn[3][4];
-        {
-            float xu[4], mu_[4], qu[4], ot[4], g[3][4];
-            row4(a.xk, L, in_, okn, xn, xnl);
-            row4(a.xkm1, L, in_, okn, mn, mnl);
-            row4(a.m, L, in_, okn, qn, qnl);
-            row4_or(a.xk, in_ - V.pitch, L.y >= 1, okn, xn, xu);
-            row4_or(a.xkm1, in_ - V.pitch, L.y >= 1, okn, mn, mu_);
-            row4_or(a.m, in_ - V.pitch, L.y >= 1, okn, qn, qu);
-            unpack4(ldz4(a.omtv + in_, okn), ot);
-            dy4(xn, mn, xnl, mnl, xu, mu_, xc, mc, beta, g);
-            hq4(g, qn, qnl, qu, qc, ot, mu, okn, L.x0, V.nx, hn);
-            *reinterpret_cast<float4 *>(&ring[(z + 1) % 3][P.r][4 * L.lane]) =
-                make_float4(hn[1][0], hn[1][1], hn[1][2], hn[1][3]);
-        }
+        float xn[4], mn[4], qn[4], hn[3][4];
+        h_rows(xc, mc, qc, true, L.act && z + 1 < V.nz, z + 1, xn, mn, qn, hn);
+        load_rows(in_ + P.PS, L.act && z + 1 < P.z1 && z + 2 < V.nz);
         __syncthreads();  // hq_y of plane z of every row of the tile is in the ring
         // hq_x at x+1: the next lane's first voxel; a chunk's last lane evaluates it
         float hxn = __shfl_down_sync(FULL, hc[0][0], 1);
@@ -1465,19 +1486,18 @@ __global__ void __launch_bounds__(adj::THREADS) adjoint_apply_kernel(AdjParams a
                 hxn = h[0];
             }
         }
-        if (P.r < adj::TY && P.row_in) {
+        if (writes) {
             float hx[4] = {hc[0][1], hc[0][2], hc[0][3], hxn};
 #pragma unroll
             for (int q = 0; q < 4; q++)
                 if (L.x0 + q + 1 >= V.nx) hx[q] = 0.f;
             const float4 hyv = *reinterpret_cast<const float4 *>(&ring[z % 3][P.r + 1][4 * L.lane]);
             const float hy[4] = {hyv.x, hyv.y, hyv.z, hyv.w};
-            float wv[4], gc[4], gp[4] = {0.f, 0.f, 0.f, 0.f};
-            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-            unpack4(L.act ? ld4_data(a.w, a.bf16, L.i) : zero, wv);
-            unpack4(ldz4(a.gcur + L.i, L.act), gc);
-            const bool alias = a.gprev == a.gcur;  // k = 0: x_{-1} = x_0
-            if (!alias && !a.prev_fresh) unpack4(ldz4(a.gprev + L.i, L.act), gp);
+            float wv[4], gc[4], gp[4];
+            unpack4(fw, wv);
+            unpack4(fgc, gc);
+            unpack4(fgp, gp);
+            load_rest(in_, L.act && z + 1 < P.z1);
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const bool valid = L.act && L.x0 + q < V.nx;
@@ -1501,10 +1521,25 @@ __global__ void __launch_bounds__(adj::THREADS) adjoint_apply_kernel(AdjParams a
 #pragma unroll
             for (int c = 0; c < 3; c++) hc[c][q] = hn[c][q];
         }
-        xl = xnl;
-        ml = mnl;
-        ql = qnl;
         L.i = in_;
+    }
+}
+
+// One CTA per step: its CTAs' scalar partials, summed in a fixed order (the
+// host read and summed all of them: 0.5 MB at 128^3 and 50 steps).
+__global__ void adjoint_scalars_kernel(const double *part, int nblk, double *out)
+{
+    __shared__ double scratch[32 * 2];
+    const double *p = part + (long long)blockIdx.x * nblk * 4;
+    double v[2] = {0.0, 0.0};
+    for (int q = threadIdx.x; q < nblk; q += blockDim.x) {
+        v[0] += p[(long long)q * 4 + 0];
+        v[1] += p[(long long)q * 4 + 1];
+    }
+    block_sum<2>(v, scratch);
+    if (threadIdx.x == 0) {
+        out[blockIdx.x * 2 + 0] = v[0];
+        out[blockIdx.x * 2 + 1] = v[1];
     }
 }
 
@@ -1775,6 +1810,12 @@ cudaError_t launch_generic_step(const GenericParams &g, cudaStream_t s)
 cudaError_t launch_adjoint_mask(const AdjParams &a, cudaStream_t s)
 {
     adjoint_mask_kernel<<<a.nblocks, adj::THREADS, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adjoint_scalars(const double *part, int nblk, int K, double *out, cudaStream_t s)
+{
+    adjoint_scalars_kernel<<<K, 128, 0, s>>>(part, nblk, out);
     return cudaGetLastError();
 }
 

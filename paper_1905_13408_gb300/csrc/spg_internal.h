@@ -163,6 +163,8 @@ struct AdjParams {
 // (H_mu D m and ybar). Each is one kernel of adjoint_blocks(...) CTAs.
 int adjoint_blocks(int nx, int ny, int nz);
 cudaError_t launch_adjoint_mask(const AdjParams &a, cudaStream_t s);
+// out[k] = {sum of [0], sum of [1]} of the nblk partials of step k, k < K.
+cudaError_t launch_adjoint_scalars(const double *part, int nblk, int K, double *out, cudaStream_t s);
 cudaError_t launch_adjoint_apply(const AdjParams &a, cudaStream_t s);
 cudaError_t launch_timeout_probe(DevState *st, long long timeout_ns, cudaStream_t s);
 // One iteration under alternative readings (VolDesc.readings != 0): the fused
