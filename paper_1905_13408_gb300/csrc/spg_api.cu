@@ -30,6 +30,7 @@ namespace {
 thread_local std::string g_last_error = "no error";
 
 constexpr long long kTimeoutNs = 2000000000LL;  // 2 s bound on any device-side wait
+constexpr size_t kStateBytes = (sizeof(DevState) + 63) / 64 * 64;
 constexpr int kGraphLen = 10;                   // iterations per captured graph (Fourier-domain term, plain steps)
 // Bounds on the iterations of one fused launch: the partial sums it keeps
 // (32 bytes per work item and iteration) and roughly how long it may hold the
@@ -94,7 +95,7 @@ struct spg_ctx {
     double *plane_part_d = nullptr;
     WorkItem *aux_items_d = nullptr;  // march items of the auxiliary passes
     int naux = 0;
-    double *vol_out_d = nullptr;
+    double *vol_out_d = nullptr;  // behind st_d, same allocation
     double *maxw_d = nullptr;
     double *rstats_d = nullptr;
 
@@ -211,7 +212,7 @@ void free_all(spg_ctx *c)
         if (p) cudaFree(p);
     void *ps[] = {c->vols_d, c->items_d, c->sched_d, c->tmaps_d, c->plane_vol_d, c->X[0], c->X[1], c->X[2], c->X[3], c->B, c->W,
                   c->OM1, c->OMTV, c->beta_d, c->st_d, c->partials_d, c->hist_d, c->plane_part_d, c->aux_items_d,
-                  c->vol_out_d, c->maxw_d, c->rstats_d};
+                  c->maxw_d, c->rstats_d};
     for (void *p : ps)
         if (p) cudaFree(p);
     if (c->ws) cudaFree(c->ws);
@@ -610,12 +611,9 @@ AuxParams aux_params(const spg_ctx *c)
     return a;
 }
 
-// Read the device error word (synchronises); returns and clears it.
-spg_status device_status(spg_ctx *ctx)
+// The device's error word as a status; clears it.
+spg_status status_of(spg_ctx *ctx, const DevState &st)
 {
-    DevState st;
-    CK(cudaMemcpyAsync(&st, ctx->st_d, sizeof(st), cudaMemcpyDeviceToHost, ctx->stream), "read state");
-    CK(cudaStreamSynchronize(ctx->stream), "synchronise");
     if (st.err != 0) {
         int zero = 0;
         cudaMemcpyAsync(&ctx->st_d->err, &zero, sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
@@ -631,6 +629,36 @@ spg_status device_status(spg_ctx *ctx)
         return fail(ctx, (spg_status)st.err, "device error");
     }
     return SPG_OK;
+}
+
+// Read the device error word (synchronises); returns and clears it.
+spg_status device_status(spg_ctx *ctx)
+{
+    DevState st;
+    CK(cudaMemcpyAsync(&st, ctx->st_d, sizeof(st), cudaMemcpyDeviceToHost, ctx->stream), "read state");
+    CK(cudaStreamSynchronize(ctx->stream), "synchronise");
+    return status_of(ctx, st);
+}
+
+// Volume `vol`'s results and the error word (synchronises): one copy where
+// the volumes before it are few, else two.
+spg_status read_results(spg_ctx *ctx, int vol, double o[8])
+{
+    constexpr int kFew = 64;
+    if (vol >= kFew) {
+        CK(cudaMemcpyAsync(o, ctx->vol_out_d + (size_t)vol * 8, 8 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream),
+           "read results");
+        return device_status(ctx);
+    }
+    alignas(16) char buf[kStateBytes + kFew * 8 * sizeof(double)];
+    CK(cudaMemcpyAsync(buf, ctx->st_d, kStateBytes + (size_t)(vol + 1) * 8 * sizeof(double), cudaMemcpyDeviceToHost,
+                       ctx->stream),
+       "read results");
+    CK(cudaStreamSynchronize(ctx->stream), "synchronise");
+    DevState st;
+    std::memcpy(&st, buf, sizeof(st));
+    std::memcpy(o, buf + kStateBytes + (size_t)vol * 8 * sizeof(double), 8 * sizeof(double));
+    return status_of(ctx, st);
 }
 
 bool params_ok(const spg_volume_params &p)
@@ -1132,13 +1160,15 @@ spg_status spg_create_batch(int nvol, const spg_volume_params *params, const spg
     if ((e = dalloc(&ctx->OM1, vb)) != cudaSuccess) return bail(e, "alloc om1");
     if ((e = dalloc(&ctx->OMTV, vb)) != cudaSuccess) return bail(e, "alloc omtv");
     if ((e = dalloc(&ctx->beta_d, ctx->max_iters * sizeof(float))) != cudaSuccess) return bail(e, "alloc beta");
-    if ((e = dalloc(&ctx->st_d, sizeof(DevState))) != cudaSuccess) return bail(e, "alloc state");
+    // state and per-volume results side by side: one copy reads both
+    if ((e = dalloc(&ctx->st_d, kStateBytes + (size_t)nvol * 8 * sizeof(double))) != cudaSuccess)
+        return bail(e, "alloc state");
+    ctx->vol_out_d = reinterpret_cast<double *>(reinterpret_cast<char *>(ctx->st_d) + kStateBytes);
     if ((e = dalloc(&ctx->hist_d, (size_t)ctx->hist_cap * nvol * 5 * sizeof(double))) != cudaSuccess)
         return bail(e, "alloc history");
     if ((e = dalloc(&ctx->plane_part_d, (size_t)nparts * 4 * sizeof(double))) != cudaSuccess)
         return bail(e, "alloc partials");
     if ((e = dalloc(&ctx->aux_items_d, aux.size() * sizeof(WorkItem))) != cudaSuccess) return bail(e, "alloc items");
-    if ((e = dalloc(&ctx->vol_out_d, (size_t)nvol * 8 * sizeof(double))) != cudaSuccess) return bail(e, "alloc");
     if ((e = dalloc(&ctx->maxw_d, (size_t)nvol * sizeof(double))) != cudaSuccess) return bail(e, "alloc");
     if ((e = dalloc(&ctx->rstats_d, (size_t)nvol * 6 * sizeof(double))) != cudaSuccess) return bail(e, "alloc");
 
@@ -1458,9 +1488,7 @@ spg_status spg_param_scales(spg_ctx *ctx, int vol, double out[4])
     CK(launch_scales(aux_params(ctx), vol, d.nz, ctx->B, ctx->W, ctx->bf16(), ctx->stream), "scales");
     ctx->launches += 1;
     double o[8];
-    CK(cudaMemcpyAsync(o, ctx->vol_out_d + (size_t)vol * 8, sizeof(o), cudaMemcpyDeviceToHost, ctx->stream),
-       "read scales");
-    spg_status s = device_status(ctx);
+    const spg_status s = read_results(ctx, vol, o);
     if (s != SPG_OK) return s;
     for (int q = 0; q < 4; q++) out[q] = o[q];
     return SPG_OK;
@@ -1478,10 +1506,8 @@ spg_status spg_set_x(spg_ctx *ctx, int vol, const float *x)
     if ((s = copy_volume_in(ctx, ctx->X[c], 4, d, x)) != SPG_OK) return s;
     {
         // the extrapolation restarts from this iterate
-        const int zero = 0;
-        CK(cudaMemcpyAsync(&ctx->vols_d[vol].kmom, &zero, sizeof(int), cudaMemcpyHostToDevice, ctx->stream),
-           "reset extrapolation");
-        CK(cudaStreamSynchronize(ctx->stream), "synchronise");
+        CK(cudaMemsetAsync(&ctx->vols_d[vol].kmom, 0, sizeof(int), ctx->stream), "reset extrapolation");
+        CK(cudaStreamSynchronize(ctx->stream), "synchronise");  // the caller's array is read
     }
     if (ctx->xd()) {
         CK(cudaMemsetAsync(ctx->X[ctx->aux_of(c)] + d.off, 0, (size_t)d.pitch * d.ny * d.nz * 4, ctx->stream),
@@ -1543,9 +1569,12 @@ spg_status spg_objective(spg_ctx *ctx, int vol, double out[4])
        "objective");
     ctx->launches += 1;
     double o[8];
-    CK(cudaMemcpyAsync(o, ctx->vol_out_d + (size_t)vol * 8, sizeof(o), cudaMemcpyDeviceToHost, ctx->stream),
-       "read objective");
-    if (ctx->fourier) {
+    spg_status s = SPG_OK;
+    if (!ctx->fourier) {
+        s = read_results(ctx, vol, o);
+    } else {
+        CK(cudaMemcpyAsync(o, ctx->vol_out_d + (size_t)vol * 8, sizeof(o), cudaMemcpyDeviceToHost, ctx->stream),
+           "read objective");
         // data term 1/2 |y - D A x|^2 from the spectrum of x
         const VolDesc &d = ctx->vols_h[0];
         const double V = (double)d.nx * d.ny * d.nz;
@@ -1579,8 +1608,8 @@ spg_status spg_objective(spg_ctx *ctx, int vol, double out[4])
             o[0] += (double)ctx->gamma_f * sq;
         }
         o[3] = o[0] + o[1] + o[2];
+        s = device_status(ctx);
     }
-    spg_status s = device_status(ctx);
     if (s != SPG_OK) return s;
     for (int q = 0; q < 4; q++) out[q] = o[q];
     if (!std::isfinite(o[3])) return fail(ctx, SPG_ENONFINITE, "non-finite objective");
@@ -1768,9 +1797,7 @@ spg_status spg_certificate(spg_ctx *ctx, int vol, double *out)
        "certificate");
     ctx->launches += 2;
     double o[8];
-    CK(cudaMemcpyAsync(o, ctx->vol_out_d + (size_t)vol * 8, sizeof(o), cudaMemcpyDeviceToHost, ctx->stream),
-       "read certificate");
-    spg_status s = device_status(ctx);
+    const spg_status s = read_results(ctx, vol, o);
     if (s != SPG_OK) return s;
     *out = o[4];
     return SPG_OK;
