@@ -422,7 +422,7 @@ cudaError_t resident_ctas(const spg_ctx *ctx, const StepVariant &v, int *occ)
 // Built-in tile choice: the variant with the shortest makespan times its time
 // per plane step. Measured on volumes that stay in L2 (every resident CTA
 // marching; iteration time less the 3.2-3.5 us an iteration takes whatever its
-// steps): 128x7 with 4 copy stages 1.05 us a step, 64x7 0.80, 64x4 0.77. A
+// steps): 128x7 with 4 copy stages 1.05 us a step, 64x7 and 64x4 0.80. A
 // 128-wide step costs far less than two 64-wide ones, so the wide tile is the
 // better one as soon as a row is longer than 64, however much of its last
 // tile lies outside: 128x7 against 64-wide tiles, iterations with the objective:
@@ -436,7 +436,7 @@ StepVariant default_variant(const spg_ctx *ctx)
         double step_us;
     };
     const bool bf16 = ctx->bf16(), xd = ctx->xd();
-    const Choice choices[] = {{{4, 7, 4, bf16, xd}, 1.05}, {{2, 7, 4, bf16, xd}, 0.80}, {{2, 4, 4, bf16, xd}, 0.77}};
+    const Choice choices[] = {{{4, 7, 4, bf16, xd}, 1.05}, {{2, 7, 4, bf16, xd}, 0.80}, {{2, 4, 4, bf16, xd}, 0.80}};
     StepVariant best = choices[0].v;
     double best_us = -1.0;
     for (const Choice &c : choices) {

@@ -41,16 +41,20 @@
 // small volume, launch latency, a chain of five dependent loads (device state,
 // schedule, item, descriptor, extrapolation weight) before the first copy
 // could start, and the last CTA's objective sums and state update before the
-// next launch could read the state. Here schedule and descriptors are read
-// once, the extrapolation index is counted, and the objective partials of
+// next launch could read the state. Here the schedule's items are held in
+// shared memory, the extrapolation index is counted, and the objective partials of
 // every iteration are kept ([niter][nitems]) and reduced after the last one
 // by all CTAs together (a warp per iteration and volume). The copies of an
 // item's first planes are issued while the previous item's last ones are
-// computed. An iteration with the objective, one per launch (replayed from a
-// graph) -> this form: 28 x 32 x 40 9.7 -> 5.4 us, 64^3 11.3 -> 7.2,
-// 128^3 18.6 -> 14.0, 101 x 147 x 183 30.7 -> 24.4, 180^3 57.6 -> 47.9,
-// 256^3 86.8 -> 81.2, 512^3 618.4 -> 617.7; a batch of 24 volumes of 96^3 ..
-// 256^3 995 -> 992. (With the producer's position in shared memory instead of
+// computed, and of an iteration's first planes those that no iteration writes
+// before the barrier. An iteration with the objective, one per launch
+// (replayed from a graph) -> many per launch -> items in shared memory (the
+// barrier drops L1, and the chain schedule, item, descriptor from L2 delayed
+// the first copies) and copies before the barrier, same tiles for the last two:
+// 28 x 32 x 40 9.7 -> 5.4 -> 5.1 us, 64^3 11.3 -> 7.6 -> 7.0, 128^3 18.6 -> 14.1
+// -> 13.5, 101 x 147 x 183 30.7 -> 20.8 -> 20.0, 180^3 57.6 -> 43.3 -> 41.3,
+// 256^3 86.8 -> 81.5 -> 79.7, 512^3 618.4 -> 617.2 -> 614.1; 24 volumes of 96^3 ..
+// 256^3 777 -> 767. (With the producer's position in shared memory instead of
 // the item's registers the long marches lost: 623.6 at 512^3, 1128 for the
 // batch: its warp is the last to arrive at every plane's barrier.)
 #pragma once
@@ -64,6 +68,7 @@ namespace spg {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
+constexpr int kItemCache = 16;  // work items of a CTA held in its shared memory
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
@@ -417,7 +422,8 @@ struct Cfg {
     static constexpr int OFF_BAR = OFF_RED + 32 * 4 * 8;      // S mbarriers
     static constexpr int OFF_ST = OFF_BAR + al(S * 8);        // state snapshot
     static constexpr int OFF_KM = OFF_ST + 128;               // extrapolation index per item (restart)
-    static constexpr int TOTAL = OFF_KM + kMaxCtaItems * 4 + 128;  // + alignment slack
+    static constexpr int OFF_IT = OFF_KM + kMaxCtaItems * 4;  // the CTA's first items
+    static constexpr int TOTAL = OFF_IT + kItemCache * (int)sizeof(WorkItem) + 128;  // + alignment slack
     static_assert(sizeof(StateSnap) <= 64 && sizeof(WorkItem) <= 64, "state snapshot and next item share 128 bytes");
     static constexpr int THREADS = 32 * (TY + 1);
     static_assert(TY + 1 <= 32, "reduction scratch sized for at most 32 warps");
@@ -427,10 +433,12 @@ struct Cfg {
 // Producer (one thread): stage contents for step j of work item W, i.e.
 // plane z = z0-1+j of x_k (buffer ia) and of x_{k-1} or d_k (buffer ib), both
 // with halo, and of omtv, and plane z-1 of b, w and om1. Steps 0 and 1 skip
-// what they do not consume.
+// what they do not consume. In two parts: what no iteration writes, with the
+// stage's byte count (it can be fetched before the iterate is final), and the
+// iterate.
 template <class C, int S, bool LOADW>
-__device__ __forceinline__ void issue_stage(unsigned char *sm, uint64_t *bars, const TmapSet *tm,
-                                            const WorkItem &W, int ia, int ib, unsigned gstep, int j)
+__device__ __forceinline__ void issue_fixed(unsigned char *sm, uint64_t *bars, const TmapSet *tm, const WorkItem &W,
+                                            unsigned gstep, int j)
 {
     const int s = (int)((gstep + (unsigned)j) % S);
     unsigned char *base = sm + s * C::STAGE;
@@ -439,14 +447,23 @@ __device__ __forceinline__ void issue_stage(unsigned char *sm, uint64_t *bars, c
     const uint32_t bytes = 2 * C::XT_BYTES + (need_om ? C::OM_BYTES : 0) +
                            (need_bwo ? (LOADW ? 2 : 1) * C::BW_BYTES + C::O1_BYTES : 0);
     mbar_arrive_expect_tx(&bars[s], bytes);
-    tma_load_3d(base + C::OFF_XK, &tm->x[ia], W.x0 - 4, W.y0 - 1, z, &bars[s]);
-    tma_load_3d(base + C::OFF_XM, &tm->x[ib], W.x0 - 4, W.y0 - 1, z, &bars[s]);
     if (need_om) tma_load_3d(base + C::OFF_OM, &tm->omtv, W.x0, W.y0, z, &bars[s]);
     if (need_bwo) {
         tma_load_3d(base + C::OFF_B, &tm->b, W.x0, W.y0, z - 1, &bars[s]);
         if (LOADW) tma_load_3d(base + C::OFF_W, &tm->w, W.x0, W.y0, z - 1, &bars[s]);
         tma_load_3d(base + C::OFF_O1, &tm->om1, W.x0, W.y0, z - 1, &bars[s]);
     }
+}
+
+template <class C, int S>
+__device__ __forceinline__ void issue_iterate(unsigned char *sm, uint64_t *bars, const TmapSet *tm, const WorkItem &W,
+                                              int ia, int ib, unsigned gstep, int j)
+{
+    const int s = (int)((gstep + (unsigned)j) % S);
+    unsigned char *base = sm + s * C::STAGE;
+    const int z = W.z0 - 1 + j;
+    tma_load_3d(base + C::OFF_XK, &tm->x[ia], W.x0 - 4, W.y0 - 1, z, &bars[s]);
+    tma_load_3d(base + C::OFF_XM, &tm->x[ib], W.x0 - 4, W.y0 - 1, z, &bars[s]);
 }
 
 // Shared-memory carve-up of one CTA.
@@ -458,6 +475,7 @@ struct Smem {
     double *red;
     StateSnap *snap;
     WorkItem *next;  // the item after the current one (producer lane only)
+    WorkItem *items; // the CTA's first kItemCache items
     int *kmom;  // restart: extrapolation index of each of the CTA's items
 };
 
@@ -472,14 +490,15 @@ struct Pipe {
 // One work item: plane-by-plane march over [z0, z1) of one x-y tile.
 // REC adds the three sums of F(x_k) (data, l1, TV) for the item, written to
 // `part`. kmom: the volume's extrapolation index in this iteration; tm: the
-// iteration's tensor maps (of every volume); next_it: the CTA's next item in
-// this iteration (-1: none), whose first planes the producer fetches while
-// this item's last ones are computed. Ends with a barrier over the CTA
+// iteration's tensor maps (of every volume); has_next: the CTA has another item
+// in this iteration (*sh.next), whose first planes the producer fetches while
+// this item's last ones are computed. The copies of the iteration's first S
+// steps are issued by the caller. Ends with a barrier over the CTA
 // after the item's last stores. Returns true when a barrier wait gave up (the
 // CTA then stops).
 template <int VX, int TY, int S, bool BF16, bool XD, bool REC, bool DOT, bool FOURIER>
 __device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pipe &pp_, const WorkItem &W,
-                                         int next_it, double *part, int kmom, const TmapSet *tm, int ia, int ib,
+                                         bool has_next, double *part, int kmom, const TmapSet *tm, int ia, int ib,
                                          float *xout_base, float *dout_base)
 {
     using C = Cfg<VX, TY, S, BF16>;
@@ -505,20 +524,19 @@ __device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pi
     static_assert(S <= 4, "the producer runs at most 3 steps ahead");
     auto issue = [&](int d) {
         if (d < nsteps) {
-            issue_stage<C, S, !FOURIER>(sh.sm, sh.bars, tm + W.vol, W, ia, ib, g0, d);
-        } else if (next_it >= 0) {
+            const TmapSet *t = tm + W.vol;
+            issue_fixed<C, S, !FOURIER>(sh.sm, sh.bars, t, W, g0, d);
+            issue_iterate<C, S>(sh.sm, sh.bars, t, W, ia, ib, g0, d);
+        } else if (has_next) {
             const WorkItem N = *sh.next;
-            issue_stage<C, S, !FOURIER>(sh.sm, sh.bars, tm + N.vol, N, ia, ib, g0 + (unsigned)nsteps, d - nsteps);
+            const TmapSet *t = tm + N.vol;
+            issue_fixed<C, S, !FOURIER>(sh.sm, sh.bars, t, N, g0 + (unsigned)nsteps, d - nsteps);
+            issue_iterate<C, S>(sh.sm, sh.bars, t, N, ia, ib, g0 + (unsigned)nsteps, d - nsteps);
         } else {
             return;
         }
         pp_.issued++;
     };
-    if (producer) {
-        if (next_it >= 0) *sh.next = P.items[next_it];
-        if (g0 == pp_.iter_first)
-            for (int d = 0; d < S; d++) issue(d);
-    }
 
     // registers carried across z-steps
     float xz[VX], dz[VX];         // x_k and d on plane z-1, own columns
@@ -739,7 +757,6 @@ __device__ __forceinline__ bool grid_barrier(DevState *st, unsigned target, long
     // the next copies (async proxy) read what the grid's threads wrote with
     // ordinary stores
     asm volatile("fence.proxy.async;" ::: "memory");
-    __threadfence();
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&st->bar) : "memory");
     const long long t0 = global_ns();
     for (;;) {
@@ -747,7 +764,6 @@ __device__ __forceinline__ bool grid_barrier(DevState *st, unsigned target, long
             unsigned v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&st->bar) : "memory");
             if (v >= target) {
-                __threadfence();
                 asm volatile("fence.proxy.async;" ::: "memory");
                 return true;
             }
@@ -831,6 +847,7 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     sh.next = reinterpret_cast<WorkItem *>(sh.sm + C::OFF_ST + 64);
+    sh.items = reinterpret_cast<WorkItem *>(sh.sm + C::OFF_IT);
     sh.kmom = reinterpret_cast<int *>(sh.sm + C::OFF_KM);
     const bool producer = (warp == TY) && (lane == 0);
 
@@ -849,6 +866,19 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     const int p0 = P.sched[blockIdx.x], p1 = P.sched[blockIdx.x + 1];
+    // the CTA's items, with their number (pad0) and the volume's extrapolation
+    // index at the start of the launch (pad1): the barrier between iterations
+    // drops L1, and the chain schedule, item, descriptor from L2 would delay the
+    // next iteration's first copies
+    auto fetch_item = [&](int p) {
+        const int it = P.sched[gridDim.x + 1 + p];
+        WorkItem W = P.items[it];
+        W.pad0 = it;
+        W.pad1 = P.vols[W.vol].kmom;
+        return W;
+    };
+    auto item_at = [&](int p) { return p - p0 < kItemCache ? sh.items[p - p0] : fetch_item(p); };
+    if (tid < kItemCache && p0 + tid < p1) sh.items[tid] = fetch_item(p0 + tid);
     __syncthreads();
     // select without indexing the parameter array (keeps the parameters out of local memory)
     auto pick = [&](int i) { return i == 0 ? P.xbuf[0] : (i == 1 ? P.xbuf[1] : (i == 2 ? P.xbuf[2] : P.xbuf[3])); };
@@ -856,6 +886,31 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
 
     Pipe pipe{0, 0, 0, 0};
     bool aborted = false;
+    // copies of the first S plane steps of an iteration (of its first item, or
+    // of the first two where that has only 3 steps)
+    auto first_steps = [&](auto f) {
+        const WorkItem W = sh.items[0];
+        const int n = (W.z1 - W.z0) + 2;
+#pragma unroll
+        for (int d = 0; d < S; d++) {
+            if (d < n) f(W, pipe.gstep, d);
+            else if (p0 + 1 < p1) f(item_at(p0 + 1), pipe.gstep + (unsigned)n, d - n);
+        }
+    };
+    auto first_fixed = [&](const TmapSet *tm) {
+        first_steps([&](const WorkItem &W, unsigned g, int j) {
+            if (!BF16 && XD && P.fourier)
+                issue_fixed<C, S, false>(sh.sm, sh.bars, tm + W.vol, W, g, j);
+            else
+                issue_fixed<C, S, true>(sh.sm, sh.bars, tm + W.vol, W, g, j);
+            pipe.issued++;
+        });
+    };
+    auto first_iterate = [&](const TmapSet *tm, int ia, int ib) {
+        first_steps([&](const WorkItem &W, unsigned g, int j) {
+            issue_iterate<C, S>(sh.sm, sh.bars, tm + W.vol, W, ia, ib, g, j);
+        });
+    };
     int cur = sh.snap->cur;
     int rec_in = sh.snap->rec0;  // iterations since the last recorded one (0: this one records)
     for (int itn = 0; itn < P.niter && !aborted; itn++) {
@@ -867,48 +922,67 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
         float *const dout_base = XD ? pick(2 + nxt) : nullptr;
         const TmapSet *const tm = P.tmaps + (long long)itn * P.tm_step;
         pipe.iter_first = pipe.gstep;
-        if (producer && p0 < p1 && (itn == 0 || P.tm_step)) {
-            const TmapSet *t = tm + P.items[P.sched[gridDim.x + 1 + p0]].vol;
+        if (producer && itn == 0 && p0 < p1) {
+            const TmapSet *t = tm + sh.items[0].vol;
             prefetch_tmap(&t->x[ia]);
             prefetch_tmap(&t->x[ib]);
             prefetch_tmap(&t->omtv);
             prefetch_tmap(&t->b);
             prefetch_tmap(&t->w);
             prefetch_tmap(&t->om1);
+            first_fixed(tm);
+            first_iterate(tm, ia, ib);
         }
         for (int p = p0; p < p1 && !aborted; p++) {
-            const int it = P.sched[gridDim.x + 1 + p];
+            const WorkItem W = item_at(p);
+            const int it = W.pad0;
             if (!SPG_GUARD(P.st, p1 <= P.nitems && it >= 0 && it < P.nitems, 1u)) {
                 aborted = true;
                 pipe.drain_from = pipe.gstep;
                 break;
             }
-            const WorkItem W = P.items[it];
-            const int next_it = p + 1 < p1 ? P.sched[gridDim.x + 2 + p] : -1;
-            const int kmom = (P.restart && many && itn > 0) ? sh.kmom[p - p0] : P.vols[W.vol].kmom + itn;
+            const bool has_next = p + 1 < p1;
+            if (producer && has_next) *sh.next = item_at(p + 1);
+            const int kmom = (P.restart && many && itn > 0) ? sh.kmom[p - p0] : W.pad1 + itn;
             double *const part = P.partials + ((long long)itn * P.nitems + it) * 4;
             bool done = false;
             if constexpr (!BF16 && XD) {
                 // Fourier-domain data term (float32 storage, increment storage only)
                 if (P.fourier) {
-                    aborted = rec ? run_item<VX, TY, S, BF16, XD, true, false, true>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base)
-                                  : run_item<VX, TY, S, BF16, XD, false, false, true>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base);
+                    aborted = rec ? run_item<VX, TY, S, BF16, XD, true, false, true>(P, sh, pipe, W, has_next, part, kmom, tm, ia, ib, xout_base, dout_base)
+                                  : run_item<VX, TY, S, BF16, XD, false, false, true>(P, sh, pipe, W, has_next, part, kmom, tm, ia, ib, xout_base, dout_base);
                     done = true;
                 }
             }
             if (!done) {
                 if (P.restart)
-                    aborted = rec ? run_item<VX, TY, S, BF16, XD, true, true, false>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base)
-                                  : run_item<VX, TY, S, BF16, XD, false, true, false>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base);
+                    aborted = rec ? run_item<VX, TY, S, BF16, XD, true, true, false>(P, sh, pipe, W, has_next, part, kmom, tm, ia, ib, xout_base, dout_base)
+                                  : run_item<VX, TY, S, BF16, XD, false, true, false>(P, sh, pipe, W, has_next, part, kmom, tm, ia, ib, xout_base, dout_base);
                 else
-                    aborted = rec ? run_item<VX, TY, S, BF16, XD, true, false, false>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base)
-                                  : run_item<VX, TY, S, BF16, XD, false, false, false>(P, sh, pipe, W, next_it, part, kmom, tm, ia, ib, xout_base, dout_base);
+                    aborted = rec ? run_item<VX, TY, S, BF16, XD, true, false, false>(P, sh, pipe, W, has_next, part, kmom, tm, ia, ib, xout_base, dout_base)
+                                  : run_item<VX, TY, S, BF16, XD, false, false, false>(P, sh, pipe, W, has_next, part, kmom, tm, ia, ib, xout_base, dout_base);
             }
         }
         if (aborted) break;
         if (many) {
             bool ok = true;
-            if (producer) ok = grid_barrier(P.st, (unsigned)(itn + 1) * gridDim.x, P.timeout_ns);
+            if (producer) {
+                // the next iteration's first copies: what no iteration writes before
+                // the barrier, the iterate behind it (also after a failure, so that
+                // the stages complete and can be drained)
+                const bool more = itn + 1 < P.niter && p0 < p1;
+                const TmapSet *const tn = tm + P.tm_step;
+                const int ja = nxt, jb = XD ? 2 + nxt : (nxt + 2) % 3;
+                if (more) {
+                    if (P.tm_step) {
+                        prefetch_tmap(&tn[sh.items[0].vol].x[ja]);
+                        prefetch_tmap(&tn[sh.items[0].vol].x[jb]);
+                    }
+                    first_fixed(tn);
+                }
+                ok = grid_barrier(P.st, (unsigned)(itn + 1) * gridDim.x, P.timeout_ns);
+                if (more) first_iterate(tn, ja, jb);
+            }
             if (__syncthreads_or(ok ? 0 : 1)) {
                 aborted = true;
                 pipe.drain_from = pipe.gstep;
@@ -916,7 +990,7 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
                 // the extrapolation index of the next iteration, per item
                 const double *const parts = P.partials + (long long)itn * P.nitems * 4;
                 for (int p = p0 + warp; p < p1; p += TY + 1) {
-                    const VolDesc V = P.vols[P.items[P.sched[gridDim.x + 1 + p]].vol];
+                    const VolDesc V = P.vols[item_at(p).vol];
                     const int km = itn > 0 ? sh.kmom[p - p0] : V.kmom;
                     const bool again = volume_dot(V, parts, lane) > 0.0;
                     if (lane == 0) sh.kmom[p - p0] = again ? 0 : km + 1;
