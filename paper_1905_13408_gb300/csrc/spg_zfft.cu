@@ -297,10 +297,12 @@ struct Tma {
     static constexpr int BOXES = P::N / ROWS;
     static constexpr int TILE = P::N * 16;                 // complex values per tile
     static constexpr size_t SMEM = (size_t)TILE * (2 * sizeof(float2) + sizeof(float) + sizeof(float2)) + 4 * 8;
+    // CTAs per SM: as many as shared memory holds, 1024 threads in all
+    static constexpr int CTAS = P::N >= 512 ? 1 : 512 / P::N;
 };
 
 template <int LOG2N>
-__global__ void __launch_bounds__(Pow2<LOG2N>::THREADS, 1)
+__global__ void __launch_bounds__(Pow2<LOG2N>::THREADS, Tma<LOG2N>::CTAS)
     zfft_tma_kernel(float2 *F, float scale, long long M, const float2 *__restrict__ tw,
                     const __grid_constant__ ZMaps maps, int *err)
 {
