@@ -82,7 +82,7 @@ struct spg_ctx {
 
     VolDesc *vols_d = nullptr;
     WorkItem *items_d = nullptr;
-    int *sched_d = nullptr;   // per-CTA item ranges (grid + 1) then the item order
+    int *sched_d = nullptr;   // per-CTA item ranges (grid + 1)
     TmapSet *tmaps_d = nullptr;
     int *plane_vol_d = nullptr;
     float *X[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -102,7 +102,6 @@ struct spg_ctx {
     StepVariant var{4, 8, 3, false, true};
     int zchunk = 0, grid = 0, ctas_per_sm = 0, nitems = 0;
     int iters_per_launch = 1;  // most iterations one launch of the plan runs
-    std::vector<WorkItem> items_h;
 
     long long k_total = 0;  // host mirror of the device counters
     int k_round = 0;
@@ -510,8 +509,17 @@ spg_status build_plan(spg_ctx *ctx, const StepVariant &v, int zchunk_opt)
     for (size_t i = 0; i < items.size(); i++) cost[i] = item_cost(items[i].z0, items[i].z1);
     std::vector<int> order, first;
     lpt_schedule(cost, G, &order, &first);
-    std::vector<int> sched(first);
-    sched.insert(sched.end(), order.begin(), order.end());
+    // the items in schedule order (pad0: their number), so that a CTA finds its
+    // first one with one load
+    const std::vector<int> &sched = first;
+    {
+        std::vector<WorkItem> in_order(items.size());
+        for (size_t p = 0; p < items.size(); p++) {
+            in_order[p] = items[order[p]];
+            in_order[p].pad0 = order[p];
+        }
+        items.swap(in_order);
+    }
 
     if (ctx->items_d) cudaFree(ctx->items_d);
     if (ctx->partials_d) cudaFree(ctx->partials_d);
@@ -554,7 +562,6 @@ spg_status build_plan(spg_ctx *ctx, const StepVariant &v, int zchunk_opt)
 
     ctx->var = v;
     ctx->zchunk = chunk;
-    ctx->items_h = items;
     ctx->nitems = (int)items.size();
     ctx->ctas_per_sm = occ;
     ctx->grid = G;

@@ -40,7 +40,8 @@ struct VolDesc {
 };
 
 // One work item of the fused step: an x-y tile [x0, x0+TX) x [y0, y0+TY) of
-// volume `vol`, marching over the z-planes [z0, z1).
+// volume `vol`, marching over the z-planes [z0, z1). pad0: the item's number
+// (its place among the partial sums); pad1, pad2: unused in memory.
 struct WorkItem {
     int vol, x0, y0, z0, z1, pad0, pad1, pad2;
 };
@@ -69,8 +70,8 @@ struct DevState {
 
 struct StepParams {
     const VolDesc *vols;
-    const WorkItem *items;
-    const int *sched;        // CTA g runs items sched[G+1+p] for p in [sched[g], sched[g+1]), G = gridDim.x
+    const WorkItem *items;   // in schedule order
+    const int *sched;        // CTA g runs items [sched[g], sched[g+1]), G = gridDim.x
     const TmapSet *tmaps;
     float *xbuf[4];
     const float *beta;       // extrapolation table beta_k (float32)

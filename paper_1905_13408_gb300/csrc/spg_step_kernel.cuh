@@ -783,8 +783,15 @@ __device__ __forceinline__ int recorded_before(int rec0, int every, int i)
 __device__ __forceinline__ void volume_sums(const VolDesc &V, const double *part, int lane, double (&a)[4])
 {
     a[0] = a[1] = a[2] = a[3] = 0.0;
-    for (int q = V.item_begin + lane; q < V.item_end; q += 32)
-        for (int c = 0; c < 4; c++) a[c] += __ldcg(part + (long long)q * 4 + c);
+#pragma unroll 4
+    for (int q = V.item_begin + lane; q < V.item_end; q += 32) {
+        const double2 *p = reinterpret_cast<const double2 *>(part + (long long)q * 4);
+        const double2 u = __ldcg(p), w = __ldcg(p + 1);
+        a[0] += u.x;
+        a[1] += u.y;
+        a[2] += w.x;
+        a[3] += w.y;
+    }
     const double s = ff::warp_sum4(a, lane);
 #pragma unroll
     for (int c = 0; c < 4; c++) a[c] = __shfl_sync(FULL, s, 8 * c);
@@ -794,10 +801,26 @@ __device__ __forceinline__ void volume_sums(const VolDesc &V, const double *part
 __device__ __forceinline__ double volume_dot(const VolDesc &V, const double *part, int lane)
 {
     double a = 0.0;
+#pragma unroll 4
     for (int q = V.item_begin + lane; q < V.item_end; q += 32) a += __ldcg(part + (long long)q * 4 + 3);
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) a += __shfl_xor_sync(FULL, a, m);
     return a;
+}
+
+// History entry number `entry` of volume v: F(x_k) from its sums (one thread).
+__device__ __forceinline__ void history_entry(const StepParams &P, const VolDesc &V, int v, long long entry,
+                                              long long k, const double (&a)[4])
+{
+    double *h = P.hist + ((entry % P.hist_cap) * P.nvol + v) * 5;
+    const double l1 = (double)V.lambda_l1 * a[1], tv = (double)V.lambda_tv * a[2];
+    const double tot = a[0] + l1 + tv;
+    h[0] = (double)k;
+    h[1] = a[0];
+    h[2] = l1;
+    h[3] = tv;
+    h[4] = tot;
+    if (!isfinite(tot)) atomicCAS(&P.st->err, 0, (int)SPG_ENONFINITE);
 }
 
 // Objective history of the launch: warp w of `nw` takes the (iteration,
@@ -814,18 +837,7 @@ __device__ __forceinline__ void write_history(const StepParams &P, const StateSn
         const VolDesc V = P.vols[v];
         double a[4];
         volume_sums(V, P.partials + (long long)i * P.nitems * 4, lane, a);
-        if (lane == 0) {
-            const int slot = (int)(((long long)S.hist_count + rank) % P.hist_cap);
-            double *h = P.hist + ((long long)slot * P.nvol + v) * 5;
-            const double l1 = (double)V.lambda_l1 * a[1], tv = (double)V.lambda_tv * a[2];
-            const double tot = a[0] + l1 + tv;
-            h[0] = (double)(S.k_total + i);
-            h[1] = a[0];
-            h[2] = l1;
-            h[3] = tv;
-            h[4] = tot;
-            if (!isfinite(tot)) atomicCAS(&P.st->err, 0, (int)SPG_ENONFINITE);
-        }
+        if (lane == 0) history_entry(P, V, v, (long long)S.hist_count + rank, S.k_total + i, a);
     }
 }
 
@@ -866,19 +878,23 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     const int p0 = P.sched[blockIdx.x], p1 = P.sched[blockIdx.x + 1];
-    // the CTA's items, with their number (pad0) and the volume's extrapolation
-    // index at the start of the launch (pad1): the barrier between iterations
+    // the CTA's items (P.items is in schedule order; pad0: the item's number among
+    // its volume's partial sums), with the volume's extrapolation index at the
+    // start of the launch (pad1): the barrier between iterations
     // drops L1, and the chain schedule, item, descriptor from L2 would delay the
     // next iteration's first copies
-    auto fetch_item = [&](int p) {
-        const int it = P.sched[gridDim.x + 1 + p];
-        WorkItem W = P.items[it];
-        W.pad0 = it;
+    auto item_at = [&](int p) {
+        if (p - p0 < kItemCache) return sh.items[p - p0];
+        WorkItem W = P.items[p];
         W.pad1 = P.vols[W.vol].kmom;
         return W;
     };
-    auto item_at = [&](int p) { return p - p0 < kItemCache ? sh.items[p - p0] : fetch_item(p); };
-    if (tid < kItemCache && p0 + tid < p1) sh.items[tid] = fetch_item(p0 + tid);
+    if (tid < kItemCache && p0 + tid < p1) {
+        const WorkItem W = P.items[p0 + tid];
+        sh.items[tid] = W;
+        // not waited for by the copies below: stored once it arrives
+        sh.items[tid].pad1 = P.vols[W.vol].kmom;
+    }
     __syncthreads();
     // select without indexing the parameter array (keeps the parameters out of local memory)
     auto pick = [&](int i) { return i == 0 ? P.xbuf[0] : (i == 1 ? P.xbuf[1] : (i == 2 ? P.xbuf[2] : P.xbuf[3])); };
@@ -1020,10 +1036,10 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
         const double *const parts = P.partials + (long long)(P.niter - 1) * P.nitems * 4;
         for (int p = p0 + warp; p < p1; p += TY + 1) {
             // a volume's descriptor is advanced by the CTA that runs its first item
-            const int it = P.sched[gridDim.x + 1 + p];
-            const int v = P.items[it].vol;
+            const WorkItem W = item_at(p);
+            const int v = W.vol;
             const VolDesc V = P.vols[v];
-            if (it != V.item_begin) continue;
+            if (W.pad0 != V.item_begin) continue;
             const int km = P.restart ? sh.kmom[p - p0] : V.kmom + P.niter - 1;  // index of the last iteration
             const bool again = P.restart && volume_dot(V, parts, lane) > 0.0;
             if (lane == 0) {
@@ -1042,15 +1058,18 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
     if (!sh.snap->last) return;
     __threadfence();
     if (!many) {
-        // one iteration: the last CTA sums the objective and advances every volume
-        write_history(P, snap, warp, TY + 1, lane);
+        // one iteration: the last CTA sums the objective and advances every
+        // volume, a warp per volume
+        const bool rec = P.hist_every > 0 && snap.rec0 == 0;
         for (int v = warp; v < P.nvol; v += TY + 1) {
             const VolDesc V = P.vols[v];
-            const bool again = P.restart && volume_dot(V, P.partials, lane) > 0.0;
-            __syncwarp();
+            const float beta_used = P.beta[V.kmom];
+            double a[4] = {0.0, 0.0, 0.0, 0.0};
+            if (rec || P.restart) volume_sums(V, P.partials, lane, a);
             if (lane == 0) {
-                vols_rw[v].beta_last = P.beta[V.kmom];
-                vols_rw[v].kmom = again ? 0 : V.kmom + 1;
+                if (rec) history_entry(P, V, v, snap.hist_count, snap.k_total, a);
+                vols_rw[v].beta_last = beta_used;
+                vols_rw[v].kmom = (P.restart && a[3] > 0.0) ? 0 : V.kmom + 1;
             }
         }
     }
