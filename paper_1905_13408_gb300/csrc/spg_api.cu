@@ -122,7 +122,6 @@ struct spg_ctx {
     float *Anc = nullptr;    // its anchor (pitched volume)
     float *Nst = nullptr;    // N + 2 gamma and C + 2 gamma A a / V: what the step uses when gamma_f > 0
     float2 *Cst = nullptr;
-    float *certQ = nullptr;  // 3-vector field of the certificate passes (allocated on first use)
     float *Nmax = nullptr;
     double *fpart = nullptr; // reduction partials of the Fourier data value
     // zown: per-plane 2-D transforms (batch nz) and the own transform along z
@@ -205,7 +204,7 @@ void free_all(spg_ctx *c)
         spg::cufft_api().destroy(c->pc2r);
     }
     if (c->xown) spg::cufft_api().destroy(c->pyc);
-    void *fs[] = {c->Ybuf, c->Fh, c->Yh, c->Nh, c->Ch, c->Nmax, c->fpart, c->Anc, c->Nst, c->Cst, c->certQ, c->ztw, c->xtw, c->Nx,
+    void *fs[] = {c->Ybuf, c->Fh, c->Yh, c->Nh, c->Ch, c->Nmax, c->fpart, c->Anc, c->Nst, c->Cst, c->ztw, c->xtw, c->Nx,
                   c->Cx, c->Nstx, c->Cstx};
     for (void *p : fs)
         if (p) cudaFree(p);
@@ -1136,11 +1135,12 @@ spg_status spg_create_batch(int nvol, const spg_volume_params *params, const spg
     std::vector<std::pair<int, int>> aux_range;
     const std::vector<WorkItem> aux = aux_items(ctx->vols_h, &aux_range);
     ctx->naux = (int)aux.size();
-    const int nparts = std::max(plane * AUX_SEG, ctx->naux);
+    int nparts = std::max(plane * AUX_SEG, ctx->naux);
     for (int j = 0; j < nvol; j++) {
         VolDesc &d = ctx->vols_h[j];
         d.aux_begin = aux_range[j].first;
         d.aux_end = aux_range[j].second;
+        nparts = std::max(nparts, certificate_blocks(d.nx, d.ny, d.nz));
     }
 
     auto bail = [&](cudaError_t err, const char *what) {
@@ -1798,11 +1798,10 @@ spg_status spg_certificate(spg_ctx *ctx, int vol, double *out)
     const int k = (c + ctx->nbuf() - 1) % ctx->nbuf();
     const float *xb[4] = {ctx->X[c], ctx->X[k], ctx->xd() ? nullptr : ctx->X[ctx->aux_of(k)],
                           ctx->xd() ? ctx->X[ctx->aux_of(k)] : nullptr};
-    if (!ctx->certQ) CK(dalloc(&ctx->certQ, (size_t)ctx->total * 3 * sizeof(float)), "alloc certificate field");
-    CK(launch_certificate(aux_params(ctx), vol, ctx->vols_h[vol].nz, xb, ctx->W, ctx->bf16(), ctx->OMTV, ctx->certQ,
-                          ctx->total, ctx->stream),
+    const VolDesc &d = ctx->vols_h[vol];
+    CK(launch_certificate(aux_params(ctx), vol, d.nx, d.ny, d.nz, xb, ctx->W, ctx->bf16(), ctx->OMTV, ctx->stream),
        "certificate");
-    ctx->launches += 2;
+    ctx->launches += 1;
     double o[8];
     const spg_status s = read_results(ctx, vol, o);
     if (s != SPG_OK) return s;

@@ -487,17 +487,17 @@ __global__ void __launch_bounds__(AUX_THREADS)
     }
     if (!last_block(&a.st->ticket_aux, &flag)) return;
     float m = 0.f, n = -INFINITY;
-    unsigned long long bw = 0, bb = 0;
+    int bw = 0, bb = 0;
     for (int q = threadIdx.x; q < V.aux_end - V.aux_begin; q += blockDim.x) {
         const float4 p = __ldcg(reinterpret_cast<const float4 *>(a.plane_part + (long long)q * 4));
         m = fmaxf(m, p.x);
         n = fmaxf(n, p.y);
-        bw += (unsigned)__float_as_int(p.z);
-        bb += (unsigned)__float_as_int(p.w);
+        bw |= __float_as_int(p.z);
+        bb |= __float_as_int(p.w);
     }
     m = block_fmax(m, red);
     n = block_fmax(n, red);
-    const bool any_w = __syncthreads_or(bw != 0) != 0, any_b = __syncthreads_or(bb != 0) != 0;
+    const bool any_w = __syncthreads_or(bw) != 0, any_b = __syncthreads_or(bb) != 0;
     if (threadIdx.x != 0) return;
     double *o = a.vol_out + (long long)vol * 8;
     o[0] = m;
@@ -1099,35 +1099,6 @@ __device__ __forceinline__ void st4(float *p, const float (&v)[4])
     *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
-// f at x0-1 .. x0+2 (the backward x-neighbours of the lane's voxels), x0-1
-// from the previous lane or, for a chunk's first lane, loaded; f(x0-1) := f(x0)
-// at the volume's first column (zero difference).
-__device__ __forceinline__ void left4(const float *f, const Lane4 &L, const float (&c)[4], float (&l)[4])
-{
-    float xl = __shfl_up_sync(FULL, c[3], 1);
-    if (L.lane == 0) xl = (L.act && L.x0 >= 1) ? f[L.i - 1] : c[0];
-    if (L.x0 == 0) xl = c[0];
-    l[0] = xl;
-    l[1] = c[0];
-    l[2] = c[1];
-    l[3] = c[2];
-}
-
-// f at x0+1 .. x0+4 (the forward x-neighbours), zero beyond the volume.
-__device__ __forceinline__ void right4(const VolDesc &V, const float *f, const Lane4 &L, const float (&c)[4],
-                                       float (&r)[4])
-{
-    float xr = __shfl_down_sync(FULL, c[0], 1);
-    if (L.lane == 31) xr = (L.act && L.x0 + 4 < V.nx) ? f[L.i + 4] : 0.f;
-    r[0] = c[1];
-    r[1] = c[2];
-    r[2] = c[3];
-    r[3] = xr;
-#pragma unroll
-    for (int q = 0; q < 4; q++)
-        if (L.x0 + q + 1 >= V.nx) r[q] = 0.f;
-}
-
 namespace adj {
 constexpr int TY = 7;                  // output rows per CTA
 constexpr int THREADS = 32 * (TY + 1); // warp TY: the row below the tile
@@ -1200,7 +1171,7 @@ struct AdjPlace {
     long long PS;  // plane stride
 };
 
-__device__ __forceinline__ AdjPlace adj_place(const VolDesc &V)
+__device__ __forceinline__ AdjPlace adj_place(const VolDesc &V, int zc = adj::ZC)
 {
     AdjPlace P;
     const int nchunk = (V.nx + 127) / 128, ntile = (V.ny + adj::TY - 1) / adj::TY;
@@ -1214,8 +1185,8 @@ __device__ __forceinline__ AdjPlace adj_place(const VolDesc &V)
     P.L.y = by * adj::TY + P.r;
     P.row_in = P.L.y < V.ny;
     P.L.act = P.row_in && P.L.x0 < V.nx;
-    P.z0 = bz * adj::ZC;
-    P.z1 = min(V.nz, P.z0 + adj::ZC);
+    P.z0 = bz * zc;
+    P.z1 = min(V.nz, P.z0 + zc);
     P.PS = (long long)V.pitch * V.ny;
     return P;
 }
@@ -1543,130 +1514,163 @@ __global__ void adjoint_scalars_kernel(const double *part, int nblk, double *out
     }
 }
 
-// closes the row walks of the certificate passes below
-#define ADJ_WALK_END }
-
-// ---------------- certificate, two row-vector passes ----------------
-// Q = P(x+) - P(y) with P = omtv grad h_mu(D .), stored as 3 fields; then
+// ---------------- certificate ----------------
+// Q = P(x+) - P(y) with P = omtv grad h_mu(D .), then
 // r = (y - x+)(1/tau - w) + lambda_tv D^T Q and the sum of r^2 (D^T is
-// linear: D^T P(x+) - D^T P(y) = D^T Q), each P evaluated once per voxel.
-// xbuf = {x_{k+1}, x_k, x_{k-1} or null, d_k or null}.
-#define CERT_WALK_BEGIN                                                                  \
-    const int plane_ = blockIdx.x / AUX_SEG;                                             \
-    const VolDesc V = a.vols[vol];                                                       \
-    const int zz_ = plane_;                                                              \
-    int r0, r1;                                                                          \
-    seg_rows(V.ny, blockIdx.x % AUX_SEG, r0, r1);                                        \
-    const int lane_ = threadIdx.x & 31, warp_ = threadIdx.x >> 5, nw_ = blockDim.x >> 5; \
-    const int nchunk_ = (V.nx + 127) / 128;                                              \
-    const long long PS = (long long)V.pitch * V.ny;                                      \
-    for (int rc = warp_; rc < (r1 - r0) * nchunk_; rc += nw_) {                          \
-        Lane4 L;                                                                         \
-        L.y = r0 + rc / nchunk_;                                                         \
-        L.z = zz_;                                                                       \
-        L.x0 = (rc % nchunk_) * 128 + 4 * lane_;                                         \
-        L.lane = lane_;                                                                  \
-        L.act = L.x0 < V.nx;                                                             \
-        L.i = V.off + ((long long)L.z * V.ny + L.y) * V.pitch + L.x0;
+// linear: D^T P(x+) - D^T P(y) = D^T Q). One march like the adjoint passes'
+// (a CTA owns TY rows of a 128-voxel chunk over zc planes, one more warp the
+// row below the tile): Q is evaluated once per voxel on the next plane and kept
+// in registers, its y-component passing through a 3-plane shared ring; nothing
+// is stored. Bound: x+, x_k, the pair, omtv and w, 20 bytes a voxel; as in the
+// adjoint passes the loads of a plane are issued an iteration before their use
+// (issued where they were used, this march took 1649 us at 512^3, more than the
+// 1307 of two passes that stored Q as three fields). Whole call, the two passes ->
+// this: 128^3 56 -> 43 us, 256^3 224 -> 159, 512^3 1307 -> 1024 (at the copy rate
+// 396): with 16 warps per SM still the latency of their loads.
+// x+, x_k and aux (d_k with xd, else x_{k-1}) are iterate buffers.
+struct CertRow {
+    float xp[4], xk[4], d[4];  // x+, x_k, d_k
+};
 
-// D y at the lane's voxels, y = x + beta d with d = aux (increment storage)
-// or x - aux; differences of x and of d are taken separately (Eq. 12).
-__device__ __forceinline__ void grad4_y(const VolDesc &V, const float *x, const float *aux, bool xd, float beta,
-                                        const Lane4 &L, long long PS, float (&g)[3][4])
+// Q at one voxel from the differences of x+ and of y.
+__device__ __forceinline__ void cert_q1(const float (&gp)[3], const float (&gy)[3], float ot, float mu, float (&q)[3])
 {
-    float xc[4], ac[4], xl[4], al[4], xu[4], au[4], xw[4], aw[4];
-    unpack4(ldz4(x + L.i, L.act), xc);
-    unpack4(ldz4(aux + L.i, L.act), ac);
-    left4(x, L, xc, xl);
-    left4(aux, L, ac, al);
-    if (L.y >= 1) {
-        unpack4(ldz4(x + L.i - V.pitch, L.act), xu);
-        unpack4(ldz4(aux + L.i - V.pitch, L.act), au);
-    } else {
+    const float sp = ot * fminf(1.0f / mu, rsqrtf(gp[0] * gp[0] + gp[1] * gp[1] + gp[2] * gp[2]));
+    const float sy = ot * fminf(1.0f / mu, rsqrtf(gy[0] * gy[0] + gy[1] * gy[1] + gy[2] * gy[2]));
 #pragma unroll
-        for (int q = 0; q < 4; q++) xu[q] = xc[q], au[q] = ac[q];
-    }
-    if (L.z >= 1) {
-        unpack4(ldz4(x + L.i - PS, L.act), xw);
-        unpack4(ldz4(aux + L.i - PS, L.act), aw);
-    } else {
-#pragma unroll
-        for (int q = 0; q < 4; q++) xw[q] = xc[q], aw[q] = ac[q];
-    }
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        const float dc = xd ? ac[q] : xc[q] - ac[q];
-        const float dl = xd ? al[q] : xl[q] - al[q];
-        const float du = xd ? au[q] : xu[q] - au[q];
-        const float dw = xd ? aw[q] : xw[q] - aw[q];
-        g[0][q] = (xc[q] - xl[q]) + beta * (dc - dl);
-        g[1][q] = (xc[q] - xu[q]) + beta * (dc - du);
-        g[2][q] = (xc[q] - xw[q]) + beta * (dc - dw);
-    }
+    for (int c = 0; c < 3; c++) q[c] = gp[c] * sp - gy[c] * sy;
 }
 
-__global__ void certificate_q_kernel(AuxParams a, int vol, const float *xplus, const float *xk, const float *aux, int xd,
-                                     const float *omtv, float *Q, long long S)
+__global__ void __launch_bounds__(adj::THREADS, 2)
+    certificate_kernel(AuxParams a, int vol, int zc, const float *xplus, const float *xk, const float *aux, int xd_,
+                       const void *w, bool bf16, const float *omtv)
 {
-    CERT_WALK_BEGIN
-    float gp[3][4], gy[3][4], ot[4], q3[3][4];
-    grad4_y(V, xplus, xplus, false, 0.f, L, PS, gp);
-    grad4_y(V, xk, aux, xd != 0, V.beta_last, L, PS, gy);
-    unpack4(ldz4(omtv + L.i, L.act), ot);
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        const bool valid = L.act && L.x0 + q < V.nx;
-        const float sp = ot[q] * fminf(1.0f / V.mu, rsqrtf(gp[0][q] * gp[0][q] + gp[1][q] * gp[1][q] + gp[2][q] * gp[2][q]));
-        const float sy = ot[q] * fminf(1.0f / V.mu, rsqrtf(gy[0][q] * gy[0][q] + gy[1][q] * gy[1][q] + gy[2][q] * gy[2][q]));
-#pragma unroll
-        for (int c = 0; c < 3; c++) q3[c][q] = valid ? gp[c][q] * sp - gy[c][q] * sy : 0.f;
-    }
-    if (L.act) {
-#pragma unroll
-        for (int c = 0; c < 3; c++) st4(Q + c * S + L.i, q3[c]);
-    }
-    ADJ_WALK_END
-}
-
-__global__ void certificate_r_kernel(AuxParams a, int vol, const float *xplus, const float *xk, const float *aux, int xd,
-                                     const void *w, bool bf16, const float *Q, long long S)
-{
-    __shared__ double scratch[32 * 4 + 16];
+    __shared__ __align__(16) float ring[3][adj::TY + 1][128];
+    __shared__ double red[32 * 4 + 16];
     __shared__ int flag;
-    KSum ks;
-    CERT_WALK_BEGIN
-    float q0[4], q1[4], q2[4], qx[4], qy[4], qz[4], xp[4], xc[4], ac[4], wv[4];
-    unpack4(ldz4(Q + L.i, L.act), q0);
-    unpack4(ldz4(Q + S + L.i, L.act), q1);
-    unpack4(ldz4(Q + 2 * S + L.i, L.act), q2);
-    right4(V, Q, L, q0, qx);
-    unpack4(ldz4(Q + S + L.i + V.pitch, L.act && L.y + 1 < V.ny), qy);
-    unpack4(ldz4(Q + 2 * S + L.i + PS, L.act && L.z + 1 < V.nz), qz);
-    unpack4(ldz4(xplus + L.i, L.act), xp);
-    unpack4(ldz4(xk + L.i, L.act), xc);
-    unpack4(ldz4(aux + L.i, L.act), ac);
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    unpack4(L.act ? ld4_data(w, bf16, L.i) : zero, wv);
+    const VolDesc V = a.vols[vol];
+    const bool xd = xd_ != 0;
+    AdjPlace P = adj_place(V, zc);
+    Lane4 &L = P.L;
     const float beta = V.beta_last;  // extrapolation weight of the step that produced x+
-    float acc = 0.f;
+    const float mu = V.mu, inv_tau = 1.0f / V.tau;
+    const bool writes = P.r < adj::TY && P.row_in;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    RowLoads rp, rk, ra;
+    float4 rot, fw;  // omtv of the next plane, w of this one
+    auto load_rows = [&](long long i, bool ok) {
+        rp.load(V, L, xplus, i, ok);
+        rk.load(V, L, xk, i, ok);
+        ra.load(V, L, aux, i, ok);
+        rot = ldz4(omtv + i, ok);
+    };
+    auto load_w = [&](long long i, bool ok) { fw = ok ? ld4_data(w, bf16, i) : zero; };
+    // Q at the loaded rows' plane z, the plane below in b (have: there is one);
+    // also into the ring
+    auto q_rows = [&](const CertRow &b, bool have, bool ok, int z, CertRow &c, float (&Q)[3][4]) {
+        float up[4], uk[4], ua[4], ac[4], ot[4], pl, kl, al;
+        rp.take(L, c.xp, pl, up);
+        rk.take(L, c.xk, kl, uk);
+        ra.take(L, ac, al, ua);
+        unpack4(rot, ot);
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
-        if (!(L.act && L.x0 + q < V.nx)) continue;
-        const float d = xd ? ac[q] : xc[q] - ac[q];
-        const float dy = (xc[q] - xp[q]) + beta * d;
-        const float dv = (q0[q] - qx[q]) + (q1[q] - qy[q]) + (q2[q] - qz[q]);
-        const float r = dy * (1.0f / V.tau - wv[q]) + V.lambda_tv * dv;
-        acc += r * r;
+        for (int q = 0; q < 4; q++) c.d[q] = xd ? ac[q] : c.xk[q] - ac[q];
+        const float dl = xd ? al : kl - al;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const float ud = xd ? ua[q] : uk[q] - ua[q];
+            const float wp = have ? b.xp[q] : c.xp[q], wk = have ? b.xk[q] : c.xk[q], wd = have ? b.d[q] : c.d[q];
+            const float lp = q ? c.xp[q - 1] : pl, lk = q ? c.xk[q - 1] : kl, ld = q ? c.d[q - 1] : dl;
+            const float gp[3] = {c.xp[q] - lp, c.xp[q] - up[q], c.xp[q] - wp};
+            const float gy[3] = {(c.xk[q] - lk) + beta * (c.d[q] - ld), (c.xk[q] - uk[q]) + beta * (c.d[q] - ud),
+                                 (c.xk[q] - wk) + beta * (c.d[q] - wd)};
+            float t[3];
+            cert_q1(gp, gy, ot[q], mu, t);
+            const bool valid = ok && L.x0 + q < V.nx;
+#pragma unroll
+            for (int k = 0; k < 3; k++) Q[k][q] = valid ? t[k] : 0.f;
+        }
+        *reinterpret_cast<float4 *>(&ring[z % 3][P.r][4 * L.lane]) = make_float4(Q[1][0], Q[1][1], Q[1][2], Q[1][3]);
+    };
+    KSum ks;
+    CertRow c;
+    float Qc[3][4];
+    L.i = P.row_in ? adj_row(V, L.x0, L.y, P.z0) : 0;
+    {
+        CertRow b;
+        float ab[4];
+        const bool below = L.act && P.z0 >= 1;
+        load_rows(L.i, L.act);
+        unpack4(ldz4(xplus + L.i - P.PS, below), b.xp);
+        unpack4(ldz4(xk + L.i - P.PS, below), b.xk);
+        unpack4(ldz4(aux + L.i - P.PS, below), ab);
+#pragma unroll
+        for (int q = 0; q < 4; q++) b.d[q] = xd ? ab[q] : b.xk[q] - ab[q];
+        load_w(L.i, L.act && writes);
+        q_rows(b, P.z0 >= 1, L.act, P.z0, c, Qc);
+        load_rows(L.i + P.PS, L.act && P.z0 + 1 < V.nz);
     }
-    ks.add(acc);
-    ADJ_WALK_END
-    const ff::FF fv[4] = {ks.pair(), {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-    const double s4 = block_sum4(fv, scratch);
-    if (threadIdx.x < 4) a.plane_part[(long long)blockIdx.x * 4 + threadIdx.x] = s4;
+    for (int z = P.z0; z < P.z1; z++) {
+        const long long in_ = L.i + P.PS;
+        CertRow n;
+        float Qn[3][4];
+        q_rows(c, true, L.act && z + 1 < V.nz, z + 1, n, Qn);
+        load_rows(in_ + P.PS, L.act && z + 1 < P.z1 && z + 2 < V.nz);
+        __syncthreads();  // Q_y of plane z of every row of the tile is in the ring
+        // Q_x at x+1: the next lane's first voxel; a chunk's last lane evaluates it
+        float qxn = __shfl_down_sync(FULL, Qc[0][0], 1);
+        if (L.lane == 31) {
+            qxn = 0.f;
+            if (L.act && L.x0 + 4 < V.nx) {
+                const long long j = L.i + 4;
+                auto d_at = [&](long long e) { return xd ? aux[e] : xk[e] - aux[e]; };
+                const bool u = L.y >= 1, b = z >= 1;
+                const float p0 = xplus[j], k0 = xk[j], d0 = d_at(j);
+                const long long ju = j - V.pitch, jb = j - P.PS;
+                const float pu = u ? xplus[ju] : p0, ku = u ? xk[ju] : k0, du = u ? d_at(ju) : d0;
+                const float pb = b ? xplus[jb] : p0, kb = b ? xk[jb] : k0, db = b ? d_at(jb) : d0;
+                const float gp[3] = {p0 - c.xp[3], p0 - pu, p0 - pb};
+                const float gy[3] = {(k0 - c.xk[3]) + beta * (d0 - c.d[3]), (k0 - ku) + beta * (d0 - du),
+                                     (k0 - kb) + beta * (d0 - db)};
+                float t[3];
+                cert_q1(gp, gy, omtv[j], mu, t);
+                qxn = t[0];
+            }
+        }
+        if (writes) {
+            const float4 qyv = *reinterpret_cast<const float4 *>(&ring[z % 3][P.r + 1][4 * L.lane]);
+            const float qy[4] = {qyv.x, qyv.y, qyv.z, qyv.w};  // zero when row y + 1 is outside
+            float wv[4];
+            unpack4(fw, wv);
+            load_w(in_, L.act && z + 1 < P.z1);
+            float acc = 0.f;
+            if (z >= V.halo_lo && z < V.nz - V.halo_hi) {
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    if (!(L.act && L.x0 + q < V.nx)) continue;
+                    const float qx = L.x0 + q + 1 >= V.nx ? 0.f : (q < 3 ? Qc[0][q + 1] : qxn);
+                    const float dy = (c.xk[q] - c.xp[q]) + beta * c.d[q];
+                    const float dv = (Qc[0][q] - qx) + (Qc[1][q] - qy[q]) + (Qc[2][q] - Qn[2][q]);
+                    const float r = dy * (inv_tau - wv[q]) + V.lambda_tv * dv;
+                    acc += r * r;
+                }
+            }
+            ks.add(acc);
+        }
+        c = n;
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) Qc[k][q] = Qn[k][q];
+        L.i = in_;
+    }
+    const ff::FF v[4] = {ks.pair(), {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    const double s = block_sum4(v, red);
+    if (threadIdx.x < 4) a.plane_part[(long long)blockIdx.x * 4 + threadIdx.x] = s;
     if (!last_block(&a.st->ticket_aux, &flag)) return;
     double t[4];
     float mx;
-    part_total(a.plane_part, V.halo_lo * AUX_SEG, (V.nz - V.halo_hi) * AUX_SEG, warp_, nw_, false, scratch, t, mx);
+    part_total(a.plane_part, 0, (int)gridDim.x, (int)(threadIdx.x >> 5), (int)(blockDim.x >> 5), false, red, t, mx);
     if (threadIdx.x == 0) {
         a.vol_out[(long long)vol * 8 + 4] = t[0];
         a.st->ticket_aux = 0;
@@ -1769,14 +1773,25 @@ cudaError_t launch_objective(const AuxParams &a, const float *const *xbuf, const
     return cudaGetLastError();
 }
 
-cudaError_t launch_certificate(const AuxParams &a, int vol, int nz, const float *const *xbuf, const void *w, bool bf16,
-                               const float *omtv, float *Q, long long stride, cudaStream_t s)
+// Planes per CTA of the certificate: about 4 waves of 2 CTAs per SM, at most 32.
+static int certificate_chunk(int nx, int ny, int nz)
+{
+    const long long tiles = (long long)((nx + 127) / 128) * ((ny + adj::TY - 1) / adj::TY) * nz;
+    return (int)std::max<long long>(2, std::min<long long>(32, tiles / 1216));
+}
+
+int certificate_blocks(int nx, int ny, int nz)
+{
+    const int zc = certificate_chunk(nx, ny, nz);
+    return ((nx + 127) / 128) * ((ny + adj::TY - 1) / adj::TY) * ((nz + zc - 1) / zc);
+}
+
+cudaError_t launch_certificate(const AuxParams &a, int vol, int nx, int ny, int nz, const float *const *xbuf,
+                               const void *w, bool bf16, const float *omtv, cudaStream_t s)
 {
     const bool xd = xbuf[3] != nullptr;
-    const float *aux = xd ? xbuf[3] : xbuf[2];
-    certificate_q_kernel<<<nz * AUX_SEG, AUX_THREADS, 0, s>>>(a, vol, xbuf[0], xbuf[1], aux, xd ? 1 : 0, omtv, Q, stride);
-    certificate_r_kernel<<<nz * AUX_SEG, AUX_THREADS, 0, s>>>(a, vol, xbuf[0], xbuf[1], aux, xd ? 1 : 0, w, bf16, Q,
-                                                              stride);
+    certificate_kernel<<<certificate_blocks(nx, ny, nz), adj::THREADS, 0, s>>>(
+        a, vol, certificate_chunk(nx, ny, nz), xbuf[0], xbuf[1], xd ? xbuf[3] : xbuf[2], xd ? 1 : 0, w, bf16, omtv);
     return cudaGetLastError();
 }
 

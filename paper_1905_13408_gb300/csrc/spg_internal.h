@@ -118,7 +118,7 @@ struct AuxParams {
     DevState *st;
     const WorkItem *items;   // march items of every volume
     int nitems;
-    double *plane_part;      // [max(nplanes * AUX_SEG, nitems)][4]
+    double *plane_part;      // [max(nplanes * AUX_SEG, nitems, certificate_blocks)][4]
     double *vol_out;         // [nvol][8]
     int readings;            // SPG_READ_* flags of the context (0: the row-vector kernels)
 };
@@ -136,10 +136,11 @@ cudaError_t launch_reweight(const AuxParams &a, const float *const *xbuf, float 
 cudaError_t launch_objective(const AuxParams &a, const float *const *xbuf, const void *b, const void *w,
                              bool bf16, const float *om1, const float *omtv, cudaStream_t s);
 // Strong-convexity certificate of volume `vol`'s last step, xbuf = {x_{k+1},
-// x_k, x_{k-1} or null, d_k or null}: two row-vector passes (Q = P(x+) - P(y)
-// stored in 3 fields of `stride` elements each, then the residual sum).
-cudaError_t launch_certificate(const AuxParams &a, int vol, int nz, const float *const *xbuf, const void *w, bool bf16,
-                               const float *omtv, float *Q, long long stride, cudaStream_t s);
+// x_k, x_{k-1} or null, d_k or null}: one march (certificate_blocks CTAs, one
+// partial each).
+int certificate_blocks(int nx, int ny, int nz);
+cudaError_t launch_certificate(const AuxParams &a, int vol, int nx, int ny, int nz, const float *const *xbuf,
+                               const void *w, bool bf16, const float *omtv, cudaStream_t s);
 
 // Adjoint of one step (spg_aux.cu): given gnext = dL/dx_{k+1} and the step's
 // inputs, accumulates into gcur (dL/dx_k), gprev (dL/dx_{k-1}), gb, gw and the
