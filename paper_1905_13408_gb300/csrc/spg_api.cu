@@ -1224,6 +1224,32 @@ spg_status spg_create(const spg_volume_params *params, const spg_options *opt, v
     return spg_create_batch(1, params, opt, stream, out);
 }
 
+// An array a kernel of this context can read where it lies: memory of the
+// current device, aligned to its elements.
+static bool readable_here(const void *p, size_t es)
+{
+    cudaPointerAttributes at;
+    int dev = -1;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev && reinterpret_cast<uintptr_t>(p) % es == 0;
+}
+
+// The verdict of the validation queued before (synchronises).
+static spg_status data_checked(spg_ctx *ctx, int vol)
+{
+    double o[8];
+    CK(cudaMemcpyAsync(o, ctx->vol_out_d + (size_t)vol * 8, sizeof(o), cudaMemcpyDeviceToHost, ctx->stream),
+       "read validation");
+    CK(cudaStreamSynchronize(ctx->stream), "synchronise");
+    if (o[3] > 0) return fail(ctx, SPG_ENONFINITE, "spg_set_data: b has non-finite values");
+    if (o[2] > 0) return fail(ctx, SPG_EINVAL, "spg_set_data: w must be finite and > 0");
+    ctx->data_set[vol] = 1;
+    return SPG_OK;
+}
+
 spg_status spg_set_data(spg_ctx *ctx, int vol, const void *b, const void *w, spg_dtype src)
 {
     SPG_TRACE();
@@ -1241,7 +1267,16 @@ spg_status spg_set_data(spg_ctx *ctx, int vol, const void *b, const void *w, spg
     const long long n = (long long)d.pitch * d.ny * d.nz;
     const bool store_bf16 = ctx->bf16();
     spg_status s;
-    if ((src == SPG_BF16) == store_bf16) {
+    const bool same = (src == SPG_BF16) == store_bf16;
+    if (!ctx->reversed && readable_here(b, src == SPG_BF16 ? 2 : 4) && readable_here(w, src == SPG_BF16 ? 2 : 4)) {
+        if (!same) ctx->reweighted = false;
+        ctx->launches += 1;
+        CK(launch_ingest(aux_params(ctx), vol, d.aux_end - d.aux_begin, d.nx, b, w, src == SPG_BF16, ctx->B, ctx->W,
+                         store_bf16, ctx->maxw_d, ctx->stream),
+           "copy and validate");
+        return data_checked(ctx, vol);
+    }
+    if (same) {
         if ((s = copy_volume_in(ctx, ctx->B, ctx->data_es(), d, b)) != SPG_OK) return s;
         if ((s = copy_volume_in(ctx, ctx->W, ctx->data_es(), d, w)) != SPG_OK) return s;
     } else {
@@ -1267,14 +1302,7 @@ spg_status spg_set_data(spg_ctx *ctx, int vol, const void *b, const void *w, spg
     ctx->launches += 1;
     CK(launch_validate(aux_params(ctx), vol, d.aux_end - d.aux_begin, ctx->B, ctx->W, store_bf16, ctx->maxw_d, ctx->stream),
        "validate");
-    double o[8];
-    CK(cudaMemcpyAsync(o, ctx->vol_out_d + (size_t)vol * 8, sizeof(o), cudaMemcpyDeviceToHost, ctx->stream),
-       "read validation");
-    CK(cudaStreamSynchronize(ctx->stream), "synchronise");
-    if (o[3] > 0) return fail(ctx, SPG_ENONFINITE, "spg_set_data: b has non-finite values");
-    if (o[2] > 0) return fail(ctx, SPG_EINVAL, "spg_set_data: w must be finite and > 0");
-    ctx->data_set[vol] = 1;
-    return SPG_OK;
+    return data_checked(ctx, vol);
 }
 
 spg_status spg_set_data_fourier(spg_ctx *ctx, int vol, const void *y_half, const float *N_half)

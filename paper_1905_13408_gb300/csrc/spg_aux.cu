@@ -4,12 +4,13 @@
 // and the plain step used under alternative readings of the paper.
 //
 // None of them is on the fused hot path, so they use plain global loads.
-// The adopted reading's re-weighting and objective,
-// the validation and the anchor march over z: a CTA takes 8 rows (a warp each)
-// of a 128-voxel chunk over a run of planes (AuxParams::items), each lane 4
-// voxels by 16-byte loads, the plane below kept in registers and the loads of
-// several planes issued together. The kernels of the alternative readings, the
-// certificate and the parameter scales run AUX_SEG CTAs per z-plane (one per row segment).
+// The adopted reading's re-weighting and objective, the validation and the
+// anchor march over z: a CTA takes 8 rows (a warp each) of a 128-voxel chunk over
+// a run of planes (AuxParams::items), each lane 4 voxels by 16-byte loads, the
+// plane below kept in registers and the loads of several planes issued
+// together; the certificate marches as the adjoint passes do. The kernels of the
+// alternative readings and the parameter scales run AUX_SEG CTAs per z-plane
+// (one per row segment).
 // Every reduction keeps one partial per CTA, and the last CTA to finish sums
 // the partials of each volume in a fixed order, so the results are
 // deterministic; the adjoint passes keep one scalar partial per CTA, which the
@@ -22,10 +23,8 @@
 // 101 x 147 x 183 42.9 -> 25.2, 256^3 114 -> 62, 512^3 520 -> 349 (12 bytes a
 // voxel at the copy rate: 237); objective 50.1 -> 38.2, 61.3 -> 50.3, 124 -> 100,
 // 495 -> 436 (20 bytes: 396); spg_set_data with its validation 45.2 -> 33.3,
-// 84.4 -> 71.9, 146 -> 98, 717 -> 518 (copies and one read, 24 bytes: 475).
-// The certificate as one march without its stored field was slower than its two
-// row-segment passes (256^3 254 us against 224, 512^3 1649 against 1307: 16
-// warps per SM waiting for each plane's loads) and is not kept.
+// 84.4 -> 71.9, 146 -> 98, 717 -> 518 (host arrays and reversed contexts still go
+// this way; device arrays are taken in by one pass, ingest_kernel).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -428,54 +427,61 @@ __device__ __forceinline__ March march_place(const VolDesc &V, const WorkItem &W
 }
 
 // ---------------- validation ----------------
-// max w, min w, count(w <= 0 or w not finite), count(b not finite) of volume
-// `vol`, over its march items.
-__global__ void __launch_bounds__(AUX_THREADS)
-    validate_kernel(AuxParams a, int vol, const void *b, const void *w, bool bf16, double *maxw_out)
+__device__ __forceinline__ void st_data(void *p, bool bf16, long long i, float v)
+{
+    if (bf16) {
+        __nv_bfloat16 h = __float2bfloat16_rn(v);
+        reinterpret_cast<uint16_t *>(p)[i] = *reinterpret_cast<uint16_t *>(&h);
+    } else {
+        reinterpret_cast<float *>(p)[i] = v;
+    }
+}
+
+// 4 values in one store (rows start 32-byte aligned; a value widened from
+// bfloat16 goes back unchanged).
+template <bool BF16>
+__device__ __forceinline__ void st4_data(void *p, long long i, const float (&v)[4])
+{
+    if constexpr (BF16) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
+        uint2 u;
+        u.x = *reinterpret_cast<const uint32_t *>(&lo);
+        u.y = *reinterpret_cast<const uint32_t *>(&hi);
+        *reinterpret_cast<uint2 *>(reinterpret_cast<uint16_t *>(p) + i) = u;
+    } else {
+        *reinterpret_cast<float4 *>(reinterpret_cast<float *>(p) + i) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+}
+
+// What validation collects: max and min w (finite ones), values of w that are
+// not finite and positive, values of b that are not finite.
+struct DataCheck {
+    float mx = 0.f, nmn = -INFINITY;
+    int bad_w = 0, bad_b = 0;
+    __device__ __forceinline__ void add(float bv, float wv)
+    {
+        const bool wfin = isfinite(wv);
+        bad_w += (!(wv > 0.f) || !wfin) ? 1 : 0;
+        bad_b += isfinite(bv) ? 0 : 1;
+        if (wfin) {
+            mx = fmaxf(mx, wv);
+            nmn = fmaxf(nmn, -wv);
+        }
+    }
+};
+
+// The CTA's check into its partial; the last CTA's totals into vol_out and max w.
+__device__ void check_finish(const AuxParams &a, int vol, const VolDesc &V, DataCheck c, double *maxw_out)
 {
     __shared__ float red[32];
     __shared__ int cnt[2], flag;
-    const VolDesc V = a.vols[vol];
-    const WorkItem W = a.items[V.aux_begin + blockIdx.x];
-    const March M = march_place(V, W);
-    float fmx = 0.f, nmn = -INFINITY;
-    int bad_w = 0, bad_b = 0;
-    constexpr int U = 4;
-    for (int z = M.z0; z < M.z1; z += U) {
-        float4 bv[U], wv[U];
-#pragma unroll
-        for (int u = 0; u < U; u++)
-            if (M.act && z + u < M.z1) {
-                const long long i = M.i + (long long)(z + u - M.z0) * M.PS;
-                bv[u] = ld4_data(b, bf16, i);
-                wv[u] = ld4_data(w, bf16, i);
-            }
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            if (!(M.act && z + u < M.z1)) continue;
-            float bb[4], ww[4];
-            unpack4(bv[u], bb);
-            unpack4(wv[u], ww);
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                if (M.x0 + q >= V.nx) continue;
-                const bool wfin = isfinite(ww[q]);
-                bad_w += (!(ww[q] > 0.f) || !wfin) ? 1 : 0;
-                bad_b += isfinite(bb[q]) ? 0 : 1;
-                if (wfin) {
-                    fmx = fmaxf(fmx, ww[q]);
-                    nmn = fmaxf(nmn, -ww[q]);
-                }
-            }
-        }
-    }
     if (threadIdx.x < 2) cnt[threadIdx.x] = 0;
-    const float mx = block_fmax(fmx, red), nm = block_fmax(nmn, red);
-    bad_w = __reduce_add_sync(FULL, bad_w);
-    bad_b = __reduce_add_sync(FULL, bad_b);
-    if (M.lane == 0 && (bad_w | bad_b)) {
-        atomicAdd(&cnt[0], bad_w);
-        atomicAdd(&cnt[1], bad_b);
+    const float mx = block_fmax(c.mx, red), nm = block_fmax(c.nmn, red);
+    c.bad_w = __reduce_add_sync(FULL, c.bad_w);
+    c.bad_b = __reduce_add_sync(FULL, c.bad_b);
+    if ((threadIdx.x & 31) == 0 && (c.bad_w | c.bad_b)) {
+        atomicAdd(&cnt[0], c.bad_w);
+        atomicAdd(&cnt[1], c.bad_b);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -509,17 +515,109 @@ __global__ void __launch_bounds__(AUX_THREADS)
     __threadfence();
 }
 
-// ---------------- implicit-gradient anchor (Eq. 22 / Eq. 31) ----------------
-__device__ __forceinline__ void st_data(void *p, bool bf16, long long i, float v)
+// The stored b and w of volume `vol`, over its march items.
+__global__ void __launch_bounds__(AUX_THREADS)
+    validate_kernel(AuxParams a, int vol, const void *b, const void *w, bool bf16, double *maxw_out)
 {
-    if (bf16) {
-        __nv_bfloat16 h = __float2bfloat16_rn(v);
-        reinterpret_cast<uint16_t *>(p)[i] = *reinterpret_cast<uint16_t *>(&h);
-    } else {
-        reinterpret_cast<float *>(p)[i] = v;
+    const VolDesc V = a.vols[vol];
+    const WorkItem W = a.items[V.aux_begin + blockIdx.x];
+    const March M = march_place(V, W);
+    DataCheck C;
+    constexpr int U = 4;
+    for (int z = M.z0; z < M.z1; z += U) {
+        float4 bv[U], wv[U];
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (M.act && z + u < M.z1) {
+                const long long i = M.i + (long long)(z + u - M.z0) * M.PS;
+                bv[u] = ld4_data(b, bf16, i);
+                wv[u] = ld4_data(w, bf16, i);
+            }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (!(M.act && z + u < M.z1)) continue;
+            float bb[4], ww[4];
+            unpack4(bv[u], bb);
+            unpack4(wv[u], ww);
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if (M.x0 + q < V.nx) C.add(bb[q], ww[q]);
+        }
     }
+    check_finish(a, vol, V, C, maxw_out);
 }
 
+// Device-resident b and w: copied (or converted) into the context's layout and
+// validated in one pass, 16 bytes a voxel, instead of a copy of each and a pass
+// over the copies, 24 (and 4 more with a staged conversion). VEC: rows of the
+// caller's arrays start on 4-element boundaries and a lane takes 4 neighbouring
+// voxels; otherwise a lane takes voxels 32 apart, so that any row start gives
+// coalesced accesses (and rows narrower than their pitch need no 2-D copy).
+// Checked are the values as stored. Whole call, before -> after:
+// 101 x 147 x 183 72 -> 33 us, 256^3 98 -> 69, 512^3 518 -> 343 (at the copy rate 317).
+template <bool SRC16, bool DST16, bool VEC>
+__global__ void __launch_bounds__(AUX_THREADS)
+    ingest_kernel(AuxParams a, int vol, const void *__restrict__ sb, const void *__restrict__ sw, void *b, void *w,
+                  double *maxw_out)
+{
+    const VolDesc V = a.vols[vol];
+    const WorkItem W = a.items[V.aux_begin + blockIdx.x];
+    const int lane = threadIdx.x & 31, y = W.y0 + (threadIdx.x >> 5);
+    DataCheck C;
+    auto stored = [](float v) {
+        return DST16 && !SRC16 ? __uint_as_float((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v)) << 16) : v;
+    };
+    if (y < V.ny) {
+        constexpr int U = VEC ? 4 : 2;
+        const long long sps = (long long)V.nx * V.ny, dps = (long long)V.pitch * V.ny;
+        const long long si = (long long)W.z0 * sps + (long long)y * V.nx + W.x0;
+        const long long di = V.off + (long long)W.z0 * dps + (long long)y * V.pitch + W.x0;
+        for (int z = W.z0; z < W.z1; z += U) {
+            float bv[U][4], wv[U][4];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const long long i = si + (long long)(z + u - W.z0) * sps;
+                if constexpr (VEC) {
+                    if (z + u < W.z1 && W.x0 + 4 * lane < V.nx) {
+                        unpack4(ld4_data(sb, SRC16, i + 4 * lane), bv[u]);
+                        unpack4(ld4_data(sw, SRC16, i + 4 * lane), wv[u]);
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; q++)
+                        if (z + u < W.z1 && W.x0 + lane + 32 * q < V.nx) {
+                            bv[u][q] = ld_data(sb, SRC16, i + lane + 32 * q);
+                            wv[u][q] = ld_data(sw, SRC16, i + lane + 32 * q);
+                        }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (z + u >= W.z1) break;
+                const long long i = di + (long long)(z + u - W.z0) * dps;
+                if constexpr (VEC) {
+                    if (W.x0 + 4 * lane < V.nx) {
+#pragma unroll
+                        for (int q = 0; q < 4; q++) C.add(stored(bv[u][q]), stored(wv[u][q]));
+                        st4_data<DST16>(b, i + 4 * lane, bv[u]);
+                        st4_data<DST16>(w, i + 4 * lane, wv[u]);
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; q++)
+                        if (W.x0 + lane + 32 * q < V.nx) {
+                            C.add(stored(bv[u][q]), stored(wv[u][q]));
+                            st_data(b, DST16, i + lane + 32 * q, bv[u][q]);
+                            st_data(w, DST16, i + lane + 32 * q, wv[u][q]);
+                        }
+                }
+            }
+        }
+    }
+    check_finish(a, vol, V, C, maxw_out);
+}
+
+// ---------------- implicit-gradient anchor (Eq. 22 / Eq. 31) ----------------
 // w' = w + 2 gamma, b' = (w b + 2 gamma a) / w'; then max w' of the volume.
 __global__ void __launch_bounds__(AUX_THREADS)
     anchor_kernel(AuxParams a, int vol, void *b, void *w, bool bf16, const float *anchor, float gamma, double *maxw_out)
@@ -1684,6 +1782,23 @@ cudaError_t launch_validate(const AuxParams &a, int vol, int nitems, const void 
                             double *maxw_out, cudaStream_t s)
 {
     validate_kernel<<<nitems, AUX_THREADS, 0, s>>>(a, vol, b, w, bf16, maxw_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_ingest(const AuxParams &a, int vol, int nitems, int nx, const void *sb, const void *sw, bool src16,
+                          void *b, void *w, bool dst16, double *maxw_out, cudaStream_t s)
+{
+    const uintptr_t align = src16 ? 8 : 16;
+    const bool vec = nx % 4 == 0 && ((reinterpret_cast<uintptr_t>(sb) | reinterpret_cast<uintptr_t>(sw)) % align) == 0;
+    auto go = [&](auto k) { k<<<nitems, AUX_THREADS, 0, s>>>(a, vol, sb, sw, b, w, maxw_out); };
+    if (src16 && dst16)
+        vec ? go(ingest_kernel<true, true, true>) : go(ingest_kernel<true, true, false>);
+    else if (src16)
+        vec ? go(ingest_kernel<true, false, true>) : go(ingest_kernel<true, false, false>);
+    else if (dst16)
+        vec ? go(ingest_kernel<false, true, true>) : go(ingest_kernel<false, true, false>);
+    else
+        vec ? go(ingest_kernel<false, false, true>) : go(ingest_kernel<false, false, false>);
     return cudaGetLastError();
 }
 

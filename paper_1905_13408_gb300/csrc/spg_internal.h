@@ -128,6 +128,10 @@ std::vector<WorkItem> aux_items(const std::vector<VolDesc> &vols, std::vector<st
 // nitems: march items of volume `vol`.
 cudaError_t launch_validate(const AuxParams &a, int vol, int nitems, const void *b, const void *w, bool bf16,
                             double *maxw_out, cudaStream_t s);
+// The caller's device arrays sb, sw (contiguous [nz][ny][nx], naturally aligned)
+// into volume `vol` of b, w, converted if the types differ, and validated.
+cudaError_t launch_ingest(const AuxParams &a, int vol, int nitems, int nx, const void *sb, const void *sw, bool src16,
+                          void *b, void *w, bool dst16, double *maxw_out, cudaStream_t s);
 cudaError_t launch_convert_to_bf16(const float *src, uint16_t *dst, long long n, cudaStream_t s);
 cudaError_t launch_convert_to_f32(const uint16_t *src, float *dst, long long n, cudaStream_t s);
 cudaError_t launch_reverse_axes(void *v, size_t es, int nx, int ny, int nz, int pitch, cudaStream_t s);
