@@ -15,7 +15,7 @@
 // or, mirrored, at -n, whichever lies in the stored half spectrum
 // [n][n][n/2+1] (both on the planes kx = 0 and kx = n/2). This halves both
 // the atomics and the accumulator against a full-spectrum scatter and gives
-// the same sums. A warp takes an 8 x 8 tile of one image's coefficients,
+// the same sums. A warp takes an 8 x 4 tile of one image's coefficients,
 // sums their FP32 deposits in a shared-memory box of its own and adds each
 // touched point once, with FP64 atomics, into an interleaved accumulator
 // (Re num, Im num, N, unused: one 32-byte sector per grid point). A finishing
@@ -200,9 +200,11 @@ __device__ __forceinline__ double widen(float v)
 // in L2.
 //
 // Measured, add and finish, against the thread-per-sample form (8 x 8 tiles,
-// float32 atomics in the box): 2048 images of 256^2 12.4 -> 7.4 ms (trilinear
-// 7.8 -> 5.6), 128 images 1.08 -> 0.73, 2048 of 128^2 3.20 -> 1.96, 4096 of 64^2
-// 1.64 -> 1.12, 512 of 288^2 4.24 -> 2.65. What bounds it now, at 256^2: shared
+// float32 atomics in the box): 2048 images of 256^2 12.4 -> 7.3 ms (trilinear
+// 7.8 -> 5.6), 128 images 1.08 -> 0.73, 2048 of 128^2 3.20 -> 1.95, 4096 of 64^2
+// 1.64 -> 1.10, 512 of 288^2 4.24 -> 2.63; with one wrapping addition per index of
+// the boxes that cross the box's faces, instead of two integer divisions for
+// each of six indices of a point, 7.0 (5.35), 0.72, 1.78, 0.99 and 2.54. What bounds it now, at 256^2: shared
 // memory (800 wavefronts a tile, 64 % of its rate) and issue (2900 instructions
 // a tile, 53 %) with the 16 warps an SM's shared memory holds.
 constexpr int kTileX = 8, kTileY = 4;
@@ -373,13 +375,51 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
                     }
                 }
             } else {
-                // a lane per box point, every index wrapped on its own
+                // a lane per box point, every index wrapped on its own (by one
+                // addition: the box starts in [0, n) after wrapping its corner,
+                // and is no longer than n on any axis for rotations)
+                const bool near = EX <= n && EY <= n && EZ <= n;
                 const int EXY = EX * EY;
+                const int q0 = lane < EXY * EZ ? lane : 0;
+                int z = q0 / EXY, y = (q0 - z * EXY) / EX, x = q0 - z * EXY - y * EX;
+                // 32 points on
+                const int sz = 32 / EXY, sy = (32 - sz * EXY) / EX, sx = 32 - sz * EXY - sy * EX;
                 for (int q = lane; q < EXY * EZ; q += 32) {
-                    const int z = q / EXY, r = q - z * EXY, y = r / EX, x = r - y * EX;
                     const float4 v = box[z * DXY + y * DX + x];
-                    if (v.x == 0.f && v.y == 0.f && v.z == 0.f) continue;
-                    deposit(acc, n, lx + x, ly + y, lz + z, widen(v.x), widen(v.y), widen(v.z), false);
+                    if (v.x != 0.f || v.y != 0.f || v.z != 0.f) {
+                        const double re = widen(v.x), im = widen(v.y), nn = widen(v.z);
+                        if (near) {
+                            const int ax = wx0 + x < n ? wx0 + x : wx0 + x - n;
+                            const int ay = wy0 + y < n ? wy0 + y : wy0 + y - n;
+                            const int az = wz0 + z < n ? wz0 + z : wz0 + z - n;
+                            if (ax < nh) {
+                                double *p = acc + (4LL * ax + zs * az + ys * ay);
+                                atomicAdd(p, re);
+                                atomicAdd(p + 1, im);
+                                atomicAdd(p + 2, nn);
+                            }
+                            const int mx = ax == 0 ? 0 : n - ax;
+                            if (mx < nh) {
+                                double *p = acc + (4LL * mx + zs * (az == 0 ? 0 : n - az) + ys * (ay == 0 ? 0 : n - ay));
+                                atomicAdd(p, re);
+                                atomicAdd(p + 1, -im);
+                                atomicAdd(p + 2, nn);
+                            }
+                        } else {
+                            deposit(acc, n, lx + x, ly + y, lz + z, re, im, nn, false);
+                        }
+                    }
+                    x += sx;
+                    y += sy;
+                    z += sz;
+                    if (x >= EX) {
+                        x -= EX;
+                        y++;
+                    }
+                    if (y >= EY) {
+                        y -= EY;
+                        z++;
+                    }
                 }
             }
             __syncwarp();
