@@ -50,11 +50,13 @@
 // before the barrier. An iteration with the objective, one per launch
 // (replayed from a graph) -> many per launch -> items in shared memory (the
 // barrier drops L1, and the chain schedule, item, descriptor from L2 delayed
-// the first copies) and copies before the barrier, same tiles for the last two:
-// 28 x 32 x 40 9.7 -> 5.4 -> 5.1 us, 64^3 11.3 -> 7.6 -> 7.0, 128^3 18.6 -> 14.1
-// -> 13.5, 101 x 147 x 183 30.7 -> 20.8 -> 20.0, 180^3 57.6 -> 43.3 -> 41.3,
-// 256^3 86.8 -> 81.5 -> 79.7, 512^3 618.4 -> 617.2 -> 614.1; 24 volumes of 96^3 ..
-// 256^3 777 -> 767. (With the producer's position in shared memory instead of
+// the first copies) and copies before the barrier -> missing neighbours by
+// address (16 selects fewer among 360 instructions of a 4-voxel plane step),
+// same tiles but for the first: 28 x 32 x 40 9.7 -> 5.4 -> 5.1 -> 4.8 us, 64^3 11.3
+// -> 7.6 -> 7.0 -> 6.9, 128^3 18.6 -> 14.1 -> 13.5 -> 13.2, 101 x 147 x 183 30.7 ->
+// 20.8 -> 20.0 -> 19.8, 180^3 57.6 -> 43.3 -> 41.3 -> 40.4, 256^3 86.8 -> 81.5 ->
+// 79.7 -> 78.7, 512^3 618.4 -> 617.2 -> 614.1 -> 606.6; 24 volumes of 96^3 .. 256^3
+// (the last three) 777 -> 767 -> 755. (With the producer's position in shared memory instead of
 // the item's registers the long marches lost: 623.6 at 512^3, 1128 for the
 // batch: its warp is the last to arrive at every plane's barrier.)
 #pragma once
