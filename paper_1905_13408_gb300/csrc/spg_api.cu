@@ -133,12 +133,16 @@ struct spg_ctx {
     float2 *ztw = nullptr;           // twiddle table of the transform along z
     ZMaps zmaps[2]{};                // TMA maps of the z pass: with (N, C), with (N + 2 gamma, C + ...)
     bool zmaps_ok[2] = {false, false};
-    // xown: each iteration's in-plane transforms are the own row pass
-    // (power-of-two nx 128 .. 1024) and the library's transform along y over
-    // the contiguous lines of the kx-major spectrum [nz][nx/2+1][ny]; the z
-    // pass then reads N and C (and their anchor variants) in that order
-    bool xown = false;
+    // xown: each iteration's in-plane transforms are an own row pass and the
+    // library's transform along y over the contiguous lines of the kx-major
+    // spectrum [nz][nx/2+1][ny]; the z pass then reads N and C (and their
+    // anchor variants) in that order. The row pass is spg_xpass.cu's
+    // (power-of-two nx 128 .. 1024, then with zown) or spg_mixed.cu's (xmix),
+    // which then also has the z pass if not zown.
+    bool xown = false, xmix = false;
     float2 *xtw = nullptr;           // twiddle table of the row pass
+    float2 *mztw = nullptr;          // and of the mixed-radix z pass
+    MixAxis mx{}, mz{};
     cufftHandle pyc = 0;             // complex transform along y, nz (nx/2+1) contiguous lines
     float *Nx = nullptr;             // N, C, N + 2 gamma, C + ... held kx-major
     float2 *Cx = nullptr;
@@ -204,7 +208,7 @@ void free_all(spg_ctx *c)
         spg::cufft_api().destroy(c->pc2r);
     }
     if (c->xown) spg::cufft_api().destroy(c->pyc);
-    void *fs[] = {c->Ybuf, c->Fh, c->Yh, c->Nh, c->Ch, c->Nmax, c->fpart, c->Anc, c->Nst, c->Cst, c->ztw, c->xtw, c->Nx,
+    void *fs[] = {c->Ybuf, c->Fh, c->Yh, c->Nh, c->Ch, c->Nmax, c->fpart, c->Anc, c->Nst, c->Cst, c->ztw, c->xtw, c->mztw, c->Nx,
                   c->Cx, c->Nstx, c->Cstx};
     for (void *p : fs)
         if (p) cudaFree(p);
@@ -722,11 +726,16 @@ cudaError_t issue_iteration(spg_ctx *ctx, const StepParams &p)
         const bool anc = ctx->gamma_f > 0.f;
         if (ctx->xown) {
             cufftComplex *Fc = reinterpret_cast<cufftComplex *>(ctx->Fh);
-            e = launch_xpass_r2c_extrap(d.nx, ctx->st_d, ctx->vols_d, ctx->beta_d, ctx->X, d.pitch, d.ny, d.nz,
-                                        ctx->Fh, ctx->xtw, ctx->stream);
+            e = ctx->xmix ? launch_mix_r2c(ctx->mx, ctx->xtw, ctx->st_d, ctx->vols_d, ctx->beta_d, ctx->X, d.pitch, d.ny,
+                                           d.nz, ctx->Fh, ctx->stream)
+                          : launch_xpass_r2c_extrap(d.nx, ctx->st_d, ctx->vols_d, ctx->beta_d, ctx->X, d.pitch, d.ny,
+                                                    d.nz, ctx->Fh, ctx->xtw, ctx->stream);
             if (e != cudaSuccess) return e;
             if (cf.exec_c2c(ctx->pyc, Fc, Fc, CUFFT_FORWARD) != CUFFT_SUCCESS) return cudaErrorUnknown;
-            if (ctx->zmapsx_ok[anc ? 1 : 0])
+            if (!ctx->zown)
+                e = launch_mix_residual(ctx->Fh, anc ? ctx->Nstx : ctx->Nx, anc ? ctx->Cstx : ctx->Cx, (float)(1.0 / V),
+                                        ctx->mz, ctx->mztw, (long long)d.ny * (d.nx / 2 + 1), ctx->stream);
+            else if (ctx->zmapsx_ok[anc ? 1 : 0])
                 e = launch_zfft_residual_tma(ctx->Fh, (float)(1.0 / V), ctx->zplan, ctx->ztw, ctx->zmapsx[anc ? 1 : 0],
                                              &ctx->st_d->err, ctx->stream);
             else
@@ -734,8 +743,10 @@ cudaError_t issue_iteration(spg_ctx *ctx, const StepParams &p)
                                          (float)(1.0 / V), ctx->zplan, ctx->ztw, ctx->stream);
             if (e != cudaSuccess) return e;
             if (cf.exec_c2c(ctx->pyc, Fc, Fc, CUFFT_INVERSE) != CUFFT_SUCCESS) return cudaErrorUnknown;
-            e = launch_xpass_c2r(d.nx, ctx->Fh, d.ny, d.nz, static_cast<float *>(ctx->B), d.pitch, ctx->xtw,
-                                 ctx->stream);
+            e = ctx->xmix ? launch_mix_c2r(ctx->mx, ctx->xtw, ctx->Fh, d.ny, d.nz, static_cast<float *>(ctx->B), d.pitch,
+                                           ctx->stream)
+                          : launch_xpass_c2r(d.nx, ctx->Fh, d.ny, d.nz, static_cast<float *>(ctx->B), d.pitch, ctx->xtw,
+                                             ctx->stream);
             if (e != cudaSuccess) return e;
             ctx->launches += 3;
         } else {
@@ -1367,27 +1378,36 @@ spg_status spg_set_data_fourier(spg_ctx *ctx, int vol, const void *y_half, const
         ctx->plans = true;
         ctx->zmaps_ok[0] = ctx->zown && zfft_tma_ok(ctx->zplan) &&
                            encode_zmaps(ctx->zplan, ctx->Fh, ctx->Nh, ctx->Ch, &ctx->zmaps[0]);
-        // power-of-two nx 128 .. 1024: the own row pass and the library's
-        // transform along y over contiguous lines (SPG_ROW_PASS=0 in the
-        // environment keeps the library's per-plane 2-D transforms)
+        // an own row pass and the library's transform along y over contiguous
+        // lines (SPG_ROW_PASS=0 in the environment keeps the library's
+        // transforms): power-of-two nx 128 .. 1024 with power-of-two nz, else
+        // lengths of spg_mixed.cu
         const char *rp = std::getenv("SPG_ROW_PASS");
         const long long ylines = (long long)d.nz * nxh;
-        if (ctx->zown && xpass_supported(d.nx, d.nz) && !(rp && std::strcmp(rp, "0") == 0) &&
-            ylines * d.ny <= INT_MAX) {
+        std::vector<float2> xt, zt;
+        const bool pow2 = ctx->zown && xpass_supported(d.nx, d.nz);
+        ctx->xmix = !pow2 && ylines * d.ny >= kMixMinHalf && mix_plan(d.nx, &ctx->mx, &xt) &&
+                    (ctx->zown || mix_plan(d.nz, &ctx->mz, &zt));
+        if ((pow2 || ctx->xmix) && !(rp && std::strcmp(rp, "0") == 0) && ylines * d.ny <= INT_MAX) {
             int ny1[1] = {d.ny};
             if (cf.plan_many(&ctx->pyc, 1, ny1, ny1, 1, d.ny, ny1, 1, d.ny, CUFFT_C2C, (int)ylines) == CUFFT_SUCCESS) {
                 ctx->xown = true;  // the plan exists from here on (destroyed with the context)
                 cf.set_stream(ctx->pyc, ctx->stream);
-                std::vector<float2> xt;
-                xpass_twiddles(d.nx, &xt);
+                if (pow2) xpass_twiddles(d.nx, &xt);
                 CK(dalloc(&ctx->xtw, xt.size() * sizeof(float2)), "alloc");
                 CK(cudaMemcpyAsync(ctx->xtw, xt.data(), xt.size() * sizeof(float2), cudaMemcpyHostToDevice,
                                    ctx->stream),
                    "twiddles");
+                if (!ctx->zown) {
+                    CK(dalloc(&ctx->mztw, zt.size() * sizeof(float2)), "alloc");
+                    CK(cudaMemcpyAsync(ctx->mztw, zt.data(), zt.size() * sizeof(float2), cudaMemcpyHostToDevice,
+                                       ctx->stream),
+                       "twiddles");
+                }
                 CK(dalloc(&ctx->Nx, (size_t)ctx->nhalf * sizeof(float)), "alloc");
                 CK(dalloc(&ctx->Cx, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
                 CK(cudaStreamSynchronize(ctx->stream), "synchronise");
-                ctx->zmapsx_ok[0] = zfft_tma_ok(ctx->zplan) &&
+                ctx->zmapsx_ok[0] = ctx->zown && zfft_tma_ok(ctx->zplan) &&
                                     encode_zmaps(ctx->zplan, ctx->Fh, ctx->Nx, ctx->Cx, &ctx->zmapsx[0]);
             }
         }

@@ -258,6 +258,27 @@ cudaError_t launch_xpass_c2r(int nx, const float2 *F, int ny, int nz, float *Y, 
                              cudaStream_t s);
 cudaError_t launch_kx_major(const float *in, float *out, int ny, int nxh, int nz, cudaStream_t s);
 cudaError_t launch_kx_major(const float2 *in, float2 *out, int ny, int nxh, int nz, cudaStream_t s);
+// Mixed-radix passes (spg_mixed.cu) for axes of kMixMinN .. kMixMaxN with prime
+// factors of at most 13, the spectrum held kx-major as by the row pass above.
+constexpr int kMixMinN = 16, kMixMaxN = 512, kMixStages = 6, kMixMaxThreads = 256;
+constexpr long long kMixMinHalf = 1 << 20;  // coefficients from which these passes are taken (reasons in spg_mixed.cu)
+struct MixAxis {
+    int n, nst, row_threads, col_threads;
+    int radix[kMixStages];                       // of each stage, in order
+    unsigned inv[kMixStages], rinv[kMixStages];  // ceil(2^20 / span) of the stages, forward and in reversed order
+};
+// Stages of length n; appends its table e^(-2 pi i m / n), m < n. False: not such a length.
+bool mix_plan(int n, MixAxis *ax, std::vector<float2> *table);
+// As launch_zfft_residual, F viewed as [n][inner].
+cudaError_t launch_mix_residual(float2 *F, const float *N, const float2 *C, float scale, const MixAxis &ax,
+                                const float2 *tw, long long inner, cudaStream_t s);
+// As launch_xpass_r2c_extrap and launch_xpass_c2r.
+cudaError_t launch_mix_r2c(const MixAxis &ax, const float2 *tw, const DevState *st, const VolDesc *vols,
+                           const float *beta, float *const *xbuf, int pitch, int ny, int nz, float2 *F,
+                           cudaStream_t s);
+cudaError_t launch_mix_c2r(const MixAxis &ax, const float2 *tw, float2 *F, int ny, int nz, float *out, int pitch,
+                           cudaStream_t s);
+
 // F <- A_z^-1 ((A_z F) N scale - Cd), A_z^-1 the unnormalised inverse.
 cudaError_t launch_zfft_residual(float2 *F, const float *N, const float2 *Cd, float scale, const ZPlan &p,
                                  const float2 *tw, cudaStream_t s);
