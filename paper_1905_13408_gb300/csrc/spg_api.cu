@@ -2149,7 +2149,7 @@ spg_status spg_backward(spg_ctx *ctx, int K, const float *gx, float *gb, float *
             a.plane_part = pp + (size_t)k * nblk * 4;
             a.nblocks = nblk;
             a.prev_fresh = k >= 1 ? 1 : 0;  // dL/dx_{k-1} gets its first contribution here
-            CK(launch_adjoint_mask(a, ctx->stream), "adjoint mask");
+            CK(launch_adjoint_mask(a, k < k1 - 1, ctx->stream), "adjoint mask");  // a recomputation ends before the first
             CK(launch_adjoint_apply(a, ctx->stream), "adjoint apply");
             ctx->launches += 2;
             // rotate: dL/dx_k is complete; the old dL/dx_{k+1} buffer becomes dL/dx_{k-2},

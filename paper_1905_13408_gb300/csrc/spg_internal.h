@@ -54,8 +54,9 @@ struct TmapSet {
     CUtensorMap om1;    // l1 weights,      box TX x TY x 1
 };
 
-// Device-resident solver state; the last CTA of each fused step advances it,
-// so the same launch (or captured graph node) serves every iteration.
+// Device-resident solver state; the last CTA of each launch of the fused step
+// advances it, so the same arguments (or captured graph node) serve every
+// launch.
 struct DevState {
     int cur;                 // buffer holding x_k
     int k_round;             // iterations done in the current round
@@ -168,7 +169,7 @@ struct AdjParams {
 // mask m, the scalar partials, gb, gw), then the update of the cotangents
 // (H_mu D m and ybar). Each is one kernel of adjoint_blocks(...) CTAs.
 int adjoint_blocks(int nx, int ny, int nz);
-cudaError_t launch_adjoint_mask(const AdjParams &a, cudaStream_t s);
+cudaError_t launch_adjoint_mask(const AdjParams &a, bool early, cudaStream_t s);
 // out[k] = {sum of [0], sum of [1]} of the nblk partials of step k, k < K.
 cudaError_t launch_adjoint_scalars(const double *part, int nblk, int K, double *out, cudaStream_t s);
 cudaError_t launch_adjoint_apply(const AdjParams &a, cudaStream_t s);
