@@ -182,7 +182,7 @@ spg_status spg_set_data(spg_ctx *ctx, int vol, const void *b, const void *w, spg
  * extrapolated point y_k, forms the residual spectrum N A y_k - D y and
  * transforms back to get the data gradient A^H (N A y_k - D y) for the fused
  * step. With power-of-two nx from 128 to 1024 and nz from 8 to 4096, and from
- * 2^20 coefficients on with nx and nz of 16 to 512 whose prime factors are at
+ * 2^21 coefficients on with nx and nz of 16 to 512 whose prime factors are at
  * most 13: own passes along the rows (which form y_k) and along z (which form
  * the residual), the spectrum held kx-major in between, and cuFFT along y over
  * contiguous lines. Otherwise (and where SPG_ROW_PASS=0 is in the environment

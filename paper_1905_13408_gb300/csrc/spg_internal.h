@@ -262,7 +262,7 @@ cudaError_t launch_kx_major(const float2 *in, float2 *out, int ny, int nxh, int 
 // Mixed-radix passes (spg_mixed.cu) for axes of kMixMinN .. kMixMaxN with prime
 // factors of at most 13, the spectrum held kx-major as by the row pass above.
 constexpr int kMixMinN = 16, kMixMaxN = 512, kMixStages = 6, kMixMaxThreads = 256;
-constexpr long long kMixMinHalf = 1 << 20;  // coefficients from which these passes are taken (reasons in spg_mixed.cu)
+constexpr long long kMixMinHalf = 1 << 21;  // coefficients from which these passes are taken (reasons in spg_mixed.cu)
 struct MixAxis {
     int n, nst, row_threads, col_threads;
     int radix[kMixStages];                       // of each stage, in order

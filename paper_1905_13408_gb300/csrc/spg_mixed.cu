@@ -14,11 +14,13 @@
 // taken, 42 % of an SM's warps resident), at about 29 instructions per element
 // and radix stage: rows 24 and 22 us, z pass 30 (cold caches, under a profiler).
 // An iteration, library -> here: 180^3 170 -> 144 us, 220 x 208 x 176 194 -> 182,
-// 300 x 200 x 240 350 -> 308, 400^3 2074 -> 1420, 256 x 256 x 64 90.3 -> 85.7,
-// 128 x 256 x 64 56.2 -> 51.2; below about 2^19 coefficients, where a launch's
-// fixed cost counts, the library's passes win (100^3 41.2 -> 42.4, 64^3 24.7 ->
-// 27.9), and setting the data takes two transposes more (20 us at 180^3), so
-// the line lies at 2^20 (kMixMinHalf).
+// 224^3 316 -> 260, 300 x 200 x 240 350 -> 308, 384^3 1328 -> 1061, 400^3 2074 ->
+// 1420, 448^3 2556 -> 1974, 256 x 256 x 64 90.3 -> 85.7, 112 x 512 x 90 130 -> 122.
+// Smaller boxes, where a launch's fixed cost counts, are mixed (128 x 256 x 64
+// 56.2 -> 51.2, 140 x 130 x 120 65.9 -> 61.9, 160^3 109.9 -> 108.4, 128 x 176 x 100
+// 55.2 -> 56.9) or lose (100^3 41.2 -> 42.4, 64^3 24.7 -> 27.9), and setting the
+// data takes two transposes more (20 us), so the line lies at 2^21 coefficients
+// (kMixMinHalf), above the last of these.
 //
 // Tried and slower at 180^3: own passes along y too, on the standard half
 // layout (148 us: 18 us a pass), two lines per thread (160: fewer
@@ -539,8 +541,7 @@ bool mix_plan(int n, MixAxis *ax, std::vector<float2> *table)
     // largest (a stage of radix 2 has its exchange but little else to do).
     q.row_threads = pick_threads(q, kRowLines, row_smem(n));
     q.col_threads = pick_threads(q, kColLines, col_smem(n));
-    static const cudaError_t limits = set_limits();
-    if (limits != cudaSuccess) return false;
+    if (set_limits() != cudaSuccess) return false;  // of the current device
     const double pi = 3.14159265358979323846;
     for (int j = 0; j < n; j++) {
         const double w = -2.0 * pi * (double)j / (double)n;
