@@ -716,8 +716,8 @@ def run_batch(args):
 
 def measure_batch(args):
     """24 independent volumes of uneven sizes (6 each of 96^3, 128^3, 192^3,
-    256^3, lambda_tv ~ U(0.05, 0.2)) advanced by one fused launch per
-    iteration (replayed from a CUDA graph, tile shape from the autotuner),
+    256^3, lambda_tv ~ U(0.05, 0.2)) advanced together, many
+    iterations per fused launch (tile shape from the autotuner),
     against 24 single-volume contexts launched one after another."""
     import torch
 
