@@ -4,8 +4,10 @@
 // extrapolated point y_k by per-plane real-to-complex transforms (cuFFT), one
 // pass along z that transforms, scales by N, subtracts the data spectrum and
 // transforms back (spg_zfft.cu, power-of-two nz), and per-plane
-// complex-to-real transforms; for other nz by 3-D transforms around a
-// separate spectrum pass (spec_scale_kernel). The fused step consumes it. Subtracting before the inverse transform
+// complex-to-real transforms; with own row passes in place of the per-plane
+// transforms' part along x (spg_xpass.cu, spg_mixed.cu) where the lengths
+// allow; for other nz by 3-D transforms around a separate spectrum pass
+// (spec_scale_kernel). The fused step consumes it. Subtracting before the inverse transform
 // keeps FP32 rounding relative to the residual rather than to A^H N A y_k,
 // which for the strongly uneven N of gridded data (many orders of magnitude
 // between low and high frequencies) is the difference between errors of 1e-7
