@@ -497,8 +497,9 @@ struct Pipe {
 // in this iteration (*sh.next), whose first planes the producer fetches while
 // this item's last ones are computed. The copies of the iteration's first S
 // steps are issued by the caller. Ends with a barrier over the CTA
-// after the item's last stores. Returns true when a barrier wait gave up (the
-// CTA then stops).
+// after the item's last stores to the iterate; the sums go to `part` behind it
+// (with DOT before a further barrier), so a reader in another CTA needs one more.
+// Returns true when a barrier wait gave up (the CTA then stops).
 template <int VX, int TY, int S, bool BF16, bool XD, bool REC, bool DOT, bool FOURIER>
 __device__ __forceinline__ bool run_item(const StepParams &P, const Smem &sh, Pipe &pp_, const WorkItem &W,
                                          bool has_next, double *part, int kmom, const TmapSet *tm, int ia, int ib,
@@ -976,6 +977,12 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
         if (aborted) break;
         if (many) {
             bool ok = true;
+            // The last iteration's sums are read by other CTAs behind the grid
+            // barrier, and the producer's warp does not wait for the row warps
+            // that store them (run_item): a barrier over the CTA before the
+            // producer arrives. The earlier iterations' are ordered by the
+            // barriers of the plane steps that follow them.
+            if (itn + 1 == P.niter) __syncthreads();
             if (producer) {
                 // the next iteration's first copies: what no iteration writes before
                 // the barrier, the iterate behind it (also after a failure, so that
@@ -1025,7 +1032,7 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
     VolDesc *const vols_rw = const_cast<VolDesc *>(P.vols);
     const StateSnap snap = *sh.snap;
     if (many && !aborted) {
-        // after the last grid barrier every CTA sees every partial
+        // every CTA's partials were stored before it arrived at the last grid barrier
         write_history(P, snap, blockIdx.x * (TY + 1) + warp, gridDim.x * (TY + 1), lane);
         const double *const parts = P.partials + (long long)(P.niter - 1) * P.nitems * 4;
         for (int p = p0 + warp; p < p1; p += TY + 1) {
