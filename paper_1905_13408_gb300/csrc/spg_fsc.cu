@@ -57,8 +57,9 @@ __device__ __forceinline__ int freq(int i, int n) { return i <= (n - 1) / 2 ? i 
 // shared memory without atomics. The sums' order is fixed.
 //
 // Range: the pairs need |component| < 1e14 (sums of squares below 1e38) and,
-// for the rounding terms, a largest component above 1e-8 (or 0) in each lane;
-// otherwise `flag` is set and the caller runs the double kernel below.
+// for the rounding terms, a largest component above 1e-8 (or 0) of each map in
+// each lane (the squares of one map do not see the other's scale); otherwise
+// `flag` is set and the caller runs the double kernel below.
 __device__ __forceinline__ FF two_prod_add(FF acc, float a, float b)
 {
     const float p = __fmul_rn(a, b);
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(256) fsc_shell_ff_kernel(const float2 *__restr
                 while ((s + 1) * (s + 1) <= r2) s++;
                 key = r2 > s * s + s ? s + 1 : s;
                 float2 a[8], b[8];
-                float m = 0.f;
+                float ma = 0.f, mb = 0.f;
 #pragma unroll
                 for (int c = 0; c < 8; c++) {
                     const int sw = c >> 2, ik = (c >> 1) & 1, il = c & 1;
@@ -122,12 +123,13 @@ __global__ void __launch_bounds__(256) fsc_shell_ff_kernel(const float2 *__restr
                     const float4 v = make_float4(fabsf(a[c].x), fabsf(a[c].y), fabsf(b[c].x), fabsf(b[c].y));
                     // written so that a NaN fails the test
                     if (!(v.x < 1e14f && v.y < 1e14f && v.z < 1e14f && v.w < 1e14f)) bad = true;
-                    m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                    ma = fmaxf(ma, fmaxf(v.x, v.y));
+                    mb = fmaxf(mb, fmaxf(v.z, v.w));
                     re = two_prod_add(two_prod_add(re, a[c].x, b[c].x), a[c].y, b[c].y);
                     fa = two_prod_add(two_prod_add(fa, a[c].x, a[c].x), a[c].y, a[c].y);
                     gb = two_prod_add(two_prod_add(gb, b[c].x, b[c].x), b[c].y, b[c].y);
                 }
-                if (m > 0.f && m < 1e-8f) bad = true;
+                if ((ma > 0.f && ma < 1e-8f) || (mb > 0.f && mb < 1e-8f)) bad = true;
                 cnt = nk * nl * swaps;
                 if (h > 0 && 2 * h != n) {  // the conjugates (exact doubling)
                     re = {2.f * re.hi, 2.f * re.lo};
