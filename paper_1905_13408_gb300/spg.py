@@ -219,8 +219,8 @@ def spg_param_scales(h, vol=0):
 def _workspace(nbytes, stream):
     """A device buffer of nbytes from torch's caching allocator, taken on the
     stream that will use it (so it cannot be one that work pending on another
-    stream still uses); None without torch or without room (the library then
-    allocates, and reports it, itself)."""
+    stream still uses); None without torch, with a torch that has no CUDA or
+    without room (the library then allocates, and reports it, itself)."""
     try:
         import torch
     except ImportError:  # pragma: no cover
@@ -231,7 +231,7 @@ def _workspace(nbytes, stream):
         on = torch.cuda.ExternalStream(int(stream)) if stream else torch.cuda.default_stream()
         with torch.cuda.stream(on):
             return torch.empty(nbytes, dtype=torch.uint8, device="cuda")
-    except torch.cuda.OutOfMemoryError:
+    except (RuntimeError, AssertionError):  # out of memory and no driver; not compiled with CUDA
         return None
 
 
