@@ -767,10 +767,13 @@ __device__ __forceinline__ bool grid_barrier(DevState *st, unsigned target, long
     }
 }
 
-// Iterations of this launch before iteration i that record the objective.
-__device__ __forceinline__ int recorded_before(int rec0, int every, int i)
+// Iterations of this launch before iteration i that record the objective
+// (rec0 < every; the distances fit an unsigned for every `every` an int holds).
+__host__ __device__ __forceinline__ int recorded_before(int rec0, int every, int i)
 {
-    return every <= 0 ? 0 : (i + rec0 + every - 1) / every - (rec0 + every - 1) / every;
+    if (every <= 0) return 0;
+    const unsigned first = rec0 > 0 ? (unsigned)every - (unsigned)rec0 : 0u;  // the first that records
+    return (unsigned)i <= first ? 0 : (int)(((unsigned)i - first - 1u) / (unsigned)every) + 1;
 }
 
 // Sums of volume V's item partials (one warp, fixed order): every lane gets
@@ -826,7 +829,7 @@ __device__ __forceinline__ void write_history(const StepParams &P, const StateSn
     const int total = recorded_before(S.rec0, P.hist_every, P.niter);
     for (long long e = w; e < (long long)P.niter * P.nvol; e += nw) {
         const int i = (int)(e / P.nvol), v = (int)(e % P.nvol);
-        if (P.hist_every <= 0 || (S.rec0 + i) % P.hist_every != 0) continue;
+        if (P.hist_every <= 0 || ((unsigned)S.rec0 + (unsigned)i) % (unsigned)P.hist_every != 0) continue;
         const int rank = recorded_before(S.rec0, P.hist_every, i);
         if (total - rank > P.hist_cap) continue;
         const VolDesc V = P.vols[v];
@@ -1016,7 +1019,7 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
             }
         }
         cur = nxt;
-        rec_in = rec_in + 1 == P.hist_every ? 0 : rec_in + 1;
+        rec_in = rec_in >= P.hist_every - 1 ? 0 : rec_in + 1;
     }
 
     if (aborted && producer) {
