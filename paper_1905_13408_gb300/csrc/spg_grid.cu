@@ -76,15 +76,39 @@ struct Sample {
 };
 
 // p = r0 kx + r1 ky on one axis: the nearest point (half to even, kernel 0) or
-// floor (kernel 1) b and the remainder f, as exact arithmetic on the float32
-// entries gives them. The products are exact pairs (fused multiply-add), their
+// floor (kernel 1) b and the remainder f.
+struct AxisPos {
+    int b;
+    float f;
+};
+
+// In double, for positions beyond split_axis's range (matrices that are no
+// rotations). b saturates; a Gaussian weight so far from b is zero.
+__device__ __noinline__ AxisPos split_axis_wide(float r0, float r1, int kx, int ky, int kernel)
+{
+    const double p = __dadd_rn(__dmul_rn(r0, kx), __dmul_rn(r1, ky));
+    AxisPos a;
+    if (kernel == 0) {
+        a.b = __double2int_rn(p);
+        a.f = (float)(p - a.b);
+    } else {
+        const double c = floor(p);
+        a.b = __double2int_rn(c);
+        a.f = (float)(p - c);
+    }
+    return a;
+}
+
+// As exact arithmetic on the float32 entries gives them, where |p| < 2^22. The
+// products are exact pairs (fused multiply-add), their
 // leading parts are added exactly and the sum is normalised (the tails can
 // exceed an ulp of the sum where the products cancel), so p = s + lo with |lo|
-// at most half an ulp of s and an error far below any half-way case of
+// at most half an ulp of s (an eighth) and an error far below any half-way case of
 // float32 rotations; doubles gave the same decisions at 9 FP64 operations a coefficient and
 // half a dozen conversions, more than a millisecond of GB300's FP64 pipe for
-// 2048 images of 256^2.
-__device__ __forceinline__ void split_axis(float r0, float r1, int kx, int ky, int kernel, int &b, float &f)
+// 2048 images of 256^2. False beyond 2^22, where lo grows past the point s decides
+// on: the caller then takes them (no rotation of n <= 1290 comes near).
+__device__ __forceinline__ bool split_axis(float r0, float r1, int kx, int ky, int kernel, int &b, float &f)
 {
     const float x = (float)kx, y = (float)ky;
     const float p = __fmul_rn(r0, x), q = __fmul_rn(r1, y);
@@ -106,6 +130,7 @@ __device__ __forceinline__ void split_axis(float r0, float r1, int kx, int ky, i
         b = (int)c;
         f = __fadd_rn(__fsub_rn(s, c), lo);
     }
+    return fabsf(s) < 4194304.f;  // false for NaN too
 }
 
 __device__ __forceinline__ void make_sample(int n, const float *__restrict__ R, const float2 *__restrict__ X,
@@ -120,9 +145,20 @@ __device__ __forceinline__ void make_sample(int n, const float *__restrict__ R, 
     S.vim = pc * x.y;
     S.vcc = pc * c;
     // row-major 3x3; columns 0 and 1 span the image plane
-    split_axis(R[0], R[1], kx, ky, kernel, S.bx, S.fx);
-    split_axis(R[3], R[4], kx, ky, kernel, S.by, S.fy);
-    split_axis(R[6], R[7], kx, ky, kernel, S.bz, S.fz);
+    const bool nx = split_axis(R[0], R[1], kx, ky, kernel, S.bx, S.fx);
+    const bool ny = split_axis(R[3], R[4], kx, ky, kernel, S.by, S.fy);
+    const bool nz = split_axis(R[6], R[7], kx, ky, kernel, S.bz, S.fz);
+    if (!(nx && ny && nz)) {
+        const AxisPos ax = split_axis_wide(R[0], R[1], kx, ky, kernel);
+        const AxisPos ay = split_axis_wide(R[3], R[4], kx, ky, kernel);
+        const AxisPos az = split_axis_wide(R[6], R[7], kx, ky, kernel);
+        S.bx = ax.b;
+        S.by = ay.b;
+        S.bz = az.b;
+        S.fx = ax.f;
+        S.fy = ay.f;
+        S.fz = az.f;
+    }
     if (kernel == 0) {
         S.bx -= 1;
         S.by -= 1;
