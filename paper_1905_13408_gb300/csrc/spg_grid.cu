@@ -331,11 +331,12 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
             if (DXY * EZ > kBoxCap) DXY = DX * EY;
             const int vol = DXY * EZ;
             {
-                // a lane without a sample in this pass stages a deposit of nothing
+                // a lane without a sample in this pass stages a deposit of nothing (at a
+                // position off every point: on one, 1/h = infinity would weigh it NaN)
                 float wx[3], wy[3], wz[3];
-                axis_weights(kernel, ih, mine ? S.fx : 0.f, wx);
-                axis_weights(kernel, ih, mine ? S.fy : 0.f, wy);
-                axis_weights(kernel, ih, mine ? S.fz : 0.f, wz);
+                axis_weights(kernel, ih, mine ? S.fx : 0.25f, wx);
+                axis_weights(kernel, ih, mine ? S.fy : 0.25f, wy);
+                axis_weights(kernel, ih, mine ? S.fz : 0.25f, wz);
                 const int off = mine ? (S.bz - lz) * DXY + (S.by - ly) * DX + (S.bx - lx) : 0;
 #pragma unroll
                 for (int d = 0; d < 3; d++) {
