@@ -200,6 +200,30 @@ cudaError_t dalloc(T **p, size_t bytes)
     return cudaMalloc(reinterpret_cast<void **>(p), bytes ? bytes : 16);
 }
 
+// As dalloc, unless *p is there already (from a call that could not allocate all it needs).
+template <class T>
+cudaError_t dalloc_once(T **p, size_t bytes)
+{
+    return *p ? cudaSuccess : dalloc(p, bytes);
+}
+
+// Gives up the Fourier term's own row pass: the iterations then use the
+// library's transforms, which need none of these arrays.
+void drop_row_pass(spg_ctx *c)
+{
+    if (c->xown) spg::cufft_api().destroy(c->pyc);
+    void *fs[] = {c->xtw, c->mztw, c->Nx, c->Cx, c->Nstx, c->Cstx};
+    for (void *p : fs)
+        if (p) cudaFree(p);
+    c->xtw = c->mztw = c->Cx = c->Cstx = nullptr;
+    c->Nx = c->Nstx = nullptr;
+    c->xown = c->xmix = false;
+    c->zmapsx_ok[0] = c->zmapsx_ok[1] = false;
+    c->y_fresh = false;
+    if (c->gexec) cudaGraphExecDestroy(c->gexec);
+    c->gexec = nullptr;
+}
+
 void free_all(spg_ctx *c)
 {
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
@@ -1330,14 +1354,14 @@ spg_status spg_set_data_fourier(spg_ctx *ctx, int vol, const void *y_half, const
     const VolDesc &d = ctx->vols_h[0];
     const int nxh = d.nx / 2 + 1;
     ctx->nhalf = (long long)d.nz * d.ny * nxh;
-    if (!ctx->Ybuf) {
-        CK(dalloc(&ctx->Ybuf, (size_t)ctx->total * sizeof(float)), "alloc");
-        CK(dalloc(&ctx->Fh, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
-        CK(dalloc(&ctx->Yh, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
-        CK(dalloc(&ctx->Nh, (size_t)ctx->nhalf * sizeof(float)), "alloc");
-        CK(dalloc(&ctx->Ch, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
-        CK(dalloc(&ctx->Nmax, sizeof(float)), "alloc");
-        CK(dalloc(&ctx->fpart, 1025 * sizeof(double)), "alloc");
+    if (!ctx->plans) {
+        CK(dalloc_once(&ctx->Ybuf, (size_t)ctx->total * sizeof(float)), "alloc");
+        CK(dalloc_once(&ctx->Fh, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
+        CK(dalloc_once(&ctx->Yh, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
+        CK(dalloc_once(&ctx->Nh, (size_t)ctx->nhalf * sizeof(float)), "alloc");
+        CK(dalloc_once(&ctx->Ch, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
+        CK(dalloc_once(&ctx->Nmax, sizeof(float)), "alloc");
+        CK(dalloc_once(&ctx->fpart, 1025 * sizeof(double)), "alloc");
         CK(cudaMemsetAsync(ctx->Ybuf, 0, (size_t)ctx->total * sizeof(float), ctx->stream), "memset");
     }
     if (!ctx->plans) {
@@ -1347,7 +1371,7 @@ spg_status spg_set_data_fourier(spg_ctx *ctx, int vol, const void *y_half, const
         std::vector<float2> tw;
         ctx->zown = zfft_plan(d.nz, (long long)d.ny * nxh, &ctx->zplan, &tw);
         if (ctx->zown) {
-            CK(dalloc(&ctx->ztw, tw.size() * sizeof(float2)), "alloc");
+            CK(dalloc_once(&ctx->ztw, tw.size() * sizeof(float2)), "alloc");
             CK(cudaMemcpyAsync(ctx->ztw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice,
                                ctx->stream),
                "twiddles");
@@ -1394,21 +1418,25 @@ spg_status spg_set_data_fourier(spg_ctx *ctx, int vol, const void *y_half, const
                 ctx->xown = true;  // the plan exists from here on (destroyed with the context)
                 cf.set_stream(ctx->pyc, ctx->stream);
                 if (pow2) xpass_twiddles(d.nx, &xt);
-                CK(dalloc(&ctx->xtw, xt.size() * sizeof(float2)), "alloc");
-                CK(cudaMemcpyAsync(ctx->xtw, xt.data(), xt.size() * sizeof(float2), cudaMemcpyHostToDevice,
-                                   ctx->stream),
-                   "twiddles");
-                if (!ctx->zown) {
-                    CK(dalloc(&ctx->mztw, zt.size() * sizeof(float2)), "alloc");
-                    CK(cudaMemcpyAsync(ctx->mztw, zt.data(), zt.size() * sizeof(float2), cudaMemcpyHostToDevice,
-                                       ctx->stream),
-                       "twiddles");
+                cudaError_t e = dalloc(&ctx->xtw, xt.size() * sizeof(float2));
+                if (e == cudaSuccess && !ctx->zown) e = dalloc(&ctx->mztw, zt.size() * sizeof(float2));
+                if (e == cudaSuccess) e = dalloc(&ctx->Nx, (size_t)ctx->nhalf * sizeof(float));
+                if (e == cudaSuccess) e = dalloc(&ctx->Cx, (size_t)ctx->nhalf * sizeof(float2));
+                if (e == cudaSuccess)
+                    e = cudaMemcpyAsync(ctx->xtw, xt.data(), xt.size() * sizeof(float2), cudaMemcpyHostToDevice,
+                                        ctx->stream);
+                if (e == cudaSuccess && !ctx->zown)
+                    e = cudaMemcpyAsync(ctx->mztw, zt.data(), zt.size() * sizeof(float2), cudaMemcpyHostToDevice,
+                                        ctx->stream);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+                if (e == cudaSuccess) {
+                    ctx->zmapsx_ok[0] = ctx->zown && zfft_tma_ok(ctx->zplan) &&
+                                        encode_zmaps(ctx->zplan, ctx->Fh, ctx->Nx, ctx->Cx, &ctx->zmapsx[0]);
+                } else {
+                    drop_row_pass(ctx);  // no room: the library's transforms, which are set up
+                    if (e != cudaErrorMemoryAllocation) return cuda_fail(ctx, e, "row pass");
+                    cudaGetLastError();
                 }
-                CK(dalloc(&ctx->Nx, (size_t)ctx->nhalf * sizeof(float)), "alloc");
-                CK(dalloc(&ctx->Cx, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
-                CK(cudaStreamSynchronize(ctx->stream), "synchronise");
-                ctx->zmapsx_ok[0] = ctx->zown && zfft_tma_ok(ctx->zplan) &&
-                                    encode_zmaps(ctx->zplan, ctx->Fh, ctx->Nx, ctx->Cx, &ctx->zmapsx[0]);
             }
         }
     }
@@ -1456,17 +1484,23 @@ spg_status spg_set_anchor(spg_ctx *ctx, int vol, float gamma, const float *x_anc
     const VolDesc &d = ctx->vols_h[vol];
     if (ctx->fourier) {
         // gamma |x - a|^2 enters the spectrum pass (N + 2 gamma, C + 2 gamma A a / V) and L (+ 2 gamma)
-        if (!ctx->Anc) {
-            CK(dalloc(&ctx->Anc, (size_t)ctx->total * sizeof(float)), "alloc");
-            CK(dalloc(&ctx->Nst, (size_t)ctx->nhalf * sizeof(float)), "alloc");
-            CK(dalloc(&ctx->Cst, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
+        if (!ctx->Cst) {
+            CK(dalloc_once(&ctx->Anc, (size_t)ctx->total * sizeof(float)), "alloc");
+            CK(dalloc_once(&ctx->Nst, (size_t)ctx->nhalf * sizeof(float)), "alloc");
+            CK(dalloc_once(&ctx->Cst, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
             CK(cudaMemsetAsync(ctx->Anc, 0, (size_t)ctx->total * sizeof(float), ctx->stream), "memset");
             ctx->zmaps_ok[1] = ctx->zmaps_ok[0] && encode_zmaps(ctx->zplan, ctx->Fh, ctx->Nst, ctx->Cst, &ctx->zmaps[1]);
-            if (ctx->xown) {
-                CK(dalloc(&ctx->Nstx, (size_t)ctx->nhalf * sizeof(float)), "alloc");
-                CK(dalloc(&ctx->Cstx, (size_t)ctx->nhalf * sizeof(float2)), "alloc");
+        }
+        if (ctx->xown && !ctx->Cstx) {
+            cudaError_t e = dalloc_once(&ctx->Nstx, (size_t)ctx->nhalf * sizeof(float));
+            if (e == cudaSuccess) e = dalloc_once(&ctx->Cstx, (size_t)ctx->nhalf * sizeof(float2));
+            if (e == cudaSuccess) {
                 ctx->zmapsx_ok[1] =
                     ctx->zmapsx_ok[0] && encode_zmaps(ctx->zplan, ctx->Fh, ctx->Nstx, ctx->Cstx, &ctx->zmapsx[1]);
+            } else {
+                if (e != cudaErrorMemoryAllocation) return cuda_fail(ctx, e, "alloc");
+                drop_row_pass(ctx);  // no room for the anchored spectra in the row pass's order
+                cudaGetLastError();
             }
         }
         spg_status s = copy_volume_in(ctx, ctx->Anc, 4, d, x_anchor);
