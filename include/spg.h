@@ -290,7 +290,7 @@ spg_status spg_get_x(spg_ctx *ctx, int vol, float *x);
 spg_status spg_reweight(spg_ctx *ctx);
 
 /* Run k iterations. The fused step runs many of them per launch (a cooperative
- * launch with a barrier over the grid between iterations; up to about 10 ms
+ * launch with a barrier over the grid between iterations; up to about 2 ms
  * of work each); the Fourier-domain data term and the plain kernel of the
  * alternative readings launch per iteration, replayed from a captured CUDA
  * graph when k is large. Asynchronous. Errors: SPG_ENOTREADY before the

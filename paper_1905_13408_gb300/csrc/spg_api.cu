@@ -34,10 +34,16 @@ constexpr size_t kStateBytes = (sizeof(DevState) + 63) / 64 * 64;
 constexpr int kGraphLen = 10;                   // iterations per captured graph (Fourier-domain term, plain steps)
 // Bounds on the iterations of one fused launch: the partial sums it keeps
 // (32 bytes per work item and iteration) and roughly how long it may hold the
-// GPU (work queued on other streams starts between launches). At 10 ms the
-// launch boundary, about 5 us, no longer shows.
+// GPU, because the short kernels of other contexts (validation, re-weighting,
+// objective) start only between launches. Milliseconds of set_data, then
+// reweight and objective, then 10 iterations and objective of a 256^3 context
+// beside an iterating one of 512^3: a launch per iteration 1.0, 1.4, 7.6; bound of
+// 10 ms 2.5, 4.3, 12.3; 4 ms 2.6, 4.7, 8.2; 2 ms 1.7, 3.8, 4.6 (together what they took
+// with a launch per iteration); 1 ms 0.7, 1.4, 2.1. The context that iterates, two
+// rounds of 50 iterations at 256^3 and of 15 at 512^3: 10 ms 8.60 and 21.23 ms, 2 ms
+// 8.67 and 21.37, 1 ms 8.75 and 21.52.
 constexpr size_t kPartialBytes = 1u << 20;
-constexpr double kLaunchSeconds = 10e-3;
+constexpr double kLaunchSeconds = 2e-3;
 constexpr uint64_t kStateMagic = 0x5350475354415445ull;  // "SPGSTATE"
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
