@@ -108,6 +108,7 @@ struct spg_ctx {
     StepVariant var{4, 8, 3, false, true};
     int zchunk = 0, grid = 0, ctas_per_sm = 0, nitems = 0;
     int iters_per_launch = 1;  // most iterations one launch of the plan runs
+    int part_iters = 1;        // iterations whose partial sums partials_d holds
 
     long long k_total = 0;  // host mirror of the device counters
     int k_round = 0;
@@ -598,7 +599,7 @@ spg_status build_plan(spg_ctx *ctx, const StepVariant &v, int zchunk_opt)
     ctx->nitems = (int)items.size();
     ctx->ctas_per_sm = occ;
     ctx->grid = G;
-    ctx->iters_per_launch = per_launch;
+    ctx->iters_per_launch = ctx->part_iters = per_launch;
     if (ctx->gexec) {
         cudaGraphExecDestroy(ctx->gexec);
         ctx->gexec = nullptr;
@@ -630,6 +631,7 @@ StepParams step_params(const spg_ctx *c)
     p.ybuf = (c->fourier && !c->xown) ? c->Ybuf : nullptr;
     p.timeout_ns = kTimeoutNs;
     p.niter = 1;
+    p.iter_cap = c->part_iters;
     p.tm_step = 0;
     p.xouts = nullptr;
     return p;
@@ -1062,6 +1064,7 @@ struct Sweep {
             p.fourier = 0;
             p.ybuf = nullptr;
             p.niter = std::min(n, ctx->iters_per_launch);
+            p.iter_cap = std::min(ctx->part_iters, (int)plan.size() - launched);
             p.tm_step = 1;
             p.xouts = outs + launched;
             e = step_launch(v, ctx->grid, p, ctx->stream);

@@ -41,7 +41,8 @@ struct VolDesc {
 
 // One work item of the fused step: an x-y tile [x0, x0+TX) x [y0, y0+TY) of
 // volume `vol`, marching over the z-planes [z0, z1). pad0: the item's number
-// (its place among the partial sums); pad1, pad2: unused in memory.
+// (its place among the partial sums); pad1: in a CTA's copy, its volume's
+// extrapolation index at the start of the launch; pad2: unused.
 struct WorkItem {
     int vol, x0, y0, z0, z1, pad0, pad1, pad2;
 };
@@ -86,6 +87,7 @@ struct StepParams {
     float *ybuf;             // Fourier-domain term: the step also writes y_{k+1} = x_{k+1} + beta_{k+1} d_{k+1} here
     long long timeout_ns;    // bound on any single barrier wait
     int niter;               // iterations of this launch; above 1 a cooperative launch
+    int iter_cap;            // iterations that partials (and tmaps and xouts, with tm_step) hold from here on
     int tm_step;             // tensor-map sets from one iteration's to the next's (0: the same maps)
     float *const *xouts;     // output volume of each iteration, or null (the buffers rotate)
 };

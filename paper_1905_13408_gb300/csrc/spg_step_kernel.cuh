@@ -810,6 +810,7 @@ __device__ __forceinline__ double volume_dot(const VolDesc &V, const double *par
 __device__ __forceinline__ void history_entry(const StepParams &P, const VolDesc &V, int v, long long entry,
                                               long long k, const double (&a)[4])
 {
+    if (!SPG_GUARD(P.st, entry >= 0 && v >= 0 && v < P.nvol, 11u)) return;
     double *h = P.hist + ((entry % P.hist_cap) * P.nvol + v) * 5;
     const double l1 = (double)V.lambda_l1 * a[1], tv = (double)V.lambda_tv * a[2];
     const double tot = a[0] + l1 + tv;
@@ -875,20 +876,31 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
         for (int i = 0; i < S; i++) mbar_init(&sh.bars[i], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    const int p0 = P.sched[blockIdx.x], p1 = P.sched[blockIdx.x + 1];
+    const int p0 = P.sched[blockIdx.x], p_end = P.sched[blockIdx.x + 1];
+    // the plan against the room it was made for: items, partial sums and planned
+    // steps per iteration, and (restart) extrapolation indices in shared memory
+    const bool plan_ok =
+        SPG_GUARD(P.st, p0 >= 0 && p0 <= p_end && p_end <= P.nitems && P.niter >= 1 && P.niter <= P.iter_cap &&
+                            (!P.restart || P.niter == 1 || p_end - p0 <= kMaxCtaItems), 9u);
+    const int p1 = plan_ok ? p_end : p0;
     // the CTA's items (P.items is in schedule order; pad0: the item's number among
     // its volume's partial sums), with the volume's extrapolation index at the
     // start of the launch (pad1): the barrier between iterations
     // drops L1, and the chain schedule, item, descriptor from L2 would delay the
     // next iteration's first copies
+    auto load_item = [&](int p) {
+        WorkItem W = P.items[p];
+        if (!SPG_GUARD(P.st, W.vol >= 0 && W.vol < P.nvol && W.pad0 >= 0 && W.pad0 < P.nitems, 10u)) W.vol = W.pad0 = 0;
+        return W;
+    };
     auto item_at = [&](int p) {
         if (p - p0 < kItemCache) return sh.items[p - p0];
-        WorkItem W = P.items[p];
+        WorkItem W = load_item(p);
         W.pad1 = P.vols[W.vol].kmom;
         return W;
     };
     if (tid < kItemCache && p0 + tid < p1) {
-        const WorkItem W = P.items[p0 + tid];
+        const WorkItem W = load_item(p0 + tid);
         sh.items[tid] = W;
         // not waited for by the copies below: stored once it arrives
         sh.items[tid].pad1 = P.vols[W.vol].kmom;
@@ -899,7 +911,7 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
     const bool many = P.niter > 1;
 
     Pipe pipe{0, 0, 0, 0};
-    bool aborted = false;
+    bool aborted = !plan_ok;
     // copies of the first S plane steps of an iteration (of its first item, or
     // of the first two where that has only 3 steps)
     auto first_steps = [&](auto f) {
@@ -950,11 +962,6 @@ __global__ void __launch_bounds__(32 * (TY + 1), MINB)
         for (int p = p0; p < p1 && !aborted; p++) {
             const WorkItem W = item_at(p);
             const int it = W.pad0;
-            if (!SPG_GUARD(P.st, p1 <= P.nitems && it >= 0 && it < P.nitems, 1u)) {
-                aborted = true;
-                pipe.drain_from = pipe.gstep;
-                break;
-            }
             const bool has_next = p + 1 < p1;
             if (producer && has_next) *sh.next = item_at(p + 1);
             const int kmom = (P.restart && many && itn > 0) ? sh.kmom[p - p0] : W.pad1 + itn;
