@@ -408,6 +408,14 @@ spg_status spg_unrolled(spg_ctx *ctx, int K, float *xK);
  * context stays usable), SPG_OK if it did not time out. Synchronises. */
 spg_status spg_probe_timeout(spg_ctx *ctx, long long timeout_ns);
 
+/* The same for the fused step's barrier over the grid: one launch of two
+ * iterations, on arrays of their own, whose barrier lacks an arrival for good.
+ * Returns SPG_ETIMEOUT when every CTA gave up after `timeout_ns`, SPG_OK if none
+ * did; the context's iterate and counters are left unchanged. Errors: SPG_EINVAL
+ * for contexts of several volumes, with alternative readings or whose launches
+ * hold one iteration. Synchronises. */
+spg_status spg_probe_barrier(spg_ctx *ctx, long long timeout_ns);
+
 /* Autotuner: times every compiled tile shape of the fused step, each with a
  * few z-splits of the work, for `trial_iters` iterations on this context's
  * own data, keeps the fastest plan and restores the iterate, counters and

@@ -982,6 +982,7 @@ struct Sweep {
     std::vector<Entry> plan;
     std::vector<int> kvals;  // extrapolation indices copied to the device (kept alive)
     int launched = 0, kmom_dev = 0;
+    long long timeout_ns = kTimeoutNs;  // of the steps' waits
 
     explicit Sweep(spg_ctx *c) : ctx(c), v(c->var) { v.xd = false; }
     void add(float *xk, float *xkm1, float *xout, int k) { plan.push_back({xk, xkm1, xout, k}); }
@@ -1063,6 +1064,7 @@ struct Sweep {
             p.restart = 0;
             p.fourier = 0;
             p.ybuf = nullptr;
+            p.timeout_ns = timeout_ns;
             p.niter = std::min(n, ctx->iters_per_launch);
             p.iter_cap = std::min(ctx->part_iters, (int)plan.size() - launched);
             p.tm_step = 1;
@@ -2227,6 +2229,39 @@ spg_status spg_probe_timeout(spg_ctx *ctx, long long timeout_ns)
     CK(launch_timeout_probe(ctx->st_d, timeout_ns, ctx->stream), "timeout probe");
     ctx->launches += 1;
     return device_status(ctx);
+}
+
+spg_status spg_probe_barrier(spg_ctx *ctx, long long timeout_ns)
+{
+    SPG_TRACE();
+    if (!ctx || timeout_ns <= 0 || timeout_ns > kTimeoutNs) return fail(ctx, SPG_EINVAL, "spg_probe_barrier: bad arguments");
+    if (ctx->nvol != 1 || ctx->kread || ctx->max_iters < 2 || ctx->iters_per_launch < 2)
+        return fail(ctx, SPG_EINVAL, "spg_probe_barrier: one volume, the adopted readings, launches of several iterations");
+    const size_t vb = (size_t)ctx->total * 4;
+    Carve cv;
+    {
+        Carve size;
+        for (int q = 0; q < 3; q++) size.take<float>(vb);
+        DevState *s0;
+        VolDesc *v0;
+        TmapSet *t0;
+        float **o0;
+        Sweep::carve(size, 2, &s0, &v0, &t0, &o0);
+        CK(workspace(ctx, size.off, &cv.base), "alloc workspace");
+    }
+    float *buf[3];
+    for (int q = 0; q < 3; q++) {
+        buf[q] = cv.take<float>(vb);
+        CK(cudaMemsetAsync(buf[q], 0, vb, ctx->stream), "memset");
+    }
+    Sweep sw(ctx);
+    sw.timeout_ns = timeout_ns;
+    for (int k = 0; k < 2; k++) sw.add(buf[k], buf[(k + 2) % 3], buf[k + 1], k);
+    CK(sw.upload(cv), "plan the steps");
+    // one arrival short: the first wraps the count to 0
+    CK(cudaMemsetAsync(&sw.st->bar, 0xff, sizeof(unsigned), ctx->stream), "preset the barrier");
+    CK(sw.launch(2), "fused step");
+    return sw.status();
 }
 
 namespace {

@@ -36,7 +36,7 @@ _STATUS_NAMES = {0: "SPG_OK", -1: "SPG_EINVAL", -2: "SPG_ENOMEM", -3: "SPG_ECUDA
 # Every entry point declared in include/spg.h.
 EXPORTS = ["spg_create", "spg_create_batch", "spg_set_data", "spg_set_x", "spg_get_x", "spg_reweight",
            "spg_iterate", "spg_objective", "spg_history", "spg_round_stats", "spg_certificate", "spg_counters",
-           "spg_get_state", "spg_set_state", "spg_backward", "spg_unrolled", "spg_probe_timeout",
+           "spg_get_state", "spg_set_state", "spg_backward", "spg_unrolled", "spg_probe_timeout", "spg_probe_barrier",
            "spg_autotune", "spg_launch_count", "spg_plan_info", "spg_last_error", "spg_destroy",
            "spg_objective_noalloc", "spg_noalloc_last_error", "spg_set_anchor", "spg_param_scales",
            "spg_fsc", "spg_fsc_ws", "spg_fsc_workspace", "spg_fsc_last_error", "spg_set_data_fourier", "spg_backproject",
@@ -115,6 +115,7 @@ def load():
             "spg_backward": (I, [P, I, V, V, V, ctypes.POINTER(D), I]),
             "spg_unrolled": (I, [P, I, V]),
             "spg_probe_timeout": (I, [P, LL]),
+            "spg_probe_barrier": (I, [P, LL]),
             "spg_autotune": (I, [P, I, ctypes.POINTER(I)]),
             "spg_launch_count": (LL, [P]),
             "spg_plan_info": (I, [P, ctypes.POINTER(I)]),
@@ -524,6 +525,10 @@ def spg_unrolled(h, K, out):
 
 def spg_probe_timeout(h, timeout_ns):
     return load().spg_probe_timeout(h, int(timeout_ns))
+
+
+def spg_probe_barrier(h, timeout_ns):
+    return load().spg_probe_barrier(h, int(timeout_ns))
 
 
 def spg_autotune(h, trial_iters=10):
