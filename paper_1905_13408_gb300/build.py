@@ -52,6 +52,7 @@ def _stale(lib=LIB):
     deps = [os.path.join(CSRC, s) for s in SOURCES]
     deps += [os.path.join(CSRC, "spg_internal.h"), os.path.join(CSRC, "spg_step_kernel.cuh"),
              os.path.join(CSRC, "spg_cufft.h"), os.path.join(CSRC, "spg_trace.h"), os.path.join(CSRC, "spg_fft.cuh"), os.path.join(CSRC, "spg_ff.cuh"),
+             os.path.join(CSRC, "spg_range.h"),
              os.path.join(INCLUDE, "spg.h"), __file__]
     return any(os.path.getmtime(d) > t for d in deps)
 

@@ -22,6 +22,7 @@
 #include "spg_trace.h"
 #include "spg_cufft.h"
 #include "spg_internal.h"
+#include "spg_range.h"
 
 using namespace spg;
 
@@ -1270,17 +1271,13 @@ spg_status spg_create(const spg_volume_params *params, const spg_options *opt, v
     return spg_create_batch(1, params, opt, stream, out);
 }
 
-// An array a kernel of this context can read where it lies: memory of the
-// current device, aligned to its elements.
-static bool readable_here(const void *p, size_t es)
+// Whether a kernel of this context can read an array where it lies: memory of
+// the current device whose allocation holds all of it, aligned to its elements.
+// Extent::too_short: device memory that ends before the array does.
+static Extent readable_here(const void *p, size_t es, size_t bytes)
 {
-    cudaPointerAttributes at;
-    int dev = -1;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice && at.device == dev && reinterpret_cast<uintptr_t>(p) % es == 0;
+    const Extent e = device_extent(p, bytes);
+    return e == Extent::holds && reinterpret_cast<uintptr_t>(p) % es != 0 ? Extent::unknown : e;
 }
 
 // The verdict of the validation queued before (synchronises).
@@ -1302,6 +1299,11 @@ spg_status spg_set_data(spg_ctx *ctx, int vol, const void *b, const void *w, spg
     if (!ctx) return fail(nullptr, SPG_EINVAL, "null context");
     if (vol < 0 || vol >= ctx->nvol || !b || !w) return fail(ctx, SPG_EINVAL, "spg_set_data: bad arguments");
     if (src != SPG_F32 && src != SPG_BF16) return fail(ctx, SPG_EINVAL, "spg_set_data: bad dtype");
+    const VolDesc &d = ctx->vols_h[vol];
+    const size_t es = src == SPG_BF16 ? 2 : 4, bytes = (size_t)d.nx * d.ny * d.nz * es;
+    const Extent eb = readable_here(b, es, bytes), ew = readable_here(w, es, bytes);
+    if (eb == Extent::too_short || ew == Extent::too_short)
+        return fail(ctx, SPG_EINVAL, "spg_set_data: a device array is shorter than the volume");
     if (ctx->fourier) {
         ctx->fourier = false;  // back to the real-space data term
         if (ctx->gexec) {
@@ -1309,12 +1311,11 @@ spg_status spg_set_data(spg_ctx *ctx, int vol, const void *b, const void *w, spg
             ctx->gexec = nullptr;
         }
     }
-    const VolDesc &d = ctx->vols_h[vol];
     const long long n = (long long)d.pitch * d.ny * d.nz;
     const bool store_bf16 = ctx->bf16();
     spg_status s;
     const bool same = (src == SPG_BF16) == store_bf16;
-    if (!ctx->reversed && readable_here(b, src == SPG_BF16 ? 2 : 4) && readable_here(w, src == SPG_BF16 ? 2 : 4)) {
+    if (!ctx->reversed && eb == Extent::holds && ew == Extent::holds) {
         if (!same) ctx->reweighted = false;
         ctx->launches += 1;
         CK(launch_ingest(aux_params(ctx), vol, d.aux_end - d.aux_begin, d.nx, b, w, src == SPG_BF16, ctx->B, ctx->W,

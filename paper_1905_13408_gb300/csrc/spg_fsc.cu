@@ -18,6 +18,7 @@
 #include "spg_trace.h"
 #include "spg_cufft.h"
 #include "spg_ff.cuh"
+#include "spg_range.h"
 
 namespace {
 
@@ -317,18 +318,6 @@ struct Buf {
     }
 };
 
-bool device_pointer(const void *p)
-{
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    int dev = -1;
-    cudaGetDevice(&dev);
-    return at.type == cudaMemoryTypeDevice && at.device == dev;
-}
-
 // Launch shape of the shell pass: warps per block (each with a table of the
 // shells, 28 bytes a shell) and blocks.
 struct ShellShape {
@@ -430,12 +419,16 @@ spg_status fsc_run(int n, const float *a, const float *b, double *fsc, double *c
         return fsc_fail(SPG_EINVAL, "spg_fsc: too many shells (n <= 2046)");
     const spg::CufftApi &cf = spg::cufft_api();
     if (!cf.ok) return fsc_fail(SPG_ECUDA, "spg_fsc: cuFFT library could not be loaded");
+    const size_t vox = (size_t)n * n * n * sizeof(float);
+    const spg::Extent ea = spg::device_extent(a, vox), eb = spg::device_extent(b, vox);
+    if (ea == spg::Extent::too_short || eb == spg::Extent::too_short)
+        return fsc_fail(SPG_EINVAL, "spg_fsc: a device map is shorter than n^3 values");
     CallPlan plan;
     if (!plan.get(dev, n)) return fsc_fail(SPG_ECUDA, "spg_fsc: cufft plan");
     // a transform reads a map in place when it lies on this device, aligned as
     // an allocation of its own would be; otherwise it is copied first
-    const bool ca = !device_pointer(a) || (reinterpret_cast<uintptr_t>(a) & 255) != 0;
-    const bool cb = !device_pointer(b) || (reinterpret_cast<uintptr_t>(b) & 255) != 0;
+    const bool ca = ea != spg::Extent::holds || (reinterpret_cast<uintptr_t>(a) & 255) != 0;
+    const bool cb = eb != spg::Extent::holds || (reinterpret_cast<uintptr_t>(b) & 255) != 0;
     const Layout L = layout(n, plan.e.work, ca, cb);
     if (need_out) {  // workspace query
         *need_out = L.total;
@@ -448,7 +441,6 @@ spg_status fsc_run(int n, const float *a, const float *b, double *fsc, double *c
         ws = own.p;
     }
     char *const base = static_cast<char *>(ws);
-    const size_t vox = (size_t)n * n * n * sizeof(float);
     if (ca) FSC_CK(cudaMemcpyAsync(base + L.ra, a, vox, cudaMemcpyDefault, s));
     if (cb) FSC_CK(cudaMemcpyAsync(base + L.rb, b, vox, cudaMemcpyDefault, s));
     float2 *const fa = reinterpret_cast<float2 *>(base + L.fa), *const fb = reinterpret_cast<float2 *>(base + L.fb);
