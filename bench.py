@@ -767,7 +767,7 @@ def measure_batch(args):
     roof = roofline_block(args.dtype, args.storage, nvox, ms_batch / 1e3 / args.steps, peaks["hbm_gbs"], kind,
                           profiled_traffic("batch24", args.dtype, args.storage),
                           "spg_step_kernel (24 volumes per launch)")
-    out = {"metric": "Gvoxel-iter/s, 24 uneven volumes in one fused launch per iteration", "value": value,
+    out = {"metric": "Gvoxel-iter/s, 24 uneven volumes advanced by the same fused launches", "value": value,
            "unit": UNIT, "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
            "ms_per_step": ms_batch / args.steps, "higher_is_better": True, "dtype": args.dtype,
            "data": "synthetic", "config": {"workload": "batch24: 6 each of 96^3, 128^3, 192^3, 256^3",
@@ -790,8 +790,8 @@ def adjoint_bytes_per_voxel(K, C):
     two adjoint passes per iteration (mask: x_k, x_{k-1}, omtv, b, w, om1,
     gnext, gb, gw read, m, gb, gw written, 48 B; apply: x_k, x_{k-1}, m,
     omtv, w, gcur, gprev read, gcur, gprev written, 36 B; the neighbours'
-    rows come from cache) and the fused forward steps it runs (a sweep of K
-    and the recomputation of all but the last step of each of the
+    rows come from cache) and fused forward steps (a sweep of K, of which the
+    call leaves out the last segment's, and the recomputation of all but the last step of each of the
     ceil(K / C) segments, 28 B each with previous-iterate storage)."""
     nck = (K + C - 1) // C
     return 84 * K + 28 * (2 * K - nck)
@@ -951,7 +951,7 @@ def run_grid(args):
                       "roofline": {"bound": "hbm", "achieved": hbm_bytes / sec / 1e9, "peak": peaks["hbm_gbs"],
                                    "unit": "GB/s", "frac": hbm_bytes / sec / 1e9 / peaks["hbm_gbs"], "peak_kind": kind,
                                    "algorithmic_bytes_per_launch": hbm_bytes,
-                                   "note": "far from HBM: the scatter is limited by shared-memory atomics "
+                                   "note": "far from HBM: the scatter is limited by shared memory and issue "
                                            "(27 deposits of 3 sums per coefficient)"},
                       "note": "reset + scatter timed; finish (half-spectrum write) excluded"}))
     return 0

@@ -3,7 +3,7 @@
 // the strong-convexity certificate, the passes of the adjoint of one step,
 // and the plain step used under alternative readings of the paper.
 //
-// None of them is on the fused hot path, so they use plain global loads.
+// All use plain global loads.
 // The adopted reading's re-weighting and objective, the validation and the
 // anchor march over z: a CTA takes 8 rows (a warp each) of a 128-voxel chunk over
 // a run of planes (AuxParams::items), each lane 4 voxels by 16-byte loads, the
@@ -13,8 +13,10 @@
 // (one per row segment).
 // Every reduction keeps one partial per CTA, and the last CTA to finish sums
 // the partials of each volume in a fixed order, so the results are
-// deterministic; the adjoint passes keep one scalar partial per CTA, which the
-// host sums in a fixed order. No kernel here waits on another CTA.
+// deterministic; the adjoint passes keep one scalar partial per CTA, summed per
+// step by adjoint_scalars_kernel (the host adds the steps' results). No kernel
+// here waits on another CTA of its grid; the adjoint passes, launched ahead of
+// the end of the pass before them, wait for that grid (griddepcontrol.wait).
 //
 // Sums across a CTA run in float-float (spg_ff.cuh): with double shuffles
 // GB300's narrow FP64 pipe took most of these passes' time on small volumes.

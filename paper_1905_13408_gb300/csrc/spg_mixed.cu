@@ -529,6 +529,8 @@ bool mix_plan(int n, MixAxis *ax, std::vector<float2> *table)
     if (n < kMixMinN || n > kMixMaxN) return false;
     MixAxis q{};
     q.n = n;
+    // fewest stages, and of those splits the one whose smallest radix is the
+    // largest (a stage of radix 2 has its exchange but little else to do)
     for (int depth = 2; depth <= kMixStages && !q.nst; depth++)
         for (int smallest = 13; smallest >= 2 && !q.nst; smallest--)
             if (split(n, depth, 13, smallest, q.radix)) q.nst = depth;
@@ -537,8 +539,6 @@ bool mix_plan(int n, MixAxis *ax, std::vector<float2> *table)
     // 2^20 / Ns is below 1, and j * 1 < 2^20 / Ns
     for (int s = 0, Ns = 1; s < q.nst; Ns *= q.radix[s++]) q.inv[s] = ((1u << 20) + Ns - 1) / Ns;
     for (int s = q.nst - 1, Ns = 1; s >= 0; Ns *= q.radix[s--]) q.rinv[s] = ((1u << 20) + Ns - 1) / Ns;
-    // fewest stages, and of those splits the one whose smallest radix is the
-    // largest (a stage of radix 2 has its exchange but little else to do).
     q.row_threads = pick_threads(q, kRowLines, row_smem(n));
     q.col_threads = pick_threads(q, kColLines, col_smem(n));
     if (set_limits() != cudaSuccess) return false;  // of the current device

@@ -56,7 +56,9 @@
 // -> 7.6 -> 7.0 -> 6.9, 128^3 18.6 -> 14.1 -> 13.5 -> 13.2, 101 x 147 x 183 30.7 ->
 // 20.8 -> 20.0 -> 19.8, 180^3 57.6 -> 43.3 -> 41.3 -> 40.4, 256^3 86.8 -> 81.5 ->
 // 79.7 -> 78.7, 512^3 618.4 -> 617.2 -> 614.1 -> 606.6; 24 volumes of 96^3 .. 256^3
-// (the last three) 777 -> 767 -> 755. (With the producer's position in shared memory instead of
+// (the last three) 777 -> 767 -> 755. These are of launches of up to 10 ms; with
+// the 2 ms that a launch may take (for other contexts' sake, spg_api.cu) the
+// longest iterations take 0.6-0.9 % more. (With the producer's position in shared memory instead of
 // the item's registers the long marches lost: 623.6 at 512^3, 1128 for the
 // batch: its warp is the last to arrive at every plane's barrier.)
 #pragma once

@@ -297,7 +297,8 @@ struct Tma {
     static constexpr int BOXES = P::N / ROWS;
     static constexpr int TILE = P::N * 16;                 // complex values per tile
     static constexpr size_t SMEM = (size_t)TILE * (2 * sizeof(float2) + sizeof(float) + sizeof(float2)) + 4 * 8;
-    // CTAs per SM: as many as shared memory holds, 1024 threads in all
+    // CTAs per SM that the registers are held to (64 a thread): 1, 2 and, for lines
+    // of 128, 4, of which shared memory holds 3 (57.4 KB each and 1 KB reserved)
     static constexpr int CTAS = P::N >= 512 ? 1 : 512 / P::N;
 };
 
