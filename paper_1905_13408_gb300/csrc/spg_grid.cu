@@ -240,7 +240,8 @@ __device__ __forceinline__ double widen(float v)
 // 7.8 -> 5.6), 128 images 1.08 -> 0.73, 2048 of 128^2 3.20 -> 1.95, 4096 of 64^2
 // 1.64 -> 1.10, 512 of 288^2 4.24 -> 2.63; with one wrapping addition per index of
 // the boxes that cross the box's faces, instead of two integer divisions for
-// each of six indices of a point, 7.0 (5.35), 0.72, 1.78, 0.99 and 2.54. What bounds it now, at 256^2: shared
+// each of six indices of a point, 7.0 (5.35), 0.72, 1.78, 0.99 and 2.54; 7.1 for the
+// first with the test of a position's range (make_sample). What bounds it now, at 256^2: shared
 // memory (800 wavefronts a tile, 64 % of its rate) and issue (2900 instructions
 // a tile, 53 %) with the 16 warps an SM's shared memory holds.
 constexpr int kTileX = 8, kTileY = 4;
